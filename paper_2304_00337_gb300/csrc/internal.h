@@ -174,6 +174,11 @@ void build_hierarchy(DevMem& mem, Hierarchy& H, const double* d_eps, int coarses
 void free_hierarchy(DevMem& mem, Hierarchy& H);
 void alloc_kdata(DevMem& mem, const Hierarchy& H, KData& K, int ngroups);
 void set_group_k(DevMem& mem, const Hierarchy& H, KData& K, int g, double k1, double k2, cudaStream_t s);
+// the phase tables alone, for calls that run no coarsest solve (a matrix near singular is
+// still factorised, so that such calls are refused as the solving ones are)
+void set_group_phases(const Hierarchy& H, KData& K, int g, double k1, double k2, cudaStream_t s);
+// every group at once: ks holds K.ngroups Bloch vectors
+void set_all_k(const Hierarchy& H, KData& K, const double* ks, cudaStream_t s);
 // group src's tables (phases, k = 0 flags, coarsest factors, host mirror) copied into slot dst
 void copy_group_k(KData& K, int src, int dst, cudaStream_t s);
 KData kdata_view(const KData& K, int g);  // non-owning single-group view of group g

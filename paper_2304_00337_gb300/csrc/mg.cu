@@ -112,26 +112,107 @@ __global__ void k_patch_factors(const double* __restrict__ winv, int n, int m, d
   }
 }
 
-// Dense coarsest-level matrices, column-major: column `col` = operator applied to unit vector `col`.
+// Dense coarsest-level matrices, column-major: entry (row, col) = operator applied to unit
+// vector `col`, read at `row`.
+__device__ __forceinline__ double2 coarse_edge_entry(const Lvl<double>& L, const Wts<double>& w, double mu,
+                                                     const Ph<double>& p, int row, int col) {
+  const int Nc = L.n * L.m;
+  const UnitERd<double> r{L.n, L.m, col / Nc, col % Nc, p};
+  const int kind = row / Nc, e = row % Nc, i = e % L.n, j = e / L.n;
+  return kind == 0 ? A_x<double>(r, w, i, j) + mu * M_x<double>(r, L, i, j)
+                   : A_y<double>(r, w, i, j) + mu * M_y<double>(r, L, i, j);
+}
+__device__ __forceinline__ double2 coarse_node_entry(const Lvl<double>& L, const Ph<double>& p, double shift, int row,
+                                                     int col) {
+  const int Nc = L.n * L.m;
+  const UnitNRd<double> r{L.n, L.m, col, p};
+  double2 v = P_at<double>(r, L, row % L.n, row / L.n);
+  v.x += shift / Nc;  // k = 0: the constant mode gets eigenvalue `shift` (zero-mean solutions)
+  return v;
+}
+
 __global__ void k_assemble_edge(Lvl<double> L, Wts<double> w, double mu, const double* ph, double2* K) {  // ph: the group's entry
-  const int Nc = L.n * L.m, Dc = 2 * Nc;
+  const int Dc = 2 * L.n * L.m;
   const int row = blockIdx.x * blockDim.x + threadIdx.x, col = blockIdx.y;
   if (row >= Dc || col >= Dc) return;
-  const UnitERd<double> r{L.n, L.m, col / Nc, col % Nc, load_ph<double>(ph, 0)};
-  const int kind = row / Nc, e = row % Nc, i = e % L.n, j = e / L.n;
-  double2 v = kind == 0 ? A_x<double>(r, w, i, j) + mu * M_x<double>(r, L, i, j)
-                        : A_y<double>(r, w, i, j) + mu * M_y<double>(r, L, i, j);
-  K[(long)col * Dc + row] = v;
+  K[(long)col * Dc + row] = coarse_edge_entry(L, w, mu, load_ph<double>(ph, 0), row, col);
 }
 
 __global__ void k_assemble_node(Lvl<double> L, const double* ph, double shift, double2* K) {
   const int Nc = L.n * L.m;
   const int row = blockIdx.x * blockDim.x + threadIdx.x, col = blockIdx.y;
   if (row >= Nc || col >= Nc) return;
-  const UnitNRd<double> r{L.n, L.m, col, load_ph<double>(ph, 0)};
-  double2 v = P_at<double>(r, L, row % L.n, row / L.n);
-  v.x += shift / Nc;  // k = 0: the constant mode gets eigenvalue `shift` (zero-mean solutions)
-  K[(long)col * Nc + row] = v;
+  K[(long)col * Nc + row] = coarse_node_entry(L, load_ph<double>(ph, 0), shift, row, col);
+}
+
+// The phase and k = 0 tables of one group (three copies each), from kernel arguments: one
+// launch where six small host copies took longer than the operators that follow them.
+__global__ void k_set_phases(double* d_ph, int* d_gamma, int ngroups, int g, double ar, double ai, double br, double bi,
+                             int gamma) {
+  const int rep = threadIdx.x;
+  if (rep >= 3) return;
+  double* p = d_ph + 4 * ((long)rep * ngroups + g);
+  p[0] = ar; p[1] = ai; p[2] = br; p[3] = bi;
+  d_gamma[(long)rep * ngroups + g] = gamma;
+}
+
+// Small coarsest systems (n <= kSmallFactor, the usual 4 x 4 mesh has 32 edges and 16 nodes):
+// assembly and Cholesky factorisation of both matrices of blockIdx.y's group in one launch
+// (blockIdx.x: 0 edge, 1 node), the lower triangle in shared memory.  The chain of pivots is
+// what takes the time: a step is one reciprocal square root and two barriers, with no trip to
+// global memory.
+constexpr int kSmallFactor = 64;
+__global__ void __launch_bounds__(256) k_coarse_factors(Lvl<double> L, Wts<double> w, double mu, const double* ph,
+                                                        const int* gamma, double2* e64, float2* e32, double2* n64,
+                                                        float2* n32, int* info) {
+  extern __shared__ double2 Am[];  // entry (i, j), i >= j, at j (n + 1) + i
+  const int g = blockIdx.y, node = blockIdx.x, Nc = L.n * L.m, n = node ? Nc : 2 * Nc, ld = n + 1;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const Ph<double> p = load_ph<double>(ph, g);
+  const double shift = gamma[g] ? P_diag<double>(L) : 0.0;
+  __shared__ double piv[2];  // pivot and its reciprocal
+  for (int t = tid; t < n * n; t += nt) {
+    const int row = t % n, col = t / n;
+    if (row >= col)
+      Am[col * ld + row] = node ? coarse_node_entry(L, p, shift, row, col) : coarse_edge_entry(L, w, mu, p, row, col);
+  }
+  __syncthreads();
+  for (int k = 0; k < n; ++k) {
+    if (tid == 0) {
+      const double d = Am[k * ld + k].x;
+      const bool ok = d > 0.0 && isfinite(d);
+      if (!ok) info[node] = k + 1;
+      const double r = ok ? sqrt(d) : 1.0;
+      piv[0] = r;
+      piv[1] = 1.0 / r;
+    }
+    __syncthreads();
+    const double inv = piv[1];
+    const int rem = n - k - 1;
+    // the pivot column is scaled in place by the threads of its own entries, and every update
+    // below forms the two scaled entries it needs from the unscaled ones
+    for (int t = tid; t < rem * rem; t += nt) {
+      const int jj = k + 1 + t / rem, ii = k + 1 + t % rem;
+      if (ii < jj) continue;
+      const double2 lik = inv * Am[k * ld + ii], ljk = inv * Am[k * ld + jj];
+      double2 v = Am[jj * ld + ii];
+      v.x -= lik.x * ljk.x + lik.y * ljk.y;
+      v.y -= lik.y * ljk.x - lik.x * ljk.y;
+      Am[jj * ld + ii] = v;
+    }
+    __syncthreads();
+    for (int i = k + 1 + tid; i < n; i += nt) Am[k * ld + i] = inv * Am[k * ld + i];
+    if (tid == 0) Am[k * ld + k] = make_double2(piv[0], 0.0);
+  }
+  __syncthreads();
+  double2* F = (node ? n64 : e64) + (long)g * n * n;
+  float2* F32 = (node ? n32 : e32) + (long)g * n * n;
+  for (int t = tid; t < n * n; t += nt) {
+    const int row = t % n, col = t / n;
+    const double2 v = row >= col ? Am[col * ld + row] : make_double2(0.0, 0.0);
+    F[t] = v;
+    F32[t] = make_float2(float(v.x), float(v.y));
+  }
 }
 
 // In-place Cholesky (lower, column-major) of a Hermitian positive definite matrix; one block.
@@ -592,44 +673,125 @@ void alloc_kdata(DevMem& mem, const Hierarchy& H, KData& K, int ngroups) {
   K = k;
 }
 
-void set_group_k(DevMem& mem, const Hierarchy& H, KData& K, int g, double k1, double k2, cudaStream_t s) {
-  if (g < 0 || g >= K.ngroups) fail(PBS_EINVAL, "group out of range");
-  double ph[4] = {std::cos(k1 * H.a), std::sin(k1 * H.a), std::cos(k2 * H.b), std::sin(k2 * H.b)};
+namespace {
+
+// Bloch phases (alpha, beta) of a Bloch vector; exact ones at the lattice points.  Returns
+// whether k = 0.
+bool bloch_phases(const Hierarchy& H, double k1, double k2, double ph[4]) {
+  ph[0] = std::cos(k1 * H.a);
+  ph[1] = std::sin(k1 * H.a);
+  ph[2] = std::cos(k2 * H.b);
+  ph[3] = std::sin(k2 * H.b);
   const bool gamma = std::hypot(ph[0] - 1.0, ph[1]) < 1e-14 && std::hypot(ph[2] - 1.0, ph[3]) < 1e-14;
-  if (gamma) {  // the exact phases at the lattice points
+  if (gamma) {
     ph[0] = 1.0; ph[1] = 0.0; ph[2] = 1.0; ph[3] = 0.0;
   }
+  return gamma;
+}
+
+void check_factors(const KData& K, cudaStream_t s) {
+  int info[2] = {0, 0};
+  PBS_CUDA(cudaMemcpyAsync(info, K.d_info, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
+  PBS_CUDA(cudaStreamSynchronize(s));
+  if (info[0] || info[1]) fail(PBS_ENUMERIC, "coarsest-level Cholesky factorisation failed");
+}
+
+// Coarsest factors of groups g0 .. g0 + ng - 1 from their phase tables.
+void factor_groups(const Hierarchy& H, KData& K, int g0, int ng, cudaStream_t s) {
+  const Level& C = H.lev[H.nlev - 1];
+  const size_t Dc = K.Dc, Nc = K.Nc;
+  PBS_CUDA(cudaMemsetAsync(K.d_info, 0, 2 * sizeof(int), s));
+  if (K.Dc <= kSmallFactor) {
+    const size_t smem = Dc * (Dc + 1) * sizeof(double2);
+    static PerDeviceOnce once;
+    once([] {
+      PBS_CUDA(cudaFuncSetAttribute(k_coarse_factors, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                    kSmallFactor * (kSmallFactor + 1) * (int)sizeof(double2)));
+    });
+    k_coarse_factors<<<dim3(2, ng), 256, smem, s>>>(C.lvl<double>(), C.wts<double>(), H.mu, K.d_ph + 4L * g0,
+                                                    K.d_gamma + g0, K.edge64 + g0 * Dc * Dc, K.edge32 + g0 * Dc * Dc,
+                                                    K.node64 + g0 * Nc * Nc, K.node32 + g0 * Nc * Nc, K.d_info);
+    PBS_LAUNCHED();
+    return;
+  }
+  for (int g = g0; g < g0 + ng; ++g) {
+    double2* e64 = K.edge64 + g * Dc * Dc;
+    double2* n64 = K.node64 + g * Nc * Nc;
+    const double* gph = K.d_ph + 4L * g;
+    k_assemble_edge<<<dim3(((unsigned)Dc + 127) / 128, (unsigned)Dc), 128, 0, s>>>(C.lvl<double>(), C.wts<double>(),
+                                                                                   H.mu, gph, e64);
+    PBS_LAUNCHED();
+    k_cholesky<<<1, 256, 0, s>>>(e64, K.Dc, K.edge32 + g * Dc * Dc, K.d_info);
+    PBS_LAUNCHED();
+    const double shift = K.gamma[g] ? P_diag<double>(C.lvl<double>()) : 0.0;
+    k_assemble_node<<<dim3(((unsigned)Nc + 127) / 128, (unsigned)Nc), 128, 0, s>>>(C.lvl<double>(), gph, shift, n64);
+    PBS_LAUNCHED();
+    k_cholesky<<<1, 256, 0, s>>>(n64, K.Nc, K.node32 + g * Nc * Nc, K.d_info + 1);
+    PBS_LAUNCHED();
+  }
+}
+
+// The tables of one group without its coarsest factors.
+bool put_phases(const Hierarchy& H, KData& K, int g, double k1, double k2, double ph[4], cudaStream_t s) {
+  if (g < 0 || g >= K.ngroups) fail(PBS_EINVAL, "group out of range");
+  const bool gamma = bloch_phases(H, k1, k2, ph);
   K.k1[g] = k1;
   K.k2[g] = k2;
   K.gamma[g] = gamma;
-  const int gi = gamma ? 1 : 0;
-  for (int rep = 0; rep < 3; ++rep) {
-    const long e = (long)rep * K.ngroups + g;
-    PBS_CUDA(cudaMemcpyAsync(K.d_ph + 4 * e, ph, 4 * sizeof(double), cudaMemcpyHostToDevice, s));
-    PBS_CUDA(cudaMemcpyAsync(K.d_gamma + e, &gi, sizeof(int), cudaMemcpyHostToDevice, s));
-  }
+  k_set_phases<<<1, 32, 0, s>>>(K.d_ph, K.d_gamma, K.ngroups, g, ph[0], ph[1], ph[2], ph[3], gamma ? 1 : 0);
+  PBS_LAUNCHED();
+  return gamma;
+}
+
+// Whether both coarsest matrices are so far from singular that their factorisation cannot
+// fail: A_c + mu M_c >= (mu / 3) min(mx, my), against rounding errors of about n 2^-53 times
+// the largest symbol value, and P_c >= |k|^2 a b / N_c (its lowest Bloch mode).
+bool factors_certain(const Hierarchy& H, const double ph[4], bool gamma) {
   const Level& C = H.lev[H.nlev - 1];
-  const int Dc = K.Dc, Nc = K.Nc;
-  double2* e64 = K.edge64 + (size_t)g * Dc * Dc;
-  float2* e32 = K.edge32 + (size_t)g * Dc * Dc;
-  double2* n64 = K.node64 + (size_t)g * Nc * Nc;
-  float2* n32 = K.node32 + (size_t)g * Nc * Nc;
-  const double* gph = K.d_ph + 4 * g;
-  int* d_info = K.d_info;
-  PBS_CUDA(cudaMemsetAsync(d_info, 0, 2 * sizeof(int), s));
-  k_assemble_edge<<<dim3((Dc + 127) / 128, Dc), 128, 0, s>>>(C.lvl<double>(), C.wts<double>(), H.mu, gph, e64);
-  PBS_LAUNCHED();
-  k_cholesky<<<1, 256, 0, s>>>(e64, Dc, e32, d_info);
-  PBS_LAUNCHED();
-  const double shift = gamma ? P_diag<double>(C.lvl<double>()) : 0.0;
-  k_assemble_node<<<dim3((Nc + 127) / 128, Nc), 128, 0, s>>>(C.lvl<double>(), gph, shift, n64);
-  PBS_LAUNCHED();
-  k_cholesky<<<1, 256, 0, s>>>(n64, Nc, n32, d_info + 1);
-  PBS_LAUNCHED();
-  int info[2] = {0, 0};
-  PBS_CUDA(cudaMemcpyAsync(info, d_info, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-  PBS_CUDA(cudaStreamSynchronize(s));
-  if (info[0] || info[1]) fail(PBS_ENUMERIC, "coarsest-level Cholesky factorisation failed");
+  const double mx = C.h2 / C.h1, my = C.h1 / C.h2, mn = std::min(mx, my), mxy = std::max(mx, my);
+  const double amax = 16.0 * H.winv_max / (C.h1 * C.h2) + H.mu * mxy;
+  if (!(H.mu * mn / 3.0 > 1e-10 * amax) || !std::isfinite(amax)) return false;
+  if (gamma) return true;
+  const double t1 = std::hypot(ph[0] - 1.0, ph[1]), t2 = std::hypot(ph[2] - 1.0, ph[3]);
+  const double low = 0.25 * mn * (t1 * t1 + t2 * t2) / (double)C.N();
+  return std::isfinite(low) && low > 1e-10 * mxy;
+}
+
+}  // namespace
+
+void set_group_k(DevMem& mem, const Hierarchy& H, KData& K, int g, double k1, double k2, cudaStream_t s) {
+  double ph[4];
+  put_phases(H, K, g, k1, k2, ph, s);
+  factor_groups(H, K, g, 1, s);
+  check_factors(K, s);
+}
+
+void set_group_phases(const Hierarchy& H, KData& K, int g, double k1, double k2, cudaStream_t s) {
+  double ph[4];
+  const bool gamma = put_phases(H, K, g, k1, k2, ph, s);
+  if (factors_certain(H, ph, gamma)) return;
+  factor_groups(H, K, g, 1, s);
+  check_factors(K, s);
+}
+
+void set_all_k(const Hierarchy& H, KData& K, const double* ks, cudaStream_t s) {
+  const int G = K.ngroups;
+  std::vector<double> ph(12 * (size_t)G);
+  std::vector<int> gi(3 * (size_t)G);
+  for (int g = 0; g < G; ++g) {
+    K.k1[g] = ks[2 * g];
+    K.k2[g] = ks[2 * g + 1];
+    K.gamma[g] = bloch_phases(H, ks[2 * g], ks[2 * g + 1], &ph[4 * g]);
+    gi[g] = K.gamma[g];
+  }
+  for (int rep = 1; rep < 3; ++rep) {
+    std::copy(ph.begin(), ph.begin() + 4 * G, ph.begin() + 4 * (size_t)G * rep);
+    std::copy(gi.begin(), gi.begin() + G, gi.begin() + (size_t)G * rep);
+  }
+  PBS_CUDA(cudaMemcpyAsync(K.d_ph, ph.data(), ph.size() * sizeof(double), cudaMemcpyHostToDevice, s));
+  PBS_CUDA(cudaMemcpyAsync(K.d_gamma, gi.data(), gi.size() * sizeof(int), cudaMemcpyHostToDevice, s));
+  factor_groups(H, K, 0, G, s);
+  check_factors(K, s);
 }
 
 void copy_group_k(KData& K, int src, int dst, cudaStream_t s) {

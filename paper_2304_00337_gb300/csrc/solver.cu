@@ -136,6 +136,28 @@ uint64_t fnv1a(const void* data, size_t bytes, uint64_t h = 1469598103934665603u
   return h;
 }
 
+// Hash of an array of 8-byte words in eight independent lanes (word t goes to lane t mod 8):
+// h <- mix(h xor word) with an odd multiplier and a shift, each lane bijective in every word it
+// takes, folded with the length at the end.  A byte-wise chain costs four cycles a byte, 8 ms
+// for the 8 MB of a 1024 x 1024 permittivity; this one reads several bytes a cycle.
+uint64_t hash_words(const double* data, size_t n) {
+  constexpr uint64_t kMul = 0x9e3779b97f4a7c15ull;
+  uint64_t h[8];
+  for (int l = 0; l < 8; ++l) h[l] = kMul * (uint64_t)(2 * l + 1);
+  auto step = [&](uint64_t& x, const double* p) {
+    uint64_t v;
+    std::memcpy(&v, p, sizeof v);
+    x = (x ^ v) * kMul;
+    x ^= x >> 29;
+  };
+  size_t t = 0;
+  for (; t + 8 <= n; t += 8)
+    for (int l = 0; l < 8; ++l) step(h[l], data + t + l);
+  for (; t < n; ++t) step(h[t % 8], data + t);
+  uint64_t r = fnv1a(&n, sizeof n);
+  return fnv1a(h, sizeof h, r);
+}
+
 __global__ void k_hash_eps(const double* __restrict__ eps, long n, unsigned long long* out) {
   unsigned long long h = 0;
   for (long t = blockIdx.x * (long)blockDim.x + threadIdx.x; t < n; t += (long)gridDim.x * blockDim.x) {
@@ -361,15 +383,18 @@ void validate_mesh(double a, double b, int n, int m) {
 double effective_mu(const pbs_opts& o, double a, double b) { return o.mu > 0 ? o.mu : 1.0 / (a * b); }
 
 // Make the context's hierarchy match (geometry, mu, coarsest); eps on the device.
-void ensure_hierarchy(pbs_ctx* ctx, double a, double b, int n, int m, const double* d_eps, uint64_t eps_hash, double mu,
-                      int coarsest) {
-  uint64_t key = eps_hash;
+uint64_t geometry_key(uint64_t key, double a, double b, int n, int m, double mu, int coarsest) {
   key = fnv1a(&a, sizeof a, key);
   key = fnv1a(&b, sizeof b, key);
   key = fnv1a(&n, sizeof n, key);
   key = fnv1a(&m, sizeof m, key);
   key = fnv1a(&mu, sizeof mu, key);
-  key = fnv1a(&coarsest, sizeof coarsest, key);
+  return fnv1a(&coarsest, sizeof coarsest, key);
+}
+
+void ensure_hierarchy(pbs_ctx* ctx, double a, double b, int n, int m, const double* d_eps, uint64_t eps_hash, double mu,
+                      int coarsest) {
+  const uint64_t key = geometry_key(eps_hash, a, b, n, m, mu, coarsest);
   if (ctx->have_h && ctx->H.key == key) return;
   free_work(ctx);  // workspaces depend on the hierarchy sizes
   if (ctx->have_h) free_hierarchy(ctx->mem, ctx->H);
@@ -398,9 +423,10 @@ void ensure_hierarchy_host(pbs_ctx* ctx, const pbs_geom* g, double mu, int coars
   validate_mesh(g->a, g->b, g->n, g->m);
   if (!g->eps) fail(PBS_EINVAL, "eps is NULL");
   const long N = (long)g->n * g->m;
-  const uint64_t h = fnv1a(g->eps, N * sizeof(double));
-  // the permittivity is an input of every call: it is copied each time, and the
-  // resident hierarchy is rebuilt only when geometry, mu or coarsest changed
+  const uint64_t h = hash_words(g->eps, N);
+  // the permittivity is an input of every call and is hashed each time; it is copied, and the
+  // resident hierarchy rebuilt, only when geometry, mu or coarsest changed
+  if (ctx->have_h && ctx->H.key == geometry_key(h, g->a, g->b, g->n, g->m, mu, coarsest)) return;
   if (ctx->d_eps_len != N) {
     ctx->mem.free(ctx->d_eps_in);
     ctx->d_eps_in = nullptr;
@@ -919,9 +945,9 @@ PathResult solve_chain_list(pbs_ctx* ctx, const pbs_opts& o, int nk, const doubl
     gr[g].active = true;
     kfirst[2 * g] = ks[2 * gr[g].pos];
     kfirst[2 * g + 1] = ks[2 * gr[g].pos + 1];
-    set_group_k(ctx->mem, ctx->H, ctx->K, g, kfirst[2 * g], kfirst[2 * g + 1], s);
     seed_history(g);
   }
+  set_all_k(ctx->H, ctx->K, kfirst.data(), s);
   // first Bloch vector of every chain: seeds, a given block, the nested iteration, or a
   // smoothed random start
   const double2* first = dev_init;
@@ -1228,9 +1254,11 @@ const double2* nested_blocks(pbs_ctx* ctx, const pbs_opts& o, int G, const std::
   return W.R();
 }
 
-void set_single_k(pbs_ctx* ctx, double k1, double k2) {
+// the tables of one Bloch vector; `solves`: the call runs coarsest solves and needs the factors
+void set_single_k(pbs_ctx* ctx, double k1, double k2, bool solves) {
   alloc_kdata(ctx->mem, ctx->H, ctx->K, 1);
-  set_group_k(ctx->mem, ctx->H, ctx->K, 0, k1, k2, ctx->stream);
+  if (solves) set_group_k(ctx->mem, ctx->H, ctx->K, 0, k1, k2, ctx->stream);
+  else set_group_phases(ctx->H, ctx->K, 0, k1, k2, ctx->stream);
 }
 
 }  // namespace
@@ -1656,7 +1684,7 @@ int pbs_apply(pbs_ctx* ctx, const pbs_geom* geom, const pbs_opts* opts, int op, 
     if (op < PBS_OP_A || op > PBS_OP_LH_M) fail(PBS_EINVAL, "unknown operator");
     if (op == PBS_OP_PROJECT && level != 0) fail(PBS_EINVAL, "PROJECT acts on level 0");
     if (ncols == 0) return;
-    set_single_k(ctx, k[0], k[1]);
+    set_single_k(ctx, k[0], k[1], op == PBS_OP_VCYCLE_EDGE || op == PBS_OP_VCYCLE_NODAL || op == PBS_OP_PROJECT);
     cudaStream_t us = (cudaStream_t)cuda_stream;
     cudaStream_t s = ctx->stream;
     cudaEvent_t ev;
@@ -1792,7 +1820,7 @@ int pbs_gram(pbs_ctx* ctx, const pbs_geom* geom, const double k[2], int q, const
     pbs_opts o;
     pbs_default_opts(&o);
     ensure_hierarchy_host(ctx, geom, effective_mu(o, geom->a, geom->b), o.coarsest);
-    set_single_k(ctx, k[0], k[1]);
+    set_single_k(ctx, k[0], k[1], false);
     const Level& L0 = ctx->H.lev[0];
     cudaStream_t s = ctx->stream;
     cudaEvent_t ev;
@@ -1827,7 +1855,7 @@ int pbs_m_householder(pbs_ctx* ctx, const pbs_geom* geom, const double k[2], int
     pbs_opts o;
     pbs_default_opts(&o);
     ensure_hierarchy_host(ctx, geom, effective_mu(o, geom->a, geom->b), o.coarsest);
-    set_single_k(ctx, k[0], k[1]);
+    set_single_k(ctx, k[0], k[1], false);
     const Level& L0 = ctx->H.lev[0];
     cudaStream_t s = ctx->stream;
     cudaEvent_t ev;
@@ -1861,7 +1889,7 @@ int pbs_rayleigh_ritz(pbs_ctx* ctx, const pbs_geom* geom, const pbs_opts* opts, 
     const int pw = std::max(p, (q + 2) / 3);
     if (pw > kMaxBlock) fail(PBS_EINVAL, "q too large");
     ensure_work(ctx, pw, 1, o.precision, 0);
-    set_single_k(ctx, k[0], k[1]);
+    set_single_k(ctx, k[0], k[1], project != 0);
     cudaStream_t s = ctx->stream;
     cudaEvent_t ev;
     PBS_CUDA(cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
@@ -2063,13 +2091,7 @@ int pbs_submit(pbs_ctx* ctx, const pbs_geom* geom, const pbs_opts* opts, int nk,
     j->o = *opts;
     {
       const double mu = effective_mu(*opts, geom->a, geom->b);
-      uint64_t key = fnv1a(geom->eps, N * sizeof(double));
-      key = fnv1a(&j->a, sizeof j->a, key);
-      key = fnv1a(&j->b, sizeof j->b, key);
-      key = fnv1a(&j->n, sizeof j->n, key);
-      key = fnv1a(&j->m, sizeof j->m, key);
-      key = fnv1a(&mu, sizeof mu, key);
-      key = fnv1a(&opts->coarsest, sizeof opts->coarsest, key);
+      const uint64_t key = geometry_key(hash_words(geom->eps, N), j->a, j->b, j->n, j->m, mu, opts->coarsest);
       j->gkey = key | 1;
     }
     Server& sv = ctx->srv;
