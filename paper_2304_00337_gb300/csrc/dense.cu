@@ -738,21 +738,47 @@ __global__ void k_gram_finalize(const double2* __restrict__ part, int npart, int
 // Given the Gram matrices GM = S^* M S and GA = S^* A S of a trial block S
 // (q columns), find the p smallest Ritz pairs (Section 4, eq. ritz_eigenvalue):
 //  1. scale to unit diagonal (FP64), Cholesky GM = R^* R dropping directions
-//     whose pivot falls below kDropTol (a span that lost rank);
-//  2. T = R^{-1} by Gauss-Jordan elimination, H = T^* GA T;
+//     whose pivot falls below kDropTol (a span that lost rank), with the same row
+//     operations applied to GA (which leaves R^{-*} GA);
+//  2. H = R^{-*} GA R^{-1}, lower triangle, column by column;
 //  3. Householder reduction H = Q Tr Q^*, Tr Hermitian tridiagonal, made real
-//     by a diagonal unitary scaling;
+//     by a diagonal unitary scaling and scaled by a power of two to norm 1 .. 2;
 //  4. the p smallest eigenvalues of Tr by multisection on Sturm counts, their
-//     eigenvectors by inverse iteration (re-orthogonalised inside clusters);
-//  5. back-transformation and C = D T Q U.
-// Steps 2-5 run in the arithmetic R: FP64 under the plain policy, double-float
+//     eigenvectors by inverse iteration (re-orthogonalised after every sweep);
+//  5. back-transformation and C = D R^{-1} Q U by back substitution.
+// Steps 1-5 run in the arithmetic R: FP64 under the plain policy, double-float
 // (about 48 bits, FP32 pipe) under the mixed one, where the coefficients only need
 // ~1e-14 accuracy (Ritz values and residuals are recomputed in FP64 from the
-// updated block) and a serial chain of FP64 instructions is what limited this
-// one-block kernel on GB300.
+// updated block).
+//
+// What bounds it: one block per Bloch vector, a chain of about 6 q dependent steps;
+// in FP64 every warp instruction holds its quarter of the SM's FP64 pipe for 64
+// cycles whatever its active lanes.  Hence (a) no division or square root on the
+// chains that do not need one (pivots are kept as reciprocals, Sturm counts use the
+// three-term product recurrence instead of quotients), (b) updates of Hermitian
+// matrices form one triangle and store both, spread over all threads, (c) reductions
+// inside a warp with one barrier around them, and (d) both q x q matrices in shared
+// memory up to q = 75 (odd leading dimension: no bank conflicts along rows), which
+// holding R^{-1} as a third matrix prevented beyond q = 55.
 constexpr double kDropTol = 1e-12;  // relative pivot below which a trial direction is dropped
 constexpr int kRRThreads = 512;
 constexpr int kRRWarps = kRRThreads / 32;
+
+// Reciprocal square root in FP64 of a positive finite normal number: binary32 estimate of the
+// significand (exponent handled by integer operations), then two Newton steps
+// y <- y + y (1/2 - (a/2) y^2), each doubling the correct bits (22 -> 44 -> 53, last one by
+// rounding): eleven FP64 instructions.
+__device__ __forceinline__ double rsqrt64(double a) {
+  const unsigned long long u = (unsigned long long)__double_as_longlong(a);
+  const int e = (int)((u >> 52) & 0x7FFu) - 1023, odd = e & 1;
+  const double m = __longlong_as_double((long long)((u & 0xFFFFFFFFFFFFFull) | ((unsigned long long)(1023 + odd) << 52)));
+  double y = f2d_exact(rsqrtf(d2f_rn(m)));
+  const double h = 0.5 * m;
+  y = fma(y, fma(-h * y, y, 0.5), y);
+  y = fma(y, fma(-h * y, y, 0.5), y);
+  // times 2^(-(e - odd)/2)
+  return __longlong_as_double(__double_as_longlong(y) - ((long long)((e - odd) / 2) << 52));
+}
 
 // Arithmetic of the small dense solve: R = df (double-float on the FP32 pipe,
 // the mixed policy) or double (plain FP64).  Ar<R> names the operations the
@@ -769,17 +795,34 @@ struct cd {
   }
 };
 
+// c + x1 y1 + x2 y2 in double-float with one renormalisation
+__device__ __forceinline__ df df_fma2(df c, df x1, df y1, df x2, df y2) {
+  const df p = two_prod(x1.hi, y1.hi), r = two_prod(x2.hi, y2.hi);
+  float lo = __fadd_rn(p.lo, r.lo);
+  lo = __fmaf_rn(x1.hi, y1.lo, __fmaf_rn(x1.lo, y1.hi, lo));
+  lo = __fmaf_rn(x2.hi, y2.lo, __fmaf_rn(x2.lo, y2.hi, lo));
+  const df s = two_sum(p.hi, r.hi), t = two_sum(c.hi, s.hi);
+  lo = __fadd_rn(lo, __fadd_rn(c.lo, __fadd_rn(s.lo, t.lo)));
+  return quick_two_sum(t.hi, lo);
+}
+
 template <class R> struct Ar;
 template <> struct Ar<df> {
   using C = cdf;
   using lead_t = float;  // leading part: comparisons, magnitudes and pivot limits
+  struct Acc {           // running sum of products
+    acc2 a;
+  };
   static __device__ __forceinline__ df mk(float v) { return df_make(v, 0.0f); }
   static __device__ __forceinline__ df zero() { return df_zero(); }
   static __device__ __forceinline__ float lead(df a) { return a.hi; }
   static __device__ __forceinline__ double to(df a) { return df_to(a); }
   static __device__ __forceinline__ df sqrt(df a) { return df_sqrt(a); }
+  static __device__ __forceinline__ df rsqrt(df a) { return mk(1.0f) / df_sqrt(a); }
+  static __device__ __forceinline__ df rcp(df a) { return mk(1.0f) / a; }
   static __device__ __forceinline__ bool lt(df a, df b) { return df_lt(a, b); }
   static __device__ __forceinline__ df mulf(df a, float b) { return df_mul_f(a, b); }
+  static __device__ __forceinline__ df add(df a, df b) { return dfs_add(a, b); }
   static __device__ __forceinline__ df xshfl(df v, int o) { return shfl_df(v, o); }
   static __device__ __forceinline__ df ishfl(df v, int src) {
     return df_make(__shfl_sync(0xffffffffu, v.hi, src), __shfl_sync(0xffffffffu, v.lo, src));
@@ -789,20 +832,46 @@ template <> struct Ar<df> {
   static __device__ __forceinline__ C cfrom(double2 v) { return cdf_from(v); }
   static __device__ __forceinline__ double2 cto(C z) { return cdf_to(z); }
   static __device__ __forceinline__ C conj(C a) { return cdf_conj(a); }
-  static __device__ __forceinline__ C mulc(C a, C b) { return cdf_mulc(a, b); }
   static __device__ __forceinline__ C scale(C a, df s) { return cdf_scale(a, s); }
-  static __device__ __forceinline__ df norm2(C a) { return cdf_norm2(a); }
+  static __device__ __forceinline__ df norm2(C a) { return df_fma2(df_zero(), a.re, a.re, a.im, a.im); }
+  // c + x y, c + x1 y1 + x2 y2
+  static __device__ __forceinline__ df fma1(df c, df x, df y) {
+    const df p = two_prod(x.hi, y.hi), t = two_sum(c.hi, p.hi);
+    const float lo = __fmaf_rn(x.hi, y.lo, __fmaf_rn(x.lo, y.hi, p.lo));
+    return quick_two_sum(t.hi, __fadd_rn(lo, __fadd_rn(c.lo, t.lo)));
+  }
+  static __device__ __forceinline__ df fma2(df c, df x1, df y1, df x2, df y2) { return df_fma2(c, x1, y1, x2, y2); }
+  // x times 2^e (exact while the result stays normal)
+  static __device__ __forceinline__ df pow2(df a, int e) {
+    const float s = __uint_as_float((unsigned)(127 + e) << 23);
+    return df_make(a.hi * s, a.lo * s);
+  }
+  static constexpr int kRescaleEvery = 1;        // Sturm recurrence: steps between range checks
+  static constexpr int kRescaleExp = 48;         // ... and the exponent shift they apply
+  static __device__ __forceinline__ int expo(df a) { return (int)((__float_as_uint(a.hi) >> 23) & 0xFFu) - 127; }
+  static __device__ __forceinline__ bool neg(df a) { return (__float_as_uint(a.hi) >> 31) != 0; }
+  static __device__ __forceinline__ void acc_zero(Acc& a) { a.a = acc2_zero(); }
+  static __device__ __forceinline__ void acc_mul(Acc& a, df x, df y) { dot2(a.a, x, y); }
+  static __device__ __forceinline__ df acc_get(const Acc& a) { return acc2_df(a.a); }
 };
 template <> struct Ar<double> {
   using C = cd;
   using lead_t = double;
+  struct Acc {
+    double a;
+  };
   static __device__ __forceinline__ double mk(double v) { return v; }
   static __device__ __forceinline__ double zero() { return 0.0; }
   static __device__ __forceinline__ double lead(double a) { return a; }
   static __device__ __forceinline__ double to(double a) { return a; }
   static __device__ __forceinline__ double sqrt(double a) { return a > 0.0 ? ::sqrt(a) : 0.0; }
+  static __device__ __forceinline__ double rsqrt(double a) {
+    return a > 1e-290 && a < 1e290 ? rsqrt64(a) : 1.0 / ::sqrt(a);
+  }
+  static __device__ __forceinline__ double rcp(double a) { return 1.0 / a; }
   static __device__ __forceinline__ bool lt(double a, double b) { return a < b; }
   static __device__ __forceinline__ double mulf(double a, float b) { return a * (double)b; }
+  static __device__ __forceinline__ double add(double a, double b) { return a + b; }
   static __device__ __forceinline__ double xshfl(double v, int o) { return __shfl_xor_sync(0xffffffffu, v, o); }
   static __device__ __forceinline__ double ishfl(double v, int src) { return __shfl_sync(0xffffffffu, v, src); }
   static __device__ __forceinline__ C cmk(double r, double i) { return cd{r, i}; }
@@ -810,46 +879,114 @@ template <> struct Ar<double> {
   static __device__ __forceinline__ C cfrom(double2 v) { return cd{v.x, v.y}; }
   static __device__ __forceinline__ double2 cto(C z) { return make_double2(z.re, z.im); }
   static __device__ __forceinline__ C conj(C a) { return cd{a.re, -a.im}; }
-  static __device__ __forceinline__ C mulc(C a, C b) { return cd{a.re * b.re + a.im * b.im, a.re * b.im - a.im * b.re}; }
   static __device__ __forceinline__ C scale(C a, double s) { return cd{a.re * s, a.im * s}; }
-  static __device__ __forceinline__ double norm2(C a) { return a.re * a.re + a.im * a.im; }
+  static __device__ __forceinline__ double norm2(C a) { return fma(a.re, a.re, a.im * a.im); }
+  static __device__ __forceinline__ double fma1(double c, double x, double y) { return fma(x, y, c); }
+  static __device__ __forceinline__ double fma2(double c, double x1, double y1, double x2, double y2) {
+    return fma(x2, y2, fma(x1, y1, c));
+  }
+  static __device__ __forceinline__ double pow2(double a, int e) {
+    return a * __longlong_as_double((long long)(1023 + e) << 52);
+  }
+  static constexpr int kRescaleEvery = 8;
+  static constexpr int kRescaleExp = 400;
+  static __device__ __forceinline__ int expo(double a) {
+    return (int)(((unsigned long long)__double_as_longlong(a) >> 52) & 0x7FFu) - 1023;
+  }
+  static __device__ __forceinline__ bool neg(double a) { return __double_as_longlong(a) < 0; }
+  static __device__ __forceinline__ void acc_zero(Acc& a) { a.a = 0.0; }
+  static __device__ __forceinline__ void acc_mul(Acc& a, double x, double y) { a.a = fma(x, y, a.a); }
+  static __device__ __forceinline__ double acc_get(const Acc& a) { return a.a; }
 };
 
-template <class R> __device__ __forceinline__ R warp_sum_r(R v) {
-  for (int o = 16; o > 0; o >>= 1) v = v + Ar<R>::xshfl(v, o);
+// c - a b and c - conj(a) b
+template <class R>
+__device__ __forceinline__ typename Ar<R>::C cmsub(typename Ar<R>::C c, typename Ar<R>::C a, typename Ar<R>::C b) {
+  return Ar<R>::cmk(Ar<R>::fma2(c.re, -a.re, b.re, a.im, b.im), Ar<R>::fma2(c.im, -a.re, b.im, -a.im, b.re));
+}
+template <class R>
+__device__ __forceinline__ typename Ar<R>::C cmcsub(typename Ar<R>::C c, typename Ar<R>::C a, typename Ar<R>::C b) {
+  return Ar<R>::cmk(Ar<R>::fma2(c.re, -a.re, b.re, -a.im, b.im), Ar<R>::fma2(c.im, -a.re, b.im, a.im, b.re));
+}
+// complex running sum of products
+template <class R> struct CAcc {
+  typename Ar<R>::Acc re, im;
+  __device__ __forceinline__ void zero() {
+    Ar<R>::acc_zero(re);
+    Ar<R>::acc_zero(im);
+  }
+  __device__ __forceinline__ void mul(typename Ar<R>::C a, typename Ar<R>::C b) {  // += a b
+    Ar<R>::acc_mul(re, a.re, b.re);
+    Ar<R>::acc_mul(re, -a.im, b.im);
+    Ar<R>::acc_mul(im, a.re, b.im);
+    Ar<R>::acc_mul(im, a.im, b.re);
+  }
+  __device__ __forceinline__ void mulc(typename Ar<R>::C a, typename Ar<R>::C b) {  // += conj(a) b
+    Ar<R>::acc_mul(re, a.re, b.re);
+    Ar<R>::acc_mul(re, a.im, b.im);
+    Ar<R>::acc_mul(im, a.re, b.im);
+    Ar<R>::acc_mul(im, -a.im, b.re);
+  }
+  __device__ __forceinline__ typename Ar<R>::C get() const { return Ar<R>::cmk(Ar<R>::acc_get(re), Ar<R>::acc_get(im)); }
+};
+// sum over groups of `width` lanes (a power of two); result in every lane of the group
+template <class R> __device__ __forceinline__ R lane_sum_r(R v, int width) {
+  for (int o = width >> 1; o > 0; o >>= 1) v = Ar<R>::add(v, Ar<R>::xshfl(v, o));
   return v;
 }
-template <class R> __device__ __forceinline__ typename Ar<R>::C warp_sum_c(typename Ar<R>::C v) {
-  for (int o = 16; o > 0; o >>= 1) v = v + Ar<R>::cmk(Ar<R>::xshfl(v.re, o), Ar<R>::xshfl(v.im, o));
+template <class R> __device__ __forceinline__ typename Ar<R>::C lane_sum_c(typename Ar<R>::C v, int width) {
+  for (int o = width >> 1; o > 0; o >>= 1)
+    v = Ar<R>::cmk(Ar<R>::add(v.re, Ar<R>::xshfl(v.re, o)), Ar<R>::add(v.im, Ar<R>::xshfl(v.im, o)));
   return v;
-}
-// block-wide sum (all threads participate; result in every thread)
-template <class R> __device__ __forceinline__ R block_sum_r(R v, R* red) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  v = warp_sum_r<R>(v);
-  __syncthreads();
-  if (lane == 0) red[warp] = v;
-  __syncthreads();
-  R t = Ar<R>::zero();
-  for (int w = 0; w < kRRWarps; ++w) t = t + red[w];
-  return t;
 }
 
-// number of eigenvalues of the real symmetric tridiagonal (a, e^2) below x
-template <class R, class P> __device__ int sturm_count_r(const R* a, const R* e2, int n, R x, P pivmin) {
+// Element t of a lower triangle with diagonal (m rows), rows r and m - 1 - r side by side in a
+// line of m + 1: (i, j), i >= j.  Lines: (m + 1) / 2; for odd m the middle line holds (m + 1) / 2
+// elements, the rest of it gives i < j.
+__device__ __forceinline__ void tri_index(int t, int m, float inv_w, int& i, int& j) {
+  const int w = m + 1, r = (int)(((float)t + 0.5f) * inv_w), c = t - r * w;
+  const int top = m - 1 - r;  // the longer row of the pair: top + 1 elements
+  if (c <= top) {
+    i = top;
+    j = c;
+  } else {
+    i = r;
+    j = c - top - 1;
+    if (r == top) j = i + 1;  // the middle row of an odd triangle has no partner
+  }
+}
+
+// Number of eigenvalues below x of the real symmetric tridiagonal (a, e^2) of norm 1 .. 2: sign
+// changes of the leading principal minors p_i = (a_i - x) p_{i-1} - e_{i-1}^2 p_{i-2}, kept in range
+// by common powers of two.  A vanishing minor counts as one of the opposite sign, 2^-60 times the
+// one before it (a perturbation of a_i below its rounding).
+template <class R> __device__ __forceinline__ int sturm_count_r(const R* a, const R* e2, int n, R x) {
   using A = Ar<R>;
   int cnt = 0;
-  R d = a[0] - x;
-  if (fabs(A::lead(d)) < pivmin) d = A::mk(-pivmin);
-  if (A::lead(d) < 0) ++cnt;
+  R p0 = A::mk(1.0f), p1 = a[0] - x;
+  if (A::lead(p1) == 0) p1 = A::pow2(-p0, -60);
+  cnt += A::neg(p1);
   for (int i = 1; i < n; ++i) {
-    d = (a[i] - x) - e2[i - 1] / d;
-    if (fabs(A::lead(d)) < pivmin) d = A::mk(-pivmin);
-    if (A::lead(d) < 0) ++cnt;
+    R p2 = A::fma2(A::zero(), a[i] - x, p1, -e2[i - 1], p0);
+    if (A::lead(p2) == 0) p2 = A::pow2(-p1, -60);
+    cnt += A::neg(p2) != A::neg(p1);
+    p0 = p1;
+    p1 = p2;
+    if (i % A::kRescaleEvery == 0) {
+      const int ex = max(A::expo(p0), A::expo(p1));
+      const int sh = ex > A::kRescaleExp / 2 ? -A::kRescaleExp : ex < -A::kRescaleExp / 2 ? A::kRescaleExp : 0;
+      if (sh) {
+        p0 = A::pow2(p0, sh);
+        p1 = A::pow2(p1, sh);
+      }
+    }
   }
   return cnt;
 }
 
+// Storage of the q x q matrices: in_smem 2: H, U and G in dynamic shared memory, 1: H and U
+// there and G in the scratch array, 0: all in the scratch array (no dynamic shared memory).
+inline __host__ __device__ int rr_ld(int q) { return q | 1; }
 template <class R>
 __global__ void __launch_bounds__(kRRThreads) k_small_rr(const double2* __restrict__ GM, const double2* __restrict__ GA,
                                                          int q, int p, double2* __restrict__ Cout,
@@ -870,20 +1007,22 @@ __global__ void __launch_bounds__(kRRThreads) k_small_rr(const double2* __restri
     info += 8 * g;
     if (phase_out) phase_out += 8 * g;
   }
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = kRRWarps;
-  const long qq = (long)q * q;
-  C* G = (C*)(in_smem ? dsm : scr);  // M-Gram -> R -> Y
-  C* H = G + qq;                        // A-Gram -> H -> reflectors
-  C* T = H + qq;                        // R^{-1}
-  C* U = T + qq;                        // q x p eigenvectors
+  const int tid = threadIdx.x, nt = kRRThreads, lane = tid & 31, warp = tid >> 5;
+  const int ld = rr_ld(q);
+  // H: A-Gram -> R^{-*} A -> H -> reflectors; U: q x p eigenvectors (their real ones Z of the
+  // tridiagonal in the second half of each column); G: M-Gram -> R (row k at G[j ld + k], j >= k)
+  C* H = (C*)(in_smem ? dsm : scr);
+  C* U = H + ld * q;
+  C* G = (C*)(in_smem == 1 ? scr : (double2*)(U + q * p));
+  auto Zc = [&](int j) { return (R*)(U + (long)j * q) + q; };
   __shared__ double d[kMaxTrial];         // column scales (FP64)
   __shared__ int s_keep[kMaxTrial];
+  __shared__ R rinv[kMaxTrial];           // 1 / R_kk
   __shared__ R ta[kMaxTrial], te[kMaxTrial], te2[kMaxTrial], tbeta[kMaxTrial];
-  __shared__ C talpha[kMaxTrial], tphase[kMaxTrial], tvec[kMaxTrial], tp[kMaxTrial];
-  __shared__ R lam[kMaxBlock], lo_s[kMaxBlock], hi_s[kMaxBlock];
-  __shared__ R Z[kMaxTrial * kMaxBlock];  // real eigenvectors of the tridiagonal, column j at j*q
-  __shared__ int s_r, s_bad, s_cnt[kRRThreads];
-  __shared__ R s_piv, s_red[kRRWarps];
+  __shared__ C talpha[kMaxTrial], tphase[kMaxTrial], tv[kMaxTrial], tp[kMaxTrial];
+  __shared__ R lam[kMaxBlock];
+  __shared__ int s_r, s_bad, s_exp;
+  __shared__ R s_k;
   long long t_phase[8];
   t_phase[0] = clock64();
 
@@ -894,43 +1033,56 @@ __global__ void __launch_bounds__(kRRThreads) k_small_rr(const double2* __restri
   }
   if (tid == 0) s_bad = 0;
   __syncthreads();
-  for (long t = tid; t < qq; t += nt) {
-    const int i = int(t % q), j = int(t / q);
+  for (int t = tid; t < q * q; t += nt) {
+    const int i = t % q, j = t / q;
     const double sc = d[i] * d[j];
     const double2 gm = GM[t], ga = GA[t];
     if (!isfinite(gm.x) || !isfinite(gm.y) || !isfinite(ga.x) || !isfinite(ga.y)) s_bad = 1;
-    G[t] = A::cfrom(sc * gm);
-    H[t] = A::cfrom(sc * ga);
-    T[t] = A::czero();
+    G[j * ld + i] = A::cfrom(sc * gm);
+    H[j * ld + i] = A::cfrom(sc * ga);
   }
   __syncthreads();
-  // Cholesky with dropping: R row k stored in G[j*q + k] (j >= k).  A dropped
-  // direction becomes a decoupled unit row and column of R and an isolated Ritz
-  // value above every kept one.
+  // Cholesky with dropping, the row operations applied to H as well: step k scales row k of R
+  // and of H by 1 / R_kk and removes conj(R[k][m]) times them from rows m > k.  A dropped
+  // direction becomes a decoupled unit row and column of R and an isolated Ritz value above
+  // every kept one.
   for (int k = 0; k < q; ++k) {
     if (tid == 0) {
-      const R pv = G[(long)k * q + k].re;
+      const R pv = G[k * ld + k].re;
       const bool keep = d[k] > 0.0 && A::to(pv) > kDropTol && isfinite(A::lead(pv));
       s_keep[k] = keep;
-      s_piv = keep ? A::mk(1.0f) / A::sqrt(pv) : A::zero();  // 1 / R_kk
+      rinv[k] = keep ? A::rsqrt(pv) : A::mk(1.0f);
     }
     __syncthreads();
-    const R inv = s_piv;
-    if (A::lead(inv) > 0.0f) {
-      for (int j = k + tid; j < q; j += nt) G[(long)j * q + k] = A::scale(G[(long)j * q + k], inv);
-      __syncthreads();
+    const R inv = rinv[k];
+    if (s_keep[k]) {
       const int rem = q - k - 1;
-      for (long t = tid; t < (long)rem * rem; t += nt) {
-        const int ii = k + 1 + int(t % rem), jj = k + 1 + int(t / rem);
-        if (ii > jj) continue;
-        G[(long)jj * q + ii] = G[(long)jj * q + ii] - A::mulc(G[(long)ii * q + k], G[(long)jj * q + k]);
+      for (int t = tid; t < rem + q; t += nt) {
+        C* e = t < rem ? G + (k + 1 + t) * ld + k : H + (t - rem) * ld + k;
+        *e = A::scale(*e, inv);
+      }
+      __syncthreads();
+      const int nh = rem * q, ntri = ((rem + 1) / 2) * (rem + 1);
+      const float ih = 1.0f / (float)max(rem, 1), it = 1.0f / (float)(rem + 1);
+      for (int t = tid; t < nh + ntri; t += nt) {
+        if (t < nh) {
+          const int c = (int)(((float)t + 0.5f) * ih), m = k + 1 + (t - c * rem);
+          H[c * ld + m] = cmcsub<R>(H[c * ld + m], G[m * ld + k], H[c * ld + k]);
+        } else {
+          int i, j;
+          tri_index(t - nh, rem, it, i, j);
+          if (i < j) continue;
+          i += k + 1;
+          j += k + 1;  // R row j, column i
+          G[i * ld + j] = cmcsub<R>(G[i * ld + j], G[j * ld + k], G[i * ld + k]);
+        }
       }
     } else {
       for (int j = tid; j < q; j += nt) {
-        G[(long)j * q + k] = A::cmk(A::mk(j == k ? 1.0f : 0.0f), A::zero());
-        if (j < k) G[(long)k * q + j] = A::czero();
-        H[(long)j * q + k] = A::czero();
-        H[(long)k * q + j] = A::czero();
+        if (j > k) G[j * ld + k] = A::czero();
+        if (j < k) G[k * ld + j] = A::czero();
+        H[j * ld + k] = A::czero();
+        H[k * ld + j] = A::czero();
       }
     }
     __syncthreads();
@@ -950,318 +1102,356 @@ __global__ void __launch_bounds__(kRRThreads) k_small_rr(const double2* __restri
   }
   const int r = q;
   t_phase[1] = clock64();
-  // 2a. T = R^{-1}, column c solving R t = e_c by back substitution, one warp per
-  //     column: lanes hold the right-hand side rows; at step k the owner of row k
-  //     divides by R[k][k], broadcasts t_k, and every lane removes R[m][k] t_k from
-  //     its rows m < k (R[m][k] = G[k q + m]).  Rows above c of T stay zero.
-  {
-    const int lane = tid & 31, warp = tid >> 5;
-    constexpr int kSlots = (kMaxTrial + 31) / 32;
-    for (int c = warp; c < r; c += kRRWarps) {
-      C bv[kSlots];
-#pragma unroll
-      for (int sl = 0; sl < kSlots; ++sl)
-        bv[sl] = A::cmk(A::mk(lane + 32 * sl == c ? 1.0f : 0.0f), A::zero());
-      for (int k = c; k >= 0; --k) {
-        const int owner = k & 31, slot = k >> 5;
-        C xk = A::czero();
-#pragma unroll
-        for (int sl = 0; sl < kSlots; ++sl)
-          if (sl == slot && lane == owner) {
-            const R rkk = G[(long)k * q + k].re;
-            xk = A::cmk(bv[sl].re / rkk, bv[sl].im / rkk);
-            T[(long)c * q + k] = xk;
-          }
-        xk = A::cmk(A::ishfl(xk.re, owner), A::ishfl(xk.im, owner));
-#pragma unroll
-        for (int sl = 0; sl < kSlots; ++sl) {
-          const int m = lane + 32 * sl;
-          if (m < k) bv[sl] = bv[sl] - G[(long)k * q + m] * xk;
-        }
-      }
+  // 2. H <- H R^{-1}, lower triangle: column k is scaled, then removed from the columns m > k
+  for (int k = 0; k < q; ++k) {
+    const int rem = q - k - 1;
+    for (int t = tid; t <= rem; t += nt) H[k * ld + k + t] = A::scale(H[k * ld + k + t], rinv[k]);
+    __syncthreads();
+    const int ntri = ((rem + 1) / 2) * (rem + 1);
+    const float it = 1.0f / (float)(rem + 1);
+    for (int t = tid; t < ntri; t += nt) {
+      int i, j;
+      tri_index(t, rem, it, i, j);
+      if (i < j) continue;
+      i += k + 1;
+      j += k + 1;
+      H[j * ld + i] = cmsub<R>(H[j * ld + i], H[k * ld + i], G[j * ld + k]);
     }
+    __syncthreads();
+  }
+  // the upper triangle, exactly Hermitian
+  for (int t = tid; t < q * q; t += nt) {
+    const int i = t % q, c = t / q;
+    if (i > c) H[i * ld + c] = A::conj(H[c * ld + i]);
+    else if (i == c) H[c * ld + i].im = A::zero();
   }
   __syncthreads();
-  // 2b. Y = A T into G (R is no longer needed), then H = T^* Y
-  for (long t = tid; t < (long)r * r; t += nt) {
-    const int i = int(t % r), c = int(t / r);
-    C acc = A::czero();
-    for (int m = 0; m <= c; ++m) acc = acc + H[(long)m * q + i] * T[(long)c * q + m];
-    G[(long)c * q + i] = acc;
-  }
-  __syncthreads();
-  for (long t = tid; t < (long)r * r; t += nt) {
-    const int i = int(t % r), c = int(t / r);
-    C acc = A::czero();
-    for (int m = 0; m <= i; ++m) acc = acc + A::mulc(T[(long)i * q + m], G[(long)c * q + m]);
-    H[(long)c * q + i] = acc;
-  }
-  __syncthreads();
-  // exact Hermitian symmetry, and an isolated value for dropped directions
-  for (long t = tid; t < (long)r * r; t += nt) {
-    const int i = int(t % r), c = int(t / r);
-    if (i < c) {
-      const C up = H[(long)c * q + i], lo = H[(long)i * q + c];
-      const R half = A::mk(0.5f);
-      const C m = A::cmk((up.re + lo.re) * half, (up.im - lo.im) * half);
-      H[(long)c * q + i] = m;
-      H[(long)i * q + c] = A::conj(m);
-    } else if (i == c) {
-      H[(long)c * q + i].im = A::zero();
+  if (s_r < q) {
+    // dropped directions: isolated values above the Gershgorin bound of the kept rows
+    for (int i = tid; i < r; i += nt) {
+      R rs = A::zero();
+      if (s_keep[i])
+        for (int j = 0; j < r; ++j) rs = A::add(rs, A::sqrt(A::norm2(H[j * ld + i])));
+      te[i] = rs;
     }
+    __syncthreads();
+    if (tid == 0) {
+      R bound = A::zero();
+      for (int i = 0; i < r; ++i)
+        if (A::lt(bound, te[i])) bound = te[i];
+      for (int i = 0; i < r; ++i)
+        if (!s_keep[i]) H[i * ld + i] = A::cmk(bound + bound + A::mk(1.0f), A::zero());
+    }
+    __syncthreads();
   }
-  __syncthreads();
-  // Gershgorin row sums of the kept rows (in te, which the reduction below fills
-  // before it is used again), then the bound by one thread
-  for (int i = tid; i < r; i += nt) {
-    R rs = A::zero();
-    if (s_keep[i])
-      for (int j = 0; j < r; ++j) rs = rs + A::sqrt(A::norm2(H[(long)j * q + i]));
-    te[i] = rs;
-  }
-  __syncthreads();
-  if (tid == 0) {
-    R bound = A::zero();
-    for (int i = 0; i < r; ++i)
-      if (A::lt(bound, te[i])) bound = te[i];
-    for (int i = 0; i < r; ++i)
-      if (!s_keep[i]) H[(long)i * q + i] = A::cmk(bound + bound + A::mk(1.0f), A::zero());
-  }
-  __syncthreads();
   t_phase[2] = clock64();
   // 3. Householder tridiagonalisation; reflector k acts on rows/cols k+1..r-1 and is
   //    stored in column k below the diagonal (v, with v_0 = x_0 - alpha) and tbeta[k]
   for (int k = 0; k + 2 < r; ++k) {
     const int m = r - k - 1;
-    R s2 = A::zero();
-    for (int i = tid; i < m; i += nt) s2 = s2 + A::norm2(H[(long)k * q + k + 1 + i]);
-    s2 = block_sum_r<R>(s2, s_red);
-    if (tid == 0) {
-      const R sigma = A::sqrt(s2);
-      const C x0 = H[(long)k * q + k + 1];
-      const R ax0 = A::sqrt(A::norm2(x0));
-      C ph = A::lead(ax0) > 0.0f ? A::cmk(x0.re / ax0, x0.im / ax0) : A::cmk(A::mk(1.0f), A::zero());
-      if (A::lead(sigma) > 0.0f) {
-        const C alpha = -A::scale(ph, sigma);
-        talpha[k] = alpha;
-        tbeta[k] = A::mk(1.0f) / (sigma * (sigma + ax0));
-        H[(long)k * q + k + 1] = x0 - alpha;
-      } else {
-        talpha[k] = x0;
-        tbeta[k] = A::zero();
+    C* x = H + k * ld + k + 1;
+    if (warp == 0) {
+      // alpha = -(x_0 / |x_0|) sigma, beta = 1 / (sigma (sigma + |x_0|)), sigma = |x|
+      typename A::Acc s2a;
+      A::acc_zero(s2a);
+      for (int i = lane; i < m; i += 32) {
+        A::acc_mul(s2a, x[i].re, x[i].re);
+        A::acc_mul(s2a, x[i].im, x[i].im);
+      }
+      const R s2 = lane_sum_r<R>(A::acc_get(s2a), 32);
+      if (lane == 0) {
+        const C x0 = x[0];
+        if (A::lead(s2) > LT(0)) {
+          const R n0 = A::norm2(x0), is = A::rsqrt(s2), sigma = s2 * is;
+          C ph = A::cmk(A::mk(1.0f), A::zero());
+          R ax0 = A::zero();
+          if (A::lead(n0) > LT(0)) {
+            const R i0 = A::rsqrt(n0);
+            ax0 = n0 * i0;
+            ph = A::scale(x0, i0);
+          }
+          const C alpha = -A::scale(ph, sigma);
+          talpha[k] = alpha;
+          tbeta[k] = A::rcp(A::add(s2, sigma * ax0));
+          x[0] = x0 - alpha;
+        } else {
+          talpha[k] = x0;
+          tbeta[k] = A::zero();
+        }
       }
     }
     __syncthreads();
     const R beta = tbeta[k];
-    if (A::lead(beta) != 0.0f) {
-      // p = beta * Hsub v (rows by warps, columns by lanes)
-      for (int i = warp; i < m; i += nw) {
-        C acc = A::czero();
-        for (int j = lane; j < m; j += 32) acc = acc + H[(long)(k + 1 + j) * q + k + 1 + i] * H[(long)k * q + k + 1 + j];
-        acc = warp_sum_c<R>(acc);
-        if (lane == 0) tp[i] = A::scale(acc, beta);
+    if (A::lead(beta) != LT(0)) {
+      // p = beta Hsub v: `seg` neighbouring lanes share a row
+      int seg = 16;
+      while (seg > 4 && seg * m > nt) seg >>= 1;
+      for (int base = 0; base < m; base += nt / seg) {  // the same trips in every lane
+        const int i = base + tid / seg;
+        CAcc<R> acc;
+        acc.zero();
+        if (i < m)
+          for (int j = tid % seg; j < m; j += seg) acc.mul(H[(k + 1 + j) * ld + k + 1 + i], x[j]);
+        const C sum = lane_sum_c<R>(acc.get(), seg);
+        if (i < m && tid % seg == 0) tp[i] = A::scale(sum, beta);
       }
       __syncthreads();
-      // K = beta/2 v^* p (real for Hermitian H); w = p - K v
-      R kk = A::zero();
-      for (int i = tid; i < m; i += nt) kk = kk + A::mulc(H[(long)k * q + k + 1 + i], tp[i]).re;
-      kk = block_sum_r<R>(kk, s_red);
-      const R K = kk * beta * A::mk(0.5f);
-      for (int i = tid; i < m; i += nt) tvec[i] = tp[i] - A::scale(H[(long)k * q + k + 1 + i], K);
+      if (warp == 0) {  // K = beta/2 v^* p (real for Hermitian H)
+        typename A::Acc ka;
+        A::acc_zero(ka);
+        for (int i = lane; i < m; i += 32) {
+          A::acc_mul(ka, x[i].re, tp[i].re);
+          A::acc_mul(ka, x[i].im, tp[i].im);
+        }
+        const R kk = lane_sum_r<R>(A::acc_get(ka), 32);
+        const R K = A::mulf(kk * beta, 0.5f);
+        for (int i = lane; i < m; i += 32) tv[i] = tp[i] - A::scale(x[i], K);  // w = p - K v
+      }
       __syncthreads();
-      // Hsub -= v w^* + w v^*
-      for (long t = tid; t < (long)m * m; t += nt) {
-        const int i = int(t % m), j = int(t / m);
-        const C vi = H[(long)k * q + k + 1 + i], vj = H[(long)k * q + k + 1 + j];
-        C h = H[(long)(k + 1 + j) * q + k + 1 + i];
-        h = h - vi * A::conj(tvec[j]) - tvec[i] * A::conj(vj);
-        H[(long)(k + 1 + j) * q + k + 1 + i] = h;
+      // Hsub -= v w^* + w v^*: the lower triangle, mirrored
+      const int ntri = ((m + 1) / 2) * (m + 1);
+      const float it = 1.0f / (float)(m + 1);
+      for (int t = tid; t < ntri; t += nt) {
+        int i, j;
+        tri_index(t, m, it, i, j);
+        if (i < j) continue;
+        const C vi = x[i], vj = x[j], wi = tv[i], wj = tv[j];
+        C h = H[(k + 1 + j) * ld + k + 1 + i];
+        // h - vi conj(wj) - wi conj(vj)
+        h = cmcsub<R>(h, wj, vi);
+        h = cmcsub<R>(h, vj, wi);
+        if (i == j) h.im = A::zero();
+        H[(k + 1 + j) * ld + k + 1 + i] = h;
+        if (i != j) H[(k + 1 + i) * ld + k + 1 + j] = A::conj(h);
       }
     }
     __syncthreads();
   }
   // real tridiagonal: diagonal ta, off-diagonal te = |alpha|, phases tphase
-  if (tid == 0) {
-    C ph = A::cmk(A::mk(1.0f), A::zero());
-    for (int k = 0; k < r; ++k) {
-      ta[k] = H[(long)k * q + k].re;
-      tphase[k] = ph;
-      if (k + 1 < r) {
-        const C al = (k + 2 < r) ? talpha[k] : H[(long)k * q + k + 1];
-        const R aa = A::sqrt(A::norm2(al));
-        te[k] = aa;
-        te2[k] = aa * aa;
-        if (A::lead(aa) > 0.0f) ph = ph * A::cmk(al.re / aa, al.im / aa);
+  for (int k = tid; k < r; k += nt) {
+    ta[k] = H[k * ld + k].re;
+    if (k + 1 < r) {
+      const C al = (k + 2 < r) ? talpha[k] : H[k * ld + k + 1];
+      const R n2 = A::norm2(al);
+      if (A::lead(n2) > LT(0)) {
+        const R in = A::rsqrt(n2);
+        te[k] = n2 * in;
+        tp[k] = A::scale(al, in);
+      } else {
+        te[k] = A::zero();
+        tp[k] = A::cmk(A::mk(1.0f), A::zero());
       }
     }
   }
   __syncthreads();
-  t_phase[3] = clock64();
-  // 4a. multisection: each warp refines one wanted eigenvalue at a time, its 32
-  //     lanes evaluating the Sturm count at 32 interior points of the bracket
-  R lo = A::zero(), hi = A::zero();
-  for (int k = 0; k < r; ++k) {
-    const R rad = (k > 0 ? te[k - 1] : A::zero()) + (k + 1 < r ? te[k] : A::zero());
-    const R l = ta[k] - rad, h = ta[k] + rad;
-    if (k == 0 || A::lt(l, lo)) lo = l;
-    if (k == 0 || A::lt(hi, h)) hi = h;
+  if (tid == 0) {
+    C ph = A::cmk(A::mk(1.0f), A::zero());
+    for (int k = 0; k < r; ++k) {
+      tphase[k] = ph;
+      if (k + 1 < r) ph = ph * tp[k];
+    }
   }
+  // Gershgorin interval, and the power of two that brings its larger end to 1 .. 2
+  R lo = A::zero(), hi = A::zero();
+  {
+    LT l = LT(0), h = LT(0);
+    bool first = true;
+    for (int k = lane; k < r; k += 32) {
+      const LT rad = (k > 0 ? A::lead(te[k - 1]) : LT(0)) + (k + 1 < r ? A::lead(te[k]) : LT(0)), a = A::lead(ta[k]);
+      l = first ? a - rad : fmin(l, a - rad);
+      h = first ? a + rad : fmax(h, a + rad);
+      first = false;
+    }
+    if (first) {  // fewer entries than lanes: copy lane 0's
+      l = A::lead(ta[0]);
+      h = l;
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+      l = fmin(l, __shfl_xor_sync(0xffffffffu, l, o));
+      h = fmax(h, __shfl_xor_sync(0xffffffffu, h, o));
+    }
+    lo = A::mk(l);
+    hi = A::mk(h);
+  }
+  const LT anorm = fmax(fabs(A::lead(lo)), fabs(A::lead(hi)));
+  const int ex = anorm > LT(0) ? A::expo(A::mk(anorm)) : 0;  // anorm in 2^ex .. 2^(ex+1)
+  const int sc1 = max(-100, min(100, -ex));  // |ex| stays far below 100 for any pencil of this discretisation
+  lo = A::pow2(lo, sc1);
+  hi = A::pow2(hi, sc1);
+  __syncthreads();
+  for (int k = tid; k < r; k += nt) {
+    ta[k] = A::pow2(ta[k], sc1);
+    const R e = k + 1 < r ? A::pow2(te[k], sc1) : A::zero();
+    te[k] = e;
+    te2[k] = e * e;
+  }
+  if (tid == 0) s_exp = -sc1;
+  __syncthreads();
+  t_phase[3] = clock64();
+  // 4a. multisection: a group of lanes refines one wanted eigenvalue at a time, each lane
+  //     evaluating the Sturm count at one interior point of the bracket (a warp per eigenvalue,
+  //     half a warp when more than kRRWarps are wanted)
   const LT tnorm = fmax(fabs(A::lead(lo)), fabs(A::lead(hi))) + LT(1e-30);
-  // Sturm pivots below pivmin are replaced by -pivmin: e^2 / pivmin stays far below the float range
-  const LT pivmin = fmax(LT(1e-30) * tnorm * tnorm, LT(1e-36));
   // inverse iteration: pivots are kept above the accuracy of the shift, so a solve
   // grows the vector by at most ~1e14 and never leaves the float range
   const LT pivmin_ii = LT(1e-14) * tnorm;
-  for (int j = warp; j < p; j += nw) {
-    R a0 = lo - A::mk(1e-6f * tnorm), b0 = hi + A::mk(1e-6f * tnorm);
-    for (int it = 0; it < 24; ++it) {
-      const R w = b0 - a0;
-      if (A::to(w) <= 4e-15 * (double)tnorm) break;
-      const R x = a0 + A::mulf(w, float(lane + 1) / 33.0f);
-      const int cnt = sturm_count_r<R>(ta, te2, r, x, pivmin);
-      // new bracket: largest point with count <= j, smallest with count > j
-      const unsigned below = __ballot_sync(0xffffffffu, cnt <= j);
-      const int nb = __popc(below);  // points 0..nb-1 have count <= j (counts increase with x)
-      const R xa = A::ishfl(x, nb > 0 ? nb - 1 : 0);
-      const R xb = A::ishfl(x, nb < 32 ? nb : 31);
-      if (nb > 0) a0 = xa;
-      if (nb < 32) b0 = xb;
-    }
-    if (lane == 0) {
-      lam[j] = (a0 + b0) * A::mk(0.5f);
-      lo_s[j] = a0;
-      hi_s[j] = b0;
+  {
+    const int wd = p > kRRWarps ? 16 : 32, per = 32 / wd, sub = lane / wd, sl = lane % wd;
+    const unsigned gmask = (wd == 32 ? 0xffffffffu : 0xffffu) << (sub * wd);
+    const int j = warp * per + sub, jj = min(j, p - 1);
+    if (warp * per < p) {
+      R a0 = lo - A::mk(1e-6f * tnorm), b0 = hi + A::mk(1e-6f * tnorm);
+      for (int it = 0; it < 30; ++it) {
+        const R w = b0 - a0;
+        const bool done = A::to(w) <= 4e-15 * (double)tnorm;
+        if (__all_sync(0xffffffffu, done)) break;
+        const R x = a0 + A::mulf(w, float(sl + 1) / float(wd + 1));
+        const int cnt = sturm_count_r<R>(ta, te2, r, x);
+        // new bracket: largest point with count <= jj, smallest with count > jj
+        const unsigned below = __ballot_sync(0xffffffffu, cnt <= jj) & gmask;
+        const int nb = __popc(below);  // points 0..nb-1 have count <= jj (counts increase with x)
+        const R xa = A::ishfl(x, sub * wd + (nb > 0 ? nb - 1 : 0));
+        const R xb = A::ishfl(x, sub * wd + (nb < wd ? nb : wd - 1));
+        if (!done && nb > 0) a0 = xa;
+        if (!done && nb < wd) b0 = xb;
+      }
+      if (sl == 0 && j < p) lam[j] = A::mulf(a0 + b0, 0.5f);
     }
   }
   __syncthreads();
   t_phase[4] = clock64();
   // 4b. inverse iteration on Tr - lam_j I (Gaussian elimination with partial
-  //     pivoting, factored once), one thread per eigenvalue; cluster members
+  //     pivoting, factored once, pivots as reciprocals), one thread per eigenvalue;
   //     re-orthogonalised after every sweep
   R u0[kMaxTrial], u1[kMaxTrial], u2[kMaxTrial], mult[kMaxTrial];
-  bool swp[kMaxTrial];
+  unsigned swp[(kMaxTrial + 31) / 32] = {};
   if (tid < p) {
     const R shift = lam[tid];
     R d0 = ta[0] - shift, s1 = r > 1 ? te[0] : A::zero();
     for (int i = 0; i < r; ++i) {
-      const R below_sub = i + 1 < r ? te[i] : A::zero();
-      const R below_diag = i + 1 < r ? ta[i + 1] - shift : A::zero();
-      const R below_sup = i + 2 < r ? te[i + 1] : A::zero();
-      if (i + 1 < r && fabs(A::lead(below_sub)) > fabs(A::lead(d0))) {
-        swp[i] = true;
-        u0[i] = below_sub;
-        u1[i] = below_diag;
-        u2[i] = below_sup;
-        const R mlt = d0 / below_sub;
-        mult[i] = mlt;
-        d0 = s1 - mlt * below_diag;
-        s1 = -(mlt * below_sup);
-      } else {
-        swp[i] = false;
-        R dd = d0;
-        if (fabs(A::lead(dd)) < pivmin_ii) dd = A::mk(A::lead(dd) < 0.0f ? -pivmin_ii : pivmin_ii);
-        u0[i] = dd;
-        u1[i] = s1;
-        u2[i] = A::zero();
-        const R mlt = i + 1 < r ? below_sub / dd : A::zero();
-        mult[i] = mlt;
-        d0 = below_diag - mlt * s1;
-        s1 = below_sup;
-      }
+      const R bsub = te[i], bdiag = i + 1 < r ? ta[i + 1] - shift : A::zero(), bsup = i + 1 < r ? te[i + 1] : A::zero();
+      const bool sw = i + 1 < r && fabs(A::lead(bsub)) > fabs(A::lead(d0));
+      R pv = sw ? bsub : d0;
+      if (fabs(A::lead(pv)) < pivmin_ii) pv = A::mk(A::lead(pv) < LT(0) ? -pivmin_ii : pivmin_ii);
+      const R ip = A::rcp(pv), ml = (sw ? d0 : bsub) * ip;
+      const R p1 = sw ? bdiag : s1, p2 = sw ? bsup : A::zero();
+      const R o1 = sw ? s1 : bdiag, o2 = sw ? A::zero() : bsup;
+      u0[i] = ip;
+      u1[i] = p1;
+      u2[i] = p2;
+      mult[i] = ml;
+      if (sw) swp[i >> 5] |= 1u << (i & 31);
+      d0 = A::fma1(o1, -ml, p1);
+      s1 = A::fma1(o2, -ml, p2);
     }
   }
-  for (int sweep = 0; sweep < 4; ++sweep) {
+  for (int sweep = 0; sweep < 3; ++sweep) {
     if (tid < p) {
       const int j = tid;
-      R* z = Z + j * q;
-      if (sweep == 0)
-        for (int i = 0; i < r; ++i) z[i] = A::mk(1.0f + 0.37f * __sinf(1.7f * (i + 1) * (j + 1)));
+      R* z = Zc(j);
+      // forward: the running right-hand side of row i + 1 stays in a register
+      R cur = sweep == 0 ? A::mk(1.0f + 0.37f * __sinf(1.7f * (j + 1))) : z[0];
       for (int i = 0; i + 1 < r; ++i) {
-        if (swp[i]) {
-          const R t0 = z[i];
-          z[i] = z[i + 1];
-          z[i + 1] = t0 - mult[i] * z[i];
-        } else {
-          z[i + 1] = z[i + 1] - mult[i] * z[i];
-        }
+        const R nx = sweep == 0 ? A::mk(1.0f + 0.37f * __sinf(1.7f * (i + 2) * (j + 1))) : z[i + 1];
+        const bool sw = (swp[i >> 5] >> (i & 31)) & 1u;
+        const R top = sw ? nx : cur;
+        cur = A::fma1(sw ? cur : nx, -mult[i], top);
+        z[i] = top;
       }
-      for (int i = r - 1; i >= 0; --i) {
-        R v = z[i];
-        if (i + 1 < r) v = v - u1[i] * z[i + 1];
-        if (i + 2 < r) v = v - u2[i] * z[i + 2];
-        R dd = u0[i];
-        if (fabs(A::lead(dd)) < pivmin_ii) dd = A::mk(A::lead(dd) < 0.0f ? -pivmin_ii : pivmin_ii);
-        z[i] = v / dd;
+      R z1 = cur * u0[r - 1], z2 = A::zero();
+      z[r - 1] = z1;
+      LT zmax = fabs(A::lead(z1));
+      for (int i = r - 2; i >= 0; --i) {
+        const R v = A::fma2(z[i], -u1[i], z1, -u2[i], z2) * u0[i];
+        z[i] = v;
+        zmax = fmax(zmax, fabs(A::lead(v)));
+        z2 = z1;
+        z1 = v;
       }
-      LT zmax = 0;
-      for (int i = 0; i < r; ++i) zmax = fmax(zmax, fabs(A::lead(z[i])));
-      const float sc = zmax > 0 ? float(1.0 / zmax) : 1.0f;
-      R nrm = A::zero();
+      const float sc = zmax > 0 ? float(1.0f / float(zmax)) : 1.0f;
+      typename A::Acc na;
+      A::acc_zero(na);
       for (int i = 0; i < r; ++i) {
-        z[i] = A::mulf(z[i], sc);
-        nrm = nrm + z[i] * z[i];
+        const R v = A::mulf(z[i], sc);
+        z[i] = v;
+        A::acc_mul(na, v, v);
       }
-      const R inv = A::mk(1.0f) / A::sqrt(nrm);
+      const R inv = A::rsqrt(A::acc_get(na));
       for (int i = 0; i < r; ++i) z[i] = z[i] * inv;
     }
     __syncthreads();
-    // modified Gram-Schmidt against earlier vectors whose eigenvalues lie within
-    // 1e-3 |T| (the usual reorthogonalisation window of inverse iteration);
-    // warp 0, lanes over the components
-    if (warp == 0) {
-      for (int j = 1; j < p; ++j) {
-        R* zj = Z + j * q;
-        bool touched = false;
-        for (int c = 0; c < j; ++c) {
-          if (A::to(lam[j] - lam[c]) > 1e-3 * (double)tnorm) continue;
-          const R* zc = Z + c * q;
-          R dot = A::zero();
-          for (int i = lane; i < r; i += 32) dot = dot + zc[i] * zj[i];
-          dot = warp_sum_r<R>(dot);
-          for (int i = lane; i < r; i += 32) zj[i] = zj[i] - dot * zc[i];
-          __syncwarp();
-          touched = true;
+    // modified Gram-Schmidt against every earlier vector (inverse iteration alone leaves
+    // inner products of about 2^-53 |T| / gap): vector c is removed from the later ones at
+    // once (a warp per vector, lanes over the components), and the next one normalised by
+    // its warp
+    for (int c = 0; c + 1 < p; ++c) {
+      const R* zc = Zc(c);
+      for (int j = c + 1 + warp; j < p; j += kRRWarps) {
+        R* zj = Zc(j);
+        typename A::Acc da;
+        A::acc_zero(da);
+        for (int i = lane; i < r; i += 32) A::acc_mul(da, zc[i], zj[i]);
+        const R dot = lane_sum_r<R>(A::acc_get(da), 32);
+        typename A::Acc na;
+        A::acc_zero(na);
+        for (int i = lane; i < r; i += 32) {
+          const R v = A::fma1(zj[i], -dot, zc[i]);
+          zj[i] = v;
+          if (j == c + 1) A::acc_mul(na, v, v);
         }
-        if (touched) {
-          R nrm = A::zero();
-          for (int i = lane; i < r; i += 32) nrm = nrm + zj[i] * zj[i];
-          nrm = warp_sum_r<R>(nrm);
-          const R inv = A::mk(1.0f) / A::sqrt(nrm);
+        if (j == c + 1) {
+          const R inv = A::rsqrt(lane_sum_r<R>(A::acc_get(na), 32));
           for (int i = lane; i < r; i += 32) zj[i] = zj[i] * inv;
-          __syncwarp();
         }
       }
+      __syncthreads();
     }
-    __syncthreads();
   }
   t_phase[5] = clock64();
-  // 5. back-transformation u_j = Q (phase * z_j), then C = D T u (one warp per vector)
-  for (int j = warp; j < p; j += nw) {
-    C* u = U + (long)j * q;
-    for (int i = lane; i < r; i += 32) u[i] = A::scale(tphase[i], Z[j * q + i]);
-    __syncwarp();
-    for (int k = r - 3; k >= 0; --k) {
-      const R beta = tbeta[k];
-      if (A::lead(beta) == 0.0f) continue;
-      const int m = r - k - 1;
-      C acc = A::czero();
-      for (int i = lane; i < m; i += 32) acc = acc + A::mulc(H[(long)k * q + k + 1 + i], u[k + 1 + i]);
-      acc = warp_sum_c<R>(acc);
-      const C f = A::scale(acc, beta);
-      for (int i = lane; i < m; i += 32) u[k + 1 + i] = u[k + 1 + i] - H[(long)k * q + k + 1 + i] * f;
+  // 5. back-transformation u_j = Q (phase * z_j), then C = D R^{-1} u_j, half a warp per vector
+  {
+    const int hl = lane & 15, j = 2 * warp + (lane >> 4);
+    const bool on = j < p;
+    C* u = U + (long)(on ? j : 0) * q;
+    constexpr int kSlots = kMaxTrial / 16;
+    if (2 * warp < p) {
+      R zr[kSlots];
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl)
+        if (hl + 16 * sl < r) zr[sl] = Zc(on ? j : 0)[hl + 16 * sl];
       __syncwarp();
-    }
-    for (int i = lane; i < q; i += 32) {
-      C acc = A::czero();
-      for (int m = i; m < r; ++m) acc = acc + T[(long)m * q + i] * u[m];
-      Cout[(long)j * q + i] = s_keep[i] ? d[i] * A::cto(acc) : make_double2(0, 0);
+#pragma unroll
+      for (int sl = 0; sl < kSlots; ++sl)
+        if (on && hl + 16 * sl < r) u[hl + 16 * sl] = A::scale(tphase[hl + 16 * sl], zr[sl]);
+      __syncwarp();
+      for (int k = r - 3; k >= 0; --k) {
+        const R beta = tbeta[k];
+        if (A::lead(beta) == LT(0)) continue;
+        const int m = r - k - 1;
+        const C* v = H + k * ld + k + 1;
+        CAcc<R> acc;
+        acc.zero();
+        if (on)
+          for (int i = hl; i < m; i += 16) acc.mulc(v[i], u[k + 1 + i]);
+        const C f = A::scale(lane_sum_c<R>(acc.get(), 16), beta);
+        if (on)
+          for (int i = hl; i < m; i += 16) u[k + 1 + i] = cmsub<R>(u[k + 1 + i], v[i], f);
+        __syncwarp();
+      }
+      for (int k = r - 1; k >= 0; --k) {
+        const C xk = A::scale(u[k], rinv[k]);
+        if (on)
+          for (int i = hl; i < k; i += 16) u[i] = cmsub<R>(u[i], G[k * ld + i], xk);
+        if (on && hl == (k & 15)) Cout[(long)j * q + k] = s_keep[k] ? d[k] * A::cto(xk) : make_double2(0, 0);
+        __syncwarp();
+      }
     }
   }
-  for (int j = tid; j < p; j += nt) theta_out[j] = A::to(lam[j]);
+  for (int j = tid; j < p; j += nt) theta_out[j] = ldexp(A::to(lam[j]), s_exp);
   __syncthreads();
   // a non-finite coefficient means a breakdown: report it instead of passing it on
   int bad = 0;
-  for (long t = tid; t < (long)q * p; t += nt) {
+  for (int t = tid; t < q * p; t += nt) {
     const double2 c = Cout[t];
     bad |= !(isfinite(c.x) && isfinite(c.y));
   }
@@ -1637,22 +1827,26 @@ size_t small_rr_scratch(int q) { return (3ull * q * q + (size_t)q * kMaxBlock) *
 void small_rr(const double2* GM, const double2* GA, int q, int p, double2* C, double* theta, double2* scratch,
               int* d_info, int ngroups, bool dfa, cudaStream_t s) {
   if (q > kMaxTrial || p > q || p < 1 || p > kMaxBlock || ngroups < 1) fail(PBS_EINVAL, "small_rr: bad sizes");
-  const size_t dyn = (3ull * q * q + (size_t)q * p) * sizeof(double2);
-  const int in_smem = dyn <= 150 * 1024 ? 1 : 0;
+  // H and U, then G, in dynamic shared memory as far as they fit beside the static arrays
+  constexpr size_t kRRSmem = 212 * 1024;
+  const size_t hu = ((size_t)rr_ld(q) * q + (size_t)q * p) * sizeof(double2);
+  const size_t all = hu + (size_t)rr_ld(q) * q * sizeof(double2);
+  const int in_smem = all <= kRRSmem ? 2 : hu <= kRRSmem ? 1 : 0;
+  const size_t dyn = in_smem == 2 ? all : in_smem == 1 ? hu : 0;
   static PerDeviceOnce once;
   once([] {
-    PBS_CUDA(cudaFuncSetAttribute(k_small_rr<df>, cudaFuncAttributeMaxDynamicSharedMemorySize, 150 * 1024));
-    PBS_CUDA(cudaFuncSetAttribute(k_small_rr<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, 150 * 1024));
+    PBS_CUDA(cudaFuncSetAttribute(k_small_rr<df>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRRSmem));
+    PBS_CUDA(cudaFuncSetAttribute(k_small_rr<double>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRRSmem));
   });
   const long stride = (long)(small_rr_scratch(q) / sizeof(double2));
   timer_begin(KC_SMALL_RR, s, 8.0 * 3.0 * q * q * q * ngroups);  // flops, order of magnitude
   int* phases = verbose_enabled() ? d_info + 2 : nullptr;
   if (dfa) {
-    k_small_rr<df><<<ngroups, kRRThreads, in_smem ? dyn : 0, s>>>(GM, GA, q, p, C, theta, scratch, d_info, in_smem,
+    k_small_rr<df><<<ngroups, kRRThreads, dyn, s>>>(GM, GA, q, p, C, theta, scratch, d_info, in_smem,
                                                                   phases, stride);
     count_df_launch();
   } else {
-    k_small_rr<double><<<ngroups, kRRThreads, in_smem ? dyn : 0, s>>>(GM, GA, q, p, C, theta, scratch, d_info,
+    k_small_rr<double><<<ngroups, kRRThreads, dyn, s>>>(GM, GA, q, p, C, theta, scratch, d_info,
                                                                       in_smem, phases, stride);
   }
   timer_end(KC_SMALL_RR, s);
