@@ -1345,7 +1345,8 @@ __global__ void __launch_bounds__(kRRThreads) k_small_rr(const double2* __restri
       s1 = A::fma1(o2, -ml, p2);
     }
   }
-  for (int sweep = 0; sweep < 3; ++sweep) {
+  // (an even number: each solve may flip a vector's sign with that of lam_j's rounding error)
+  for (int sweep = 0; sweep < 2; ++sweep) {
     if (tid < p) {
       const int j = tid;
       R* z = Zc(j);
