@@ -242,11 +242,21 @@ struct WtsDF {
   }
 };
 
-// Level geometry constants.
+// Level geometry constants.  The nodal operator's stencil coefficients and the reciprocal of its
+// diagonal follow from mx and my; they are formed once on the host (an FP64 division per thread
+// costs as much as a node update).
 template <class T> struct Lvl {
   int n, m;
   T mx;  // h2/h1: mass and curl-curl scaling along x-edges
   T my;  // h1/h2
+  T pe = T(1.0 / 3.0) * (my - T(2) * mx);  // east and west neighbours
+  T pn = T(1.0 / 3.0) * (mx - T(2) * my);  // north and south
+  T pd = T(-1.0 / 6.0) * (mx + my);        // diagonal neighbours
+  T pinv = T(1) / (T(4.0 / 3.0) * (mx + my));
+};
+template <> struct Lvl<df> {
+  int n, m;
+  df mx, my;
 };
 
 template <class T, class R> __device__ __forceinline__ cx<T> curl_at(const R& r, int i, int j) {
@@ -285,15 +295,17 @@ template <class T> struct UnitNRd {
     return (j * n + i == idx) ? ph : czero<T>();
   }
 };
+// Its coefficients: 4/3 (mx + my) at the centre, (my - 2 mx)/3 east and west, (mx - 2 my)/3 north
+// and south, -(mx + my)/6 on the diagonals.  They sum to zero, so the stencil is applied to the
+// differences from the centre: a constant field gives exactly zero (coefficients that only sum to
+// zero up to rounding would shift the smoothest modes), and a node takes 11 operations per
+// component instead of 20 in tensor-product form.
 template <class T, class R> __device__ __forceinline__ cx<T> P_at(const R& r, const Lvl<T>& L, int i, int j) {
-  cx<T> acc_x = czero<T>(), acc_y = czero<T>();
-#pragma unroll
-  for (int d = -1; d <= 1; ++d) {
-    const T wgt = d == 0 ? T(4) : T(1);
-    acc_x = acc_x + wgt * (T(2) * r.v(i, j + d) - r.v(i - 1, j + d) - r.v(i + 1, j + d));
-    acc_y = acc_y + wgt * (T(2) * r.v(i + d, j) - r.v(i + d, j - 1) - r.v(i + d, j + 1));
-  }
-  return (L.mx * T(1.0 / 6.0)) * acc_x + (L.my * T(1.0 / 6.0)) * acc_y;
+  const cx<T> v0 = r.v(i, j);
+  const cx<T> e = (r.v(i - 1, j) + r.v(i + 1, j)) - T(2) * v0;
+  const cx<T> n = (r.v(i, j - 1) + r.v(i, j + 1)) - T(2) * v0;
+  const cx<T> d = ((r.v(i - 1, j - 1) + r.v(i + 1, j - 1)) + (r.v(i - 1, j + 1) + r.v(i + 1, j + 1))) - T(4) * v0;
+  return L.pe * e + L.pn * n + L.pd * d;
 }
 template <class T> __host__ __device__ __forceinline__ T P_diag(const Lvl<T>& L) {
   return T(4.0 / 3.0) * (L.mx + L.my);

@@ -37,6 +37,7 @@
 #include "internal.h"
 #include "mgpoint.cuh"
 #include "nodal_tiles.cuh"
+#include "tail.cuh"
 
 namespace pbs {
 
@@ -131,18 +132,16 @@ __device__ __forceinline__ double2 coarse_node_entry(const Lvl<double>& L, const
   return v;
 }
 
-__global__ void k_assemble_edge(Lvl<double> L, Wts<double> w, double mu, const double* ph, double2* K) {  // ph: the group's entry
-  const int Dc = 2 * L.n * L.m;
+// The lower triangles of every group of the launch (blockIdx.z).
+__global__ void k_assemble(Lvl<double> L, Wts<double> w, double mu, const double* ph, const int* gamma, int node,
+                           double2* K) {
+  const int n = (node ? 1 : 2) * L.n * L.m, g = blockIdx.z;
   const int row = blockIdx.x * blockDim.x + threadIdx.x, col = blockIdx.y;
-  if (row >= Dc || col >= Dc) return;
-  K[(long)col * Dc + row] = coarse_edge_entry(L, w, mu, load_ph<double>(ph, 0), row, col);
-}
-
-__global__ void k_assemble_node(Lvl<double> L, const double* ph, double shift, double2* K) {
-  const int Nc = L.n * L.m;
-  const int row = blockIdx.x * blockDim.x + threadIdx.x, col = blockIdx.y;
-  if (row >= Nc || col >= Nc) return;
-  K[(long)col * Nc + row] = coarse_node_entry(L, load_ph<double>(ph, 0), shift, row, col);
+  if (row >= n || col > row) return;
+  const Ph<double> p = load_ph<double>(ph, g);
+  const double shift = gamma[g] ? P_diag<double>(L) : 0.0;
+  K[((long)g * n + col) * n + row] =
+      node ? coarse_node_entry(L, p, shift, row, col) : coarse_edge_entry(L, w, mu, p, row, col);
 }
 
 // The phase and k = 0 tables of one group (three copies each), from kernel arguments: one
@@ -156,32 +155,19 @@ __global__ void k_set_phases(double* d_ph, int* d_gamma, int ngroups, int g, dou
   d_gamma[(long)rep * ngroups + g] = gamma;
 }
 
-// Small coarsest systems (n <= kSmallFactor, the usual 4 x 4 mesh has 32 edges and 16 nodes):
-// assembly and Cholesky factorisation of both matrices of blockIdx.y's group in one launch
-// (blockIdx.x: 0 edge, 1 node), the lower triangle in shared memory.  The chain of pivots is
-// what takes the time: a step is one reciprocal square root and two barriers, with no trip to
-// global memory.
-constexpr int kSmallFactor = 64;
-__global__ void __launch_bounds__(256) k_coarse_factors(Lvl<double> L, Wts<double> w, double mu, const double* ph,
-                                                        const int* gamma, double2* e64, float2* e32, double2* n64,
-                                                        float2* n32, int* info) {
-  extern __shared__ double2 Am[];  // entry (i, j), i >= j, at j (n + 1) + i
-  const int g = blockIdx.y, node = blockIdx.x, Nc = L.n * L.m, n = node ? Nc : 2 * Nc, ld = n + 1;
-  const int tid = threadIdx.x, nt = blockDim.x;
-  const Ph<double> p = load_ph<double>(ph, g);
-  const double shift = gamma[g] ? P_diag<double>(L) : 0.0;
+// Cholesky factor (lower) of the bs x bs matrix at Am (shared memory, entry (i, j), i >= j, at
+// j ld + i), in place, by the whole thread block.  Returns false from every thread when a pivot
+// is not positive.  A step is one reciprocal square root and two barriers.
+__device__ __forceinline__ bool chol_shared(double2* Am, int ld, int n) {
   __shared__ double piv[2];  // pivot and its reciprocal
-  for (int t = tid; t < n * n; t += nt) {
-    const int row = t % n, col = t / n;
-    if (row >= col)
-      Am[col * ld + row] = node ? coarse_node_entry(L, p, shift, row, col) : coarse_edge_entry(L, w, mu, p, row, col);
-  }
-  __syncthreads();
+  __shared__ int good;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (tid == 0) good = 1;
   for (int k = 0; k < n; ++k) {
     if (tid == 0) {
       const double d = Am[k * ld + k].x;
       const bool ok = d > 0.0 && isfinite(d);
-      if (!ok) info[node] = k + 1;
+      if (!ok) good = 0;
       const double r = ok ? sqrt(d) : 1.0;
       piv[0] = r;
       piv[1] = 1.0 / r;
@@ -189,8 +175,8 @@ __global__ void __launch_bounds__(256) k_coarse_factors(Lvl<double> L, Wts<doubl
     __syncthreads();
     const double inv = piv[1];
     const int rem = n - k - 1;
-    // the pivot column is scaled in place by the threads of its own entries, and every update
-    // below forms the two scaled entries it needs from the unscaled ones
+    // the pivot column is scaled by the threads of its own entries after the update, which
+    // forms the two scaled entries it needs from the unscaled ones
     for (int t = tid; t < rem * rem; t += nt) {
       const int jj = k + 1 + t / rem, ii = k + 1 + t % rem;
       if (ii < jj) continue;
@@ -205,6 +191,57 @@ __global__ void __launch_bounds__(256) k_coarse_factors(Lvl<double> L, Wts<doubl
     if (tid == 0) Am[k * ld + k] = make_double2(piv[0], 0.0);
   }
   __syncthreads();
+  return good != 0;
+}
+
+// Inverse of the lower triangular bs x bs block of Am that starts at (k0, k0), in place (shared
+// memory; bs <= kCoarseBlock): column c of the inverse by forward substitution, all columns at
+// once, a barrier per row.  The block's columns are rewritten behind the row front in X.
+__device__ __forceinline__ void invert_block(double2* Am, int ld, int k0, int bs) {
+  __shared__ double2 X[kCoarseBlock][kCoarseBlock + 1];  // X[row][col]
+  __shared__ double dinv[kCoarseBlock];
+  const int tid = threadIdx.x, nt = blockDim.x;
+  if (tid < bs) dinv[tid] = 1.0 / Am[(k0 + tid) * ld + k0 + tid].x;
+  for (int t = tid; t < bs * bs; t += nt) X[t / bs][t % bs] = make_double2(t / bs == t % bs ? 1.0 : 0.0, 0.0);
+  __syncthreads();
+  for (int r = 0; r < bs; ++r) {
+    // row r is complete but for its pivot: X[r] *= 1 / L_rr, then X[i] -= L_ir X[r] for i > r
+    for (int c = tid; c <= r; c += nt) X[r][c] = dinv[r] * X[r][c];
+    __syncthreads();
+    for (int t = tid; t < (bs - r - 1) * (r + 1); t += nt) {
+      const int i = r + 1 + t / (r + 1), c = t % (r + 1);
+      X[i][c] = X[i][c] - cmul(Am[(k0 + r) * ld + k0 + i], X[r][c]);
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < bs * bs; t += nt) {
+    const int i = t % bs, c = t / bs;
+    if (i >= c) Am[(k0 + c) * ld + k0 + i] = X[i][c];
+  }
+  __syncthreads();
+}
+
+// Small coarsest systems (n <= kSmallFactor, the usual 4 x 4 mesh has 32 edges and 16 nodes):
+// assembly and factorisation of both matrices of blockIdx.y's group in one launch (blockIdx.x:
+// 0 edge, 1 node), the lower triangle in shared memory: the chain of pivots is what takes the
+// time, and it makes no trip to global memory.
+constexpr int kSmallFactor = 64;
+__global__ void __launch_bounds__(256) k_coarse_factors(Lvl<double> L, Wts<double> w, double mu, const double* ph,
+                                                        const int* gamma, double2* e64, float2* e32, double2* n64,
+                                                        float2* n32, int* info) {
+  extern __shared__ double2 Am[];  // entry (i, j), i >= j, at j (n + 1) + i
+  const int g = blockIdx.y, node = blockIdx.x, Nc = L.n * L.m, n = node ? Nc : 2 * Nc, ld = n + 1;
+  const int tid = threadIdx.x, nt = blockDim.x;
+  const Ph<double> p = load_ph<double>(ph, g);
+  const double shift = gamma[g] ? P_diag<double>(L) : 0.0;
+  for (int t = tid; t < n * n; t += nt) {
+    const int row = t % n, col = t / n;
+    if (row >= col)
+      Am[col * ld + row] = node ? coarse_node_entry(L, p, shift, row, col) : coarse_edge_entry(L, w, mu, p, row, col);
+  }
+  __syncthreads();
+  if (!chol_shared(Am, ld, n) && tid == 0) info[node] = 1;
+  for (int k0 = 0; k0 < n; k0 += kCoarseBlock) invert_block(Am, ld, k0, min(kCoarseBlock, n - k0));
   double2* F = (node ? n64 : e64) + (long)g * n * n;
   float2* F32 = (node ? n32 : e32) + (long)g * n * n;
   for (int t = tid; t < n * n; t += nt) {
@@ -215,57 +252,96 @@ __global__ void __launch_bounds__(256) k_coarse_factors(Lvl<double> L, Wts<doubl
   }
 }
 
-// In-place Cholesky (lower, column-major) of a Hermitian positive definite matrix; one block.
-__global__ void k_cholesky(double2* A, int n, float2* A32, int* info) {
-  __shared__ double piv;
-  for (int k = 0; k < n; ++k) {
-    if (threadIdx.x == 0) {
-      const double d = A[(long)k * n + k].x;
-      piv = (d > 0.0 && isfinite(d)) ? sqrt(d) : -1.0;
-      if (piv < 0 && *info == 0) *info = k + 1;
-      A[(long)k * n + k] = make_double2(piv > 0 ? piv : 1.0, 0.0);
-    }
-    __syncthreads();
-    const double p = piv > 0 ? piv : 1.0;
-    for (int i = k + 1 + threadIdx.x; i < n; i += blockDim.x) {
-      double2 v = A[(long)k * n + i];
-      A[(long)k * n + i] = make_double2(v.x / p, v.y / p);
-    }
-    __syncthreads();
-    const int rem = n - k - 1;
-    for (long t = threadIdx.x; t < (long)rem * rem; t += blockDim.x) {
-      const int jj = k + 1 + int(t / rem), ii = k + 1 + int(t % rem);
-      if (ii < jj) continue;
-      const double2 lik = A[(long)k * n + ii], ljk = A[(long)k * n + jj];
-      double2 v = A[(long)jj * n + ii];
-      // A[ii][jj] -= L[ii][k] * conj(L[jj][k])
-      v.x -= lik.x * ljk.x + lik.y * ljk.y;
-      v.y -= lik.y * ljk.x - lik.x * ljk.y;
-      A[(long)jj * n + ii] = v;
-    }
-    __syncthreads();
+// Larger ones (odd factors left on the coarsest mesh: 13 x 9 cells have 234 edges): a right-looking
+// factorisation in blocks of 32 columns over many thread blocks and all groups (blockIdx.z or .y),
+// three launches per block: the diagonal block and its inverse, the panel below it, the trailing
+// matrix.  One thread block on the whole matrix took 3.6 ms at n = 234 (the FP64 rate of one SM).
+__global__ void __launch_bounds__(256) k_chol_diag(double2* A, float2* A32, int n, int k0, int* info) {
+  __shared__ double2 Am[kCoarseBlock * (kCoarseBlock + 1)];
+  constexpr int ld = kCoarseBlock + 1;
+  const int bs = min(kCoarseBlock, n - k0), tid = threadIdx.x, nt = blockDim.x;
+  A += (long)blockIdx.x * n * n;
+  A32 += (long)blockIdx.x * n * n;
+  for (int t = tid; t < bs * bs; t += nt) {
+    const int i = t % bs, j = t / bs;
+    if (i >= j) Am[j * ld + i] = A[(long)(k0 + j) * n + k0 + i];
   }
-  for (long t = threadIdx.x; t < (long)n * n; t += blockDim.x) {
-    const int jj = int(t / n), ii = int(t % n);
-    const double2 v = ii >= jj ? A[t] : make_double2(0.0, 0.0);
-    A[t] = v;
-    A32[t] = make_float2(float(v.x), float(v.y));
+  __syncthreads();
+  if (!chol_shared(Am, ld, bs) && tid == 0) *info = 1;
+  invert_block(Am, ld, 0, bs);
+  for (int t = tid; t < bs * bs; t += nt) {
+    const int i = t % bs, j = t / bs;
+    const double2 v = i >= j ? Am[j * ld + i] : make_double2(0.0, 0.0);
+    A[(long)(k0 + j) * n + k0 + i] = v;
+    A32[(long)(k0 + j) * n + k0 + i] = make_float2(float(v.x), float(v.y));
+  }
+}
+// rows i0 .. i0 + 31 below a full diagonal block: L(i, k) = sum_{c <= k} A(i, c) conj(Dinv(k, c))
+__global__ void __launch_bounds__(256) k_chol_panel(double2* A, float2* A32, int n, int k0) {
+  __shared__ double2 D[kCoarseBlock][kCoarseBlock + 1], P[kCoarseBlock][kCoarseBlock + 1];  // D[col][row], P[col][row]
+  const int i0 = k0 + kCoarseBlock * (1 + blockIdx.x), rows = min(kCoarseBlock, n - i0), tid = threadIdx.x;
+  A += (long)blockIdx.y * n * n;
+  A32 += (long)blockIdx.y * n * n;
+  for (int t = tid; t < kCoarseBlock * kCoarseBlock; t += blockDim.x) {
+    const int i = t % kCoarseBlock, c = t / kCoarseBlock;
+    D[c][i] = A[(long)(k0 + c) * n + k0 + i];
+    P[c][i] = i < rows ? A[(long)(k0 + c) * n + i0 + i] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  for (int t = tid; t < kCoarseBlock * kCoarseBlock; t += blockDim.x) {
+    const int i = t % kCoarseBlock, k = t / kCoarseBlock;
+    double2 v = make_double2(0.0, 0.0);
+    for (int c = 0; c <= k; ++c) v = v + cmulc(D[c][k], P[c][i]);
+    if (i < rows) {
+      A[(long)(k0 + k) * n + i0 + i] = v;
+      A32[(long)(k0 + k) * n + i0 + i] = make_float2(float(v.x), float(v.y));
+    }
+  }
+}
+// tile (blockIdx.x, blockIdx.y) of the trailing matrix, lower ones: A(i, j) -= sum_c L(i, c) conj(L(j, c))
+__global__ void __launch_bounds__(256) k_chol_trail(double2* A, int n, int k0) {
+  if (blockIdx.x < blockIdx.y) return;
+  __shared__ double2 I[kCoarseBlock][kCoarseBlock + 1], J[kCoarseBlock][kCoarseBlock + 1];  // [col][row]
+  const int i0 = k0 + kCoarseBlock * (1 + blockIdx.x), j0 = k0 + kCoarseBlock * (1 + blockIdx.y), tid = threadIdx.x;
+  A += (long)blockIdx.z * n * n;
+  for (int t = tid; t < kCoarseBlock * kCoarseBlock; t += blockDim.x) {
+    const int i = t % kCoarseBlock, c = t / kCoarseBlock;
+    I[c][i] = i0 + i < n ? A[(long)(k0 + c) * n + i0 + i] : make_double2(0.0, 0.0);
+    J[c][i] = j0 + i < n ? A[(long)(k0 + c) * n + j0 + i] : make_double2(0.0, 0.0);
+  }
+  __syncthreads();
+  for (int t = tid; t < kCoarseBlock * kCoarseBlock; t += blockDim.x) {
+    const int i = t % kCoarseBlock, j = t / kCoarseBlock;
+    if (i0 + i >= n || j0 + j > i0 + i) continue;
+    double2 v = A[(long)(j0 + j) * n + i0 + i];
+    for (int c = 0; c < kCoarseBlock; ++c) {
+      const double2 a = I[c][i], b = J[c][j];
+      v.x -= a.x * b.x + a.y * b.y;
+      v.y -= a.y * b.x - a.x * b.y;
+    }
+    A[(long)(j0 + j) * n + i0 + i] = v;
   }
 }
 
-// Solve L L^* x = b for each column (one warp per column).
+// Solve L L^* x = b for each column (one block per column; a hierarchy of one level).
+constexpr int kSolveThreads = 512;
 template <class T>
-__global__ void k_chol_solve(const cx<T>* __restrict__ Lbase, int n, const cx<T>* __restrict__ B, long ldb,
-                             cx<T>* __restrict__ X, long ldx, int ncols, int cpg, int ngroups, int goff) {
-  const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (warp >= ncols) return;
-  const cx<T>* Lf = Lbase + (long)((warp / cpg + goff) % ngroups) * n * n;
-  chol_solve_warp<T>(Lf, n, B + warp * ldb, X + warp * ldx, lane);
+__global__ void __launch_bounds__(kSolveThreads) k_chol_solve(const cx<T>* __restrict__ Lbase, int n,
+                                                              const cx<T>* __restrict__ B, long ldb,
+                                                              cx<T>* __restrict__ X, long ldx, int cpg, int ngroups,
+                                                              int goff) {
+  extern __shared__ float4 fine_sm[];
+  cx<T>* x = reinterpret_cast<cx<T>*>(fine_sm);
+  const int c = blockIdx.x;
+  for (int t = threadIdx.x; t < n; t += blockDim.x) x[t] = B[c * ldb + t];
+  __syncthreads();
+  coarse_solve<T>(Lbase + (long)((c / cpg + goff) % ngroups) * n * n, n, n, x, x, x + n);
+  for (int t = threadIdx.x; t < n; t += blockDim.x) X[c * ldx + t] = x[t];
 }
 
 // One colour of the node-patch block Gauss-Seidel sweep for A + mu M.
 template <class T>
-__global__ void k_edge_smooth(Lvl<T> L, Wts<T> w, const T* __restrict__ k3, T mu, const double* ph, int cpg,
+__global__ void k_edge_smooth(Lvl<T> L, Wts<T> w, const T* __restrict__ k3, PatchCoef<T> pc, const double* ph, int cpg,
                               cx<T>* X, const cx<T>* __restrict__ B, long ld, int ci, int cj) {
   const int i = 2 * (blockIdx.x * kBX + threadIdx.x) + ci, j = 2 * (blockIdx.y * kBY + threadIdx.y) + cj;
   const int c = blockIdx.z;
@@ -274,10 +350,10 @@ __global__ void k_edge_smooth(Lvl<T> L, Wts<T> w, const T* __restrict__ k3, T mu
   const ERd<T> r{X + c * ld, L.n, L.m, p};
   const ERd<T> rb{B + c * ld, L.n, L.m, p};
   if (inside(i, j, L.n, L.m, 1, 1))
-    edge_smooth_at<T>(L, inner<T>(w), k3, mu, p, inner_e<T>(X + c * ld, L.n, L.m), inner_e<T>(B + c * ld, L.n, L.m),
+    edge_smooth_at<T>(L, inner<T>(w), k3, pc, p, inner_e<T>(X + c * ld, L.n, L.m), inner_e<T>(B + c * ld, L.n, L.m),
                       X + c * ld, i, j);
   else
-    edge_smooth_at<T>(L, w, k3, mu, p, r, rb, X + c * ld, i, j);
+    edge_smooth_at<T>(L, w, k3, pc, p, r, rb, X + c * ld, i, j);
 }
 
 // One colour of point Gauss-Seidel for P = L^* M L.
@@ -292,258 +368,6 @@ __global__ void k_node_smooth(Lvl<T> L, const double* ph, int cpg, cx<T>* X, con
     node_smooth_at<T>(L, inner_n<T>(X + c * ld, L.n), X + c * ld, B + c * ld, i, j);
   else
     node_smooth_at<T>(L, r, X + c * ld, B + c * ld, i, j);
-}
-
-// ---- fused coarse-level V-cycles ---------------------------------------------
-// The levels from `top` down to the coarsest run as one kernel: one CTA per
-// column walks the rest of the V-cycle (zero, pre-smoothing by colour, residual
-// and restriction on the way down; the coarsest triangular solves; prolongation
-// and post-smoothing on the way up) with block-wide barriers between the steps.
-// Every point update is the function the one-launch-per-step kernels call, in
-// the same colour order, so the result is the one of the unfused V-cycle.
-// The level vectors live in shared memory for the whole cycle: x on every tail
-// level, b below the top one (the top right-hand side is read in place) and one
-// residual buffer of the top level's size; the top x is written out at the end.
-template <class T> struct TailLevel {
-  Lvl<T> L;
-  Wts<T> w;     // edge cycles only
-  const T* k3;  // edge cycles only
-  int sx, sb;   // shared-memory offsets (elements) of x and b; sb unused at the top
-};
-template <class T> struct TailArgs {
-  int nl;  // levels in the tail, the last one the coarsest
-  TailLevel<T> lev[kMaxLevels];
-  int sr;           // shared-memory offset of the residual buffer
-  int sf;           // shared-memory offset of the column's coarsest factor (leading dimension nfac + 1), or -1
-  const cx<T>* b0;  // top level right-hand sides and solutions, columns at stride ld0
-  cx<T>* x0;
-  long ld0, len0;   // len0: values per top-level column
-  const double* ph;
-  int cpg;
-  const cx<T>* factor;  // per-group coarsest Cholesky factors (nfac x nfac)
-  int nfac, ngroups, goff;
-  T mu;
-  int nu_pre, nu_post;
-};
-constexpr int kTailThreads = 512;
-constexpr long kTailMaxNodes = 4096;        // a level joins the tail when it has at most this many nodes
-constexpr int kTailSmemBytes = 200 * 1024;  // and the tail's shared-memory vectors fit in this
-
-template <class T> __device__ __forceinline__ const cx<T>* tail_b(const TailArgs<T>& a, cx<T>* sm, int l, int c) {
-  return l == 0 ? a.b0 + c * a.ld0 : sm + a.lev[l].sb;
-}
-
-// Copy of the column's coarsest factor into shared memory (the block's first barrier
-// orders it before the solve).
-template <class T> __device__ __forceinline__ void stage_factor(const TailArgs<T>& a, const cx<T>* F, cx<T>* sm) {
-  if (a.sf < 0) return;
-  const int n = a.nfac;
-  for (int t = threadIdx.x; t < n * n; t += blockDim.x) sm[a.sf + (t / n) * (n + 1) + t % n] = F[t];
-}
-
-// Range [lo, hi) of lattice steps a (point i0 + s a, 0 <= a < na) whose point lies in [ilo, ihi].
-__device__ __forceinline__ void lattice_range(int i0, int s, int na, int ilo, int ihi, int& lo, int& hi) {
-  lo = ilo <= i0 ? 0 : min(na, (ilo - i0 + s - 1) / s);
-  hi = ihi < i0 ? 0 : min(na, (ihi - i0) / s + 1);
-  hi = max(hi, lo);
-}
-
-// Calls f(i, j, inner) for every point (i0 + s a, j0 + s b), 0 <= a < na, 0 <= b < nb,
-// spread over the block's threads: first the points with i in [ilo, ihi] and j in
-// [jlo, jhi] (inner = true), then the frame around them, so that only the warp at
-// the seam mixes the two kinds.
-template <class F>
-__device__ __forceinline__ void for_lattice(int i0, int j0, int s, int na, int nb, int ilo, int ihi, int jlo, int jhi,
-                                            F&& f) {
-  int alo, ahi, blo, bhi;
-  lattice_range(i0, s, na, ilo, ihi, alo, ahi);
-  lattice_range(j0, s, nb, jlo, jhi, blo, bhi);
-  const int nai = ahi - alo, nbi = bhi - blo, nin = nai * nbi;
-  const int nrows = (nb - nbi) * na, total = na * nb;
-  for (int t = threadIdx.x; t < total; t += blockDim.x) {
-    int a, b;
-    if (t < nin) {
-      a = alo + t % nai;
-      b = blo + t / nai;
-    } else if (t - nin < nrows) {  // whole rows below and above the inner block
-      const int u = t - nin, r = u / na;
-      a = u % na;
-      b = r < blo ? r : bhi + (r - blo);
-    } else {  // the side pieces of the inner rows
-      const int u = t - nin - nrows, w = na - nai, k = u % w;
-      b = blo + u / w;
-      a = k < alo ? k : ahi + (k - alo);
-    }
-    f(i0 + s * a, j0 + s * b, t < nin);
-  }
-}
-
-template <class T>
-__global__ void __launch_bounds__(kTailThreads) k_node_tail(TailArgs<T> a) {
-  extern __shared__ float4 fine_sm[];
-  cx<T>* sm = reinterpret_cast<cx<T>*>(fine_sm);
-  const int c = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-  const Ph<T> p = load_ph<T>(a.ph, c / a.cpg);
-  const cx<T>* F = a.factor + (long)((c / a.cpg + a.goff) % a.ngroups) * a.nfac * a.nfac;
-  stage_factor<T>(a, F, sm);
-  // colour q of (0,0), (1,0), (0,1), (1,1); inner nodes have all neighbours on the level
-  auto sweep = [&](const Lvl<T>& L, cx<T>* x, const cx<T>* b, int q) {
-    const int ci = q & 1, cj = q >> 1;
-    const NRdPlain<T> rx{x, L.n, L.m, p};
-    for_lattice(ci, cj, 2, (L.n - ci + 1) / 2, (L.m - cj + 1) / 2, 1, L.n - 2, 1, L.m - 2, [&](int i, int j, bool in) {
-      if (in)
-        node_smooth_at<T>(L, inner_n<T>(x, L.n), x, b, i, j);
-      else
-        node_smooth_at<T>(L, rx, x, b, i, j);
-    });
-    __syncthreads();
-  };
-  cx<T>* r = sm + a.sr;
-  for (int l = 0; l < a.nl - 1; ++l) {
-    const Lvl<T> L = a.lev[l].L;
-    const int N = L.n * L.m;
-    cx<T>* x = sm + a.lev[l].sx;
-    const cx<T>* b = tail_b(a, sm, l, c);
-    for (int t = tid; t < N; t += nt) x[t] = czero<T>();
-    __syncthreads();
-    for (int it = 0; it < a.nu_pre; ++it)
-      for (int q = 0; q < 4; ++q) sweep(L, x, b, q);
-    const NRdPlain<T> rx{x, L.n, L.m, p};
-    for_lattice(0, 0, 1, L.n, L.m, 1, L.n - 2, 1, L.m - 2, [&](int i, int j, bool in) {
-      r[j * L.n + i] = in ? apply_nodal_at<T>(L, inner_n<T>(x, L.n), b, T(-1), T(1), i, j)
-                          : apply_nodal_at<T>(L, rx, b, T(-1), T(1), i, j);
-    });
-    __syncthreads();
-    // restriction at (I, J) reads fine nodes 2I-1 .. 2I+1
-    const Lvl<T> C = a.lev[l + 1].L;
-    cx<T>* bc = sm + a.lev[l + 1].sb;
-    const NRdPlain<T> rr{r, L.n, L.m, p};
-    for_lattice(0, 0, 1, C.n, C.m, 1, (L.n - 2) / 2, 1, (L.m - 2) / 2, [&](int I, int J, bool in) {
-      bc[J * C.n + I] = in ? restrict_node_at<T>(inner_n<T>(r, L.n), I, J) : restrict_node_at<T>(rr, I, J);
-    });
-    __syncthreads();
-  }
-  if (tid < 32) {
-    const int l = a.nl - 1;
-    if (a.sf >= 0)
-      chol_solve_warp_cols<T>(sm + a.sf, a.nfac + 1, a.nfac, tail_b(a, sm, l, c), sm + a.lev[l].sx, tid);
-    else
-      chol_solve_warp<T>(F, a.nfac, tail_b(a, sm, l, c), sm + a.lev[l].sx, tid);
-  }
-  __syncthreads();
-  for (int l = a.nl - 2; l >= 0; --l) {
-    const Lvl<T> L = a.lev[l].L, C = a.lev[l + 1].L;
-    cx<T>* x = sm + a.lev[l].sx;
-    const cx<T>* b = tail_b(a, sm, l, c);
-    const cx<T>* xc = sm + a.lev[l + 1].sx;
-    const NRdPlain<T> rc{xc, C.n, C.m, p};
-    // prolongation at fine (i, j) reads coarse nodes i/2 .. i/2 + 1
-    for_lattice(0, 0, 1, L.n, L.m, 0, 2 * C.n - 3, 0, 2 * C.m - 3, [&](int i, int j, bool in) {
-      const int e = j * L.n + i;
-      x[e] = x[e] + (in ? prolong_node_at<T>(inner_n<T>(xc, C.n), i, j) : prolong_node_at<T>(rc, i, j));
-    });
-    __syncthreads();
-    for (int it = 0; it < a.nu_post; ++it)
-      for (int q = 3; q >= 0; --q) sweep(L, x, b, q);
-  }
-  const cx<T>* x = sm + a.lev[0].sx;
-  for (long t = tid; t < a.len0; t += nt) a.x0[c * a.ld0 + t] = x[t];
-}
-
-template <class T>
-__global__ void __launch_bounds__(kTailThreads) k_edge_tail(TailArgs<T> a) {
-  extern __shared__ float4 fine_sm[];
-  cx<T>* sm = reinterpret_cast<cx<T>*>(fine_sm);
-  const int c = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-  const Ph<T> p = load_ph<T>(a.ph, c / a.cpg);
-  const cx<T>* F = a.factor + (long)((c / a.cpg + a.goff) % a.ngroups) * a.nfac * a.nfac;
-  stage_factor<T>(a, F, sm);
-  // colour q of (0,0), (1,0), (0,1), (1,1); inner patches have all their edges and cells on the level
-  auto sweep = [&](const TailLevel<T>& TL, cx<T>* x, const cx<T>* b, int q) {
-    const Lvl<T>& L = TL.L;
-    const int ci = q & 1, cj = q >> 1;
-    const ERdPlain<T> rx{x, L.n, L.m, p};
-    const ERdPlain<T> rb{b, L.n, L.m, p};
-    for_lattice(ci, cj, 2, (L.n - ci + 1) / 2, (L.m - cj + 1) / 2, 1, L.n - 2, 1, L.m - 2, [&](int i, int j, bool in) {
-      if (in)
-        edge_smooth_at<T>(L, inner<T>(TL.w), TL.k3, a.mu, p, inner_e<T>(x, L.n, L.m), inner_e<T>(b, L.n, L.m), x, i,
-                          j);
-      else
-        edge_smooth_at<T>(L, TL.w, TL.k3, a.mu, p, rx, rb, x, i, j);
-    });
-    __syncthreads();
-  };
-  cx<T>* r = sm + a.sr;
-  for (int l = 0; l < a.nl - 1; ++l) {
-    const TailLevel<T> TL = a.lev[l];
-    const Lvl<T> L = TL.L;
-    const int N = L.n * L.m;
-    cx<T>* x = sm + TL.sx;
-    const cx<T>* b = tail_b(a, sm, l, c);
-    for (int t = tid; t < 2 * N; t += nt) x[t] = czero<T>();
-    __syncthreads();
-    for (int it = 0; it < a.nu_pre; ++it)
-      for (int q = 0; q < 4; ++q) sweep(TL, x, b, q);
-    const ERdPlain<T> rx{x, L.n, L.m, p};
-    for_lattice(0, 0, 1, L.n, L.m, 1, L.n - 2, 1, L.m - 2, [&](int i, int j, bool in) {
-      cx<T> yx, yy;
-      if (in)
-        apply_edge_at<T>(L, inner<T>(TL.w), inner_e<T>(x, L.n, L.m), b, T(-1), -a.mu, T(1), i, j, yx, yy);
-      else
-        apply_edge_at<T>(L, TL.w, rx, b, T(-1), -a.mu, T(1), i, j, yx, yy);
-      r[j * L.n + i] = yx;
-      r[N + j * L.n + i] = yy;
-    });
-    __syncthreads();
-    // restriction at (I, J) reads fine edges with indices 2I-1 .. 2I+1
-    const Lvl<T> C = a.lev[l + 1].L;
-    const int Nc = C.n * C.m;
-    cx<T>* bc = sm + a.lev[l + 1].sb;
-    const ERdPlain<T> rr{r, L.n, L.m, p};
-    for_lattice(0, 0, 1, C.n, C.m, 1, (L.n - 2) / 2, 1, (L.m - 2) / 2, [&](int I, int J, bool in) {
-      cx<T> vx, vy;
-      if (in)
-        restrict_edge_at<T>(inner_e<T>(r, L.n, L.m), I, J, vx, vy);
-      else
-        restrict_edge_at<T>(rr, I, J, vx, vy);
-      bc[J * C.n + I] = vx;
-      bc[Nc + J * C.n + I] = vy;
-    });
-    __syncthreads();
-  }
-  if (tid < 32) {
-    const int l = a.nl - 1;
-    if (a.sf >= 0)
-      chol_solve_warp_cols<T>(sm + a.sf, a.nfac + 1, a.nfac, tail_b(a, sm, l, c), sm + a.lev[l].sx, tid);
-    else
-      chol_solve_warp<T>(F, a.nfac, tail_b(a, sm, l, c), sm + a.lev[l].sx, tid);
-  }
-  __syncthreads();
-  for (int l = a.nl - 2; l >= 0; --l) {
-    const TailLevel<T> TL = a.lev[l];
-    const Lvl<T> L = TL.L, C = a.lev[l + 1].L;
-    const int N = L.n * L.m;
-    cx<T>* x = sm + TL.sx;
-    const cx<T>* b = tail_b(a, sm, l, c);
-    const cx<T>* xc = sm + a.lev[l + 1].sx;
-    const ERdPlain<T> rc{xc, C.n, C.m, p};
-    // prolongation at fine (i, j) reads coarse edges with indices i/2 .. i/2 + 1
-    for_lattice(0, 0, 1, L.n, L.m, 0, 2 * C.n - 3, 0, 2 * C.m - 3, [&](int i, int j, bool in) {
-      cx<T> vx, vy;
-      if (in)
-        prolong_edge_at<T>(inner_e<T>(xc, C.n, C.m), i, j, vx, vy);
-      else
-        prolong_edge_at<T>(rc, i, j, vx, vy);
-      const int e = j * L.n + i;
-      x[e] = x[e] + vx;
-      x[N + e] = x[N + e] + vy;
-    });
-    __syncthreads();
-    for (int it = 0; it < a.nu_post; ++it)
-      for (int q = 3; q >= 0; --q) sweep(TL, x, b, q);
-  }
-  const cx<T>* x = sm + a.lev[0].sx;
-  for (long t = tid; t < a.len0; t += nt) a.x0[c * a.ld0 + t] = x[t];
 }
 
 template <class T> const cx<T>* edge_factor(const KData& K);
@@ -714,20 +538,23 @@ void factor_groups(const Hierarchy& H, KData& K, int g0, int ng, cudaStream_t s)
     PBS_LAUNCHED();
     return;
   }
-  for (int g = g0; g < g0 + ng; ++g) {
-    double2* e64 = K.edge64 + g * Dc * Dc;
-    double2* n64 = K.node64 + g * Nc * Nc;
-    const double* gph = K.d_ph + 4L * g;
-    k_assemble_edge<<<dim3(((unsigned)Dc + 127) / 128, (unsigned)Dc), 128, 0, s>>>(C.lvl<double>(), C.wts<double>(),
-                                                                                   H.mu, gph, e64);
+  for (int node = 0; node < 2; ++node) {
+    const int n = node ? K.Nc : K.Dc;
+    double2* F = (node ? K.node64 : K.edge64) + (size_t)g0 * n * n;
+    float2* F32 = (node ? K.node32 : K.edge32) + (size_t)g0 * n * n;
+    k_assemble<<<dim3((n + 127) / 128, n, ng), 128, 0, s>>>(C.lvl<double>(), C.wts<double>(), H.mu, K.d_ph + 4L * g0,
+                                                            K.d_gamma + g0, node, F);
     PBS_LAUNCHED();
-    k_cholesky<<<1, 256, 0, s>>>(e64, K.Dc, K.edge32 + g * Dc * Dc, K.d_info);
-    PBS_LAUNCHED();
-    const double shift = K.gamma[g] ? P_diag<double>(C.lvl<double>()) : 0.0;
-    k_assemble_node<<<dim3(((unsigned)Nc + 127) / 128, (unsigned)Nc), 128, 0, s>>>(C.lvl<double>(), gph, shift, n64);
-    PBS_LAUNCHED();
-    k_cholesky<<<1, 256, 0, s>>>(n64, K.Nc, K.node32 + g * Nc * Nc, K.d_info + 1);
-    PBS_LAUNCHED();
+    for (int k0 = 0; k0 < n; k0 += kCoarseBlock) {
+      k_chol_diag<<<ng, 256, 0, s>>>(F, F32, n, k0, K.d_info + node);
+      PBS_LAUNCHED();
+      const int tiles = (n - k0 - 1) / kCoarseBlock;  // row tiles below the block
+      if (tiles == 0) break;
+      k_chol_panel<<<dim3(tiles, ng), 256, 0, s>>>(F, F32, n, k0);
+      PBS_LAUNCHED();
+      k_chol_trail<<<dim3(tiles, tiles, ng), 256, 0, s>>>(F, n, k0);
+      PBS_LAUNCHED();
+    }
   }
 }
 
@@ -894,27 +721,116 @@ template <class T> void zero_columns(cx<T>* x, long ld, long len, int ncols, cud
   }
 }
 
-// Shared-memory elements of a fused tail from level l: x on every level, b below
-// the top one and a residual buffer of the top level's size.
-inline long tail_smem_elems(const Hierarchy& H, int l, bool nodal) {
-  auto len = [&](int k) { return nodal ? H.lev[k].N() : H.lev[k].D(); };
-  long e = 2 * len(l);
-  for (int k = l + 1; k < H.nlev; ++k) e += 2 * len(k);
-  return e;
+// ---- fused coarse levels (tail.cuh) ----
+// The tail covers level l and everything below when l is not the coarsest, has at most
+// kTailMaxNodes nodes and its vectors fit in one CTA's shared memory.
+//
+// Layout of a tail from level l with K CTAs (the same offsets in every CTA): level vectors, the
+// residuals, the coarsest factor where it fits.  Level l + t is spread over the cluster while its
+// block rows divide by K and every CTA keeps kTailMinUnits units; the levels below run on the
+// first CTA.  Returns the shared-memory bytes, or 0 where K does not fit the mesh.
+constexpr int kTailMinUnits = 128;  // four warps: one per quarter of the SM
+template <class T> size_t tail_layout(const Hierarchy& H, int l, bool nodal, int K, TailArgs<T>& a) {
+  a.nl = H.nlev - l;
+  a.lc = 0;
+  a.K = K;
+  if (a.nl > kTailMaxLevels) return 0;
+  const int fields = nodal ? 1 : 2;
+  int off = 0;
+  bool spread = K > 1;
+  for (int t = 0; t < a.nl; ++t) {
+    const Level& L = H.lev[l + t];
+    TailLevel<T>& v = a.lev[t];
+    v.L = L.lvl<T>();
+    if (t == a.nl - 1) {  // plain vectors
+      v.H = v.V = v.Vb = 0;
+      const int len = (int)(nodal ? L.N() : L.D());
+      v.sx = off;
+      v.sb = off + len;
+      off += 2 * len;
+      break;
+    }
+    v.H = L.n / 2;
+    v.V = v.Vb = L.m / 2;
+    spread = spread && v.V % K == 0 && 2 * v.H * v.V / K >= kTailMinUnits;
+    if (spread) {
+      v.Vb = v.V / K;
+      a.lc = t + 1;
+    }
+    const int len = fields * 4 * tail_plane(v.H, v.Vb);
+    v.sx = off;
+    off += len;
+    if (t > 0) {
+      v.sb = off;
+      off += len;
+    }
+    if (t == 0) a.sr = off;  // the top residual's own place
+    if (t == 1) a.sr1 = off;
+    if (t <= 1) off += len;
+  }
+  if (K > 1 && a.lc == 0) return 0;
+  const Level& C = H.lev[H.nlev - 1];
+  a.nfac = (int)(nodal ? C.N() : C.D());
+  a.sw = off;
+  off += a.nfac;
+  a.sf = -1;
+  if ((off + (long)a.nfac * (a.nfac + 1)) * (long)sizeof(cx<T>) <= kTailSmemBytes) {
+    a.sf = off;
+    off += a.nfac * (a.nfac + 1);
+  }
+  return (size_t)off * sizeof(cx<T>);
 }
 
-// The fused tail covers level l and everything below when l is not the coarsest,
-// has at most kTailMaxNodes nodes and its vectors fit in shared memory.
-template <class T> bool tail_from(const Hierarchy& H, int l, bool nodal) {
-  return l < H.nlev - 1 && H.lev[l].N() <= kTailMaxNodes &&
-         tail_smem_elems(H, l, nodal) * (long)sizeof(cx<T>) <= kTailSmemBytes;
+template <class T> bool tail_fits(const Hierarchy& H, int l, bool nodal, int K, TailArgs<T>& a, size_t* smem) {
+  *smem = tail_layout<T>(H, l, nodal, K, a);
+  return *smem > 0 && *smem <= (size_t)kTailSmemBytes;
 }
-template <class T> void set_tail_smem() {
+template <class T> bool tail_from(const Hierarchy& H, int l, bool nodal) {
+  if (l >= H.nlev - 1 || H.lev[l].N() > kTailMaxNodes) return false;
+  TailArgs<T> a{};
+  size_t smem = 0;
+  return tail_fits<T>(H, l, nodal, 1, a, &smem);
+}
+// CTAs per column.  Binary64 levels are bound by the FP64 rate of the SMs they run on: up to four
+// while every CTA still has an SM of its own (32 x 32, 20 columns: nodal 118 -> 77 us with four,
+// edges 297 -> 191 us; 80 columns: 119 -> 232 us).  Binary32 levels are bound by latency, and a
+// cluster barrier costs more than the split saves (64 x 64: nodal 63 -> 60 us with four CTAs,
+// 32 x 32: 32 -> 46 us).
+template <class T> int tail_want(int ncols) {
+  if (sizeof(T) == 8) return ncols <= 38 ? 4 : ncols <= 76 ? 2 : 1;
+  return 1;
+}
+
+// Threads per CTA: every warp takes part in every barrier, and on the smaller levels most of them
+// have nothing else to do (64 x 64, binary32 nodal: 88 us with 256 threads, 63 with 512; 32 x 32:
+// 38 and 32 us; binary64 on four CTAs, 128 units each: 77 us with 128 threads, 81 with 512).
+template <class T> int tail_threads(const TailArgs<T>& a) {
+  const int units = 2 * a.lev[0].H * a.lev[0].Vb;
+  return units >= 512 ? 512 : units > 128 ? 256 : 128;
+}
+
+template <class T, bool CL> void launch_tail(const TailArgs<T>& a, bool nodal, int ncols, size_t smem,
+                                                     cudaStream_t s) {
   static PerDeviceOnce once;
   once([] {
-    PBS_CUDA(cudaFuncSetAttribute(k_node_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmemBytes));
-    PBS_CUDA(cudaFuncSetAttribute(k_edge_tail<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, kTailSmemBytes));
+    PBS_CUDA(cudaFuncSetAttribute(k_node_tail<T, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kTailSmemBytes));
+    PBS_CUDA(cudaFuncSetAttribute(k_edge_tail<T, CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  kTailSmemBytes));
   });
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(ncols * a.K);
+  cfg.blockDim = dim3(tail_threads<T>(a));
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = a.K;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = CL ? 1 : 0;
+  PBS_CUDA(cudaLaunchKernelEx(&cfg, nodal ? k_node_tail<T, CL> : k_edge_tail<T, CL>, a));
 }
 
 // Algorithmic bytes of a fused tail: the top right-hand sides in and solutions
@@ -1070,51 +986,39 @@ void launch_rb(bool down, const FineShape& f, const Level& L, const Level& C, co
   }
 }
 
+// The coarse levels from l down in one launch.
 template <class T>
-TailArgs<T> tail_args(const Hierarchy& H, const KData& K, int l, const cx<T>* b, cx<T>* x, long ld, int cpg,
-                      int nu_pre, int nu_post, bool nodal, size_t* smem) {
+void run_tail(const Hierarchy& H, const KData& K, int l, const cx<T>* b, cx<T>* x, long ld, int ncols, int cpg,
+              int nu_pre, int nu_post, bool nodal, cudaStream_t s) {
   TailArgs<T> a{};
-  a.nl = H.nlev - l;
-  int off = 0;
-  for (int k = 0; k < a.nl; ++k) {
-    const Level& L = H.lev[l + k];
-    const int len = (int)(nodal ? L.N() : L.D());
-    TailLevel<T>& t = a.lev[k];
-    t.L = L.lvl<T>();
-    t.w = L.wts<T>();
-    t.k3 = k3_of<T>(L);
-    t.sx = off;
-    off += len;
-    if (k > 0) {
-      t.sb = off;
-      off += len;
-    }
+  size_t smem = 0;
+  int k = tail_want<T>(ncols);
+  while (k > 1 && !tail_fits<T>(H, l, nodal, k, a, &smem)) k /= 2;
+  if (!tail_fits<T>(H, l, nodal, k, a, &smem)) fail(-1, "coarse levels: no layout fits");
+  for (int t = 0; t < a.nl; ++t) {
+    const Level& L = H.lev[l + t];
+    const Wts<T> w = L.wts<T>();
+    a.lev[t].winv = w.winv;
+    a.lev[t].wscale = w.scale;
+    a.lev[t].k3 = k3_of<T>(L);
+    a.lev[t].pc = patch_coef<T>(a.lev[t].L, H.mu);
   }
-  a.len0 = nodal ? H.lev[l].N() : H.lev[l].D();
-  a.sr = off;
-  off += (int)a.len0;
-  const Level& Cst0 = H.lev[H.nlev - 1];
-  const long nf = nodal ? Cst0.N() : Cst0.D();
-  a.sf = -1;
-  if ((off + nf * (nf + 1)) * (long)sizeof(cx<T>) <= kTailSmemBytes) {
-    a.sf = off;
-    off += (int)(nf * (nf + 1));
-  }
-  *smem = (size_t)off * sizeof(cx<T>);
   a.b0 = b;
   a.x0 = x;
   a.ld0 = ld;
   a.ph = K.d_ph;
   a.cpg = cpg;
-  const Level& Cst = H.lev[H.nlev - 1];
   a.factor = nodal ? node_factor<T>(K) : edge_factor<T>(K);
-  a.nfac = (int)(nodal ? Cst.N() : Cst.D());
   a.ngroups = K.ngroups;
   a.goff = K.goff;
-  a.mu = T(H.mu);
   a.nu_pre = nu_pre;
   a.nu_post = nu_post;
-  return a;
+  const int cls = nodal ? KC_NODE_TAIL : KC_EDGE_TAIL;
+  timer_begin(cls, s, tail_bytes<T>(H, l, ncols, cpg, nodal));
+  if (k > 1) launch_tail<T, true>(a, nodal, ncols, smem, s);
+  else launch_tail<T, false>(a, nodal, ncols, smem, s);
+  timer_end(cls, s);
+  PBS_LAUNCHED();
 }
 
 template <class T>
@@ -1122,29 +1026,24 @@ void edge_cycle(const Hierarchy& H, const KData& K, MgWork<T>& w, int l, const c
                 int cpg, int nu_pre, int nu_post, cudaStream_t s) {
   const Level& L = H.lev[l];
   if (l == H.nlev - 1) {
-    k_chol_solve<T><<<(ncols * 32 + 127) / 128, 128, 0, s>>>(edge_factor<T>(K), (int)L.D(), b, ld, x, ld, ncols, cpg,
-                                                             K.ngroups, K.goff);
+    k_chol_solve<T><<<ncols, kSolveThreads, 2 * (size_t)L.D() * sizeof(cx<T>), s>>>(edge_factor<T>(K), (int)L.D(), b, ld, x, ld,
+                                                                                cpg, K.ngroups, K.goff);
     PBS_LAUNCHED();
     return;
   }
   if (tail_from<T>(H, l, false)) {
-    size_t smem = 0;
-    const TailArgs<T> ta = tail_args<T>(H, K, l, b, x, ld, cpg, nu_pre, nu_post, false, &smem);
-    set_tail_smem<T>();
-    timer_begin(KC_EDGE_TAIL, s, tail_bytes<T>(H, l, ncols, cpg, false));
-    k_edge_tail<T><<<ncols, kTailThreads, smem, s>>>(ta);
-    timer_end(KC_EDGE_TAIL, s);
-    PBS_LAUNCHED();
+    run_tail<T>(H, K, l, b, x, ld, ncols, cpg, nu_pre, nu_post, false, s);
     return;
   }
   zero_columns<T>(x, ld, L.D(), ncols, s);
   const Lvl<T> lv = L.lvl<T>();
   const Wts<T> wt = L.wts<T>();
   const T mu = T(H.mu);
+  const PatchCoef<T> pc = patch_coef<T>(lv, H.mu);
   for (int it = 0; it < nu_pre; ++it)
     for (int q = 0; q < 4; ++q) {
       timer_begin(KC_EDGE_SMOOTH, s, smooth_bytes<T>(L, ncols));
-      k_edge_smooth<T><<<half_grid(L.n, L.m, ncols), dim3(kBX, kBY), 0, s>>>(lv, wt, k3_of<T>(L), mu, K.d_ph, cpg, x,
+      k_edge_smooth<T><<<half_grid(L.n, L.m, ncols), dim3(kBX, kBY), 0, s>>>(lv, wt, k3_of<T>(L), pc, K.d_ph, cpg, x,
                                                                              b, ld, kColours[q][0], kColours[q][1]);
       timer_end(KC_EDGE_SMOOTH, s);
       PBS_LAUNCHED();
@@ -1158,7 +1057,7 @@ void edge_cycle(const Hierarchy& H, const KData& K, MgWork<T>& w, int l, const c
   for (int it = 0; it < nu_post; ++it)
     for (int q = 3; q >= 0; --q) {
       timer_begin(KC_EDGE_SMOOTH, s, smooth_bytes<T>(L, ncols));
-      k_edge_smooth<T><<<half_grid(L.n, L.m, ncols), dim3(kBX, kBY), 0, s>>>(lv, wt, k3_of<T>(L), mu, K.d_ph, cpg, x,
+      k_edge_smooth<T><<<half_grid(L.n, L.m, ncols), dim3(kBX, kBY), 0, s>>>(lv, wt, k3_of<T>(L), pc, K.d_ph, cpg, x,
                                                                              b, ld, kColours[q][0], kColours[q][1]);
       timer_end(KC_EDGE_SMOOTH, s);
       PBS_LAUNCHED();
@@ -1177,19 +1076,13 @@ void node_cycle(const Hierarchy& H, const KData& K, MgWork<T>& w, int l, const c
   const Level& L = H.lev[l];
   if (x0 && !takes_guess<T>(H, l, nu_pre, nu_post)) fail(-1, "nodal cycle: initial iterate on an untiled level");
   if (l == H.nlev - 1) {
-    k_chol_solve<T><<<(ncols * 32 + 127) / 128, 128, 0, s>>>(node_factor<T>(K), (int)L.N(), b, ld, x, ld, ncols, cpg,
-                                                             K.ngroups, K.goff);
+    k_chol_solve<T><<<ncols, kSolveThreads, 2 * (size_t)L.N() * sizeof(cx<T>), s>>>(node_factor<T>(K), (int)L.N(), b, ld, x, ld,
+                                                                                cpg, K.ngroups, K.goff);
     PBS_LAUNCHED();
     return;
   }
   if (tail_from<T>(H, l, true)) {
-    size_t smem = 0;
-    const TailArgs<T> ta = tail_args<T>(H, K, l, b, x, ld, cpg, nu_pre, nu_post, true, &smem);
-    set_tail_smem<T>();
-    timer_begin(KC_NODE_TAIL, s, tail_bytes<T>(H, l, ncols, cpg, true));
-    k_node_tail<T><<<ncols, kTailThreads, smem, s>>>(ta);
-    timer_end(KC_NODE_TAIL, s);
-    PBS_LAUNCHED();
+    run_tail<T>(H, K, l, b, x, ld, ncols, cpg, nu_pre, nu_post, true, s);
     return;
   }
   if (fine_tiled(L, nu_pre, nu_post)) {

@@ -1,6 +1,5 @@
 // Per-point bodies of the multigrid steps (Section 5): point and patch
-// Gauss-Seidel updates, level residuals, grid transfers and the coarsest
-// triangular solves.  The one-launch-per-step kernels (ops.cu, mg.cu) and the
+// Gauss-Seidel updates, level residuals and grid transfers.  The one-launch-per-step kernels (ops.cu, mg.cu) and the
 // fused coarse-level V-cycle kernels (mg.cu) call the same functions, so both
 // schedules perform the same arithmetic on every point.
 //
@@ -91,7 +90,7 @@ template <class T, class R>
 __device__ __forceinline__ void node_smooth_at(const Lvl<T>& L, const R& r, cx<T>* x, const cx<T>* b, int i, int j) {
   const long e = (long)j * L.n + i;
   const cx<T> res = b[e] - P_at<T>(r, L, i, j);
-  x[e] = x[e] + (T(1) / P_diag<T>(L)) * res;
+  x[e] = x[e] + L.pinv * res;
 }
 
 // sP (P x)(i,j) + sB b(i,j)
@@ -149,35 +148,62 @@ __device__ __forceinline__ void apply_edge_at(const Lvl<T>& L, const W& w, const
   }
 }
 
+// Constants of the patch smoother on one level, formed on the host.
+template <class T> struct PatchCoef {
+  T m1, m2;  // 2/3 mx, 2/3 my: the mass matrix's diagonal
+  T ux, uy;  // mu mx / 6, mu my / 6
+  T cs;      // 1 / (mu g^T M_loc g), g the gradient of the node's hat function
+};
+template <class T> inline PatchCoef<T> patch_coef(const Lvl<T>& L, double mu) {
+  const double m1 = 2.0 / 3.0 * (double)L.mx, m2 = 2.0 / 3.0 * (double)L.my;
+  return PatchCoef<T>{T(m1), T(m2), T(mu * (double)L.mx / 6.0), T(mu * (double)L.my / 6.0), T(1.0 / (2.0 * mu * (m1 + m2)))};
+}
+
+// Changes of the edges L, R, B, T of a node's patch from the patch residual r* and the stored
+// K3^{-1} = (k00, k01, k02, k11, k12, k22); V is a real component or a complex value.
+template <class T, class V>
+__device__ __forceinline__ void patch_solve(const PatchCoef<T>& c, const T k00, const T k01, const T k02, const T k11,
+                                            const T k12, const T k22, V rL, V rR, V rB, V rT, V& dL, V& dR, V& dB,
+                                            V& dT) {
+  const V du = rL - rR, dv = rT - rB, s0 = c.cs * (du - dv);
+  const V ya = rL + rR, yb = rB + rT, yc = c.m2 * du + c.m1 * dv;
+  const V za = k00 * ya + k01 * yb + k02 * yc, zb = k01 * ya + k11 * yb + k12 * yc, zc = k02 * ya + k12 * yb + k22 * yc;
+  const V tx = s0 + c.m2 * zc, ty = s0 - c.m1 * zc;
+  dL = za + tx;
+  dR = za - tx;
+  dB = zb + ty;
+  dT = zb - ty;
+}
+
 // Block Gauss-Seidel update of the patch of node (i,j) (its edges L, R, B, T);
-// r reads x, rb reads b; K3^{-1} of the node in k3 (SoA [6][N]).
+// r reads x, rb reads b; K3^{-1} of the node in k3 (SoA [6][N]).  The residual
+// b - (A + mu M) x on the four edges shares the curls of the four cells around the node.
 template <class T, class R, class RB, class W>
-__device__ __forceinline__ void edge_smooth_at(const Lvl<T>& L, const W& w, const T* k3, T mu, const Ph<T>& p,
-                                               const R& r, const RB& rb, cx<T>* X, int i, int j) {
-  // residual b - (A + mu M) x on the patch, in ghost coordinates
-  const cx<T> rL = rb.x(i - 1, j) - (A_x<T>(r, w, i - 1, j) + mu * M_x<T>(r, L, i - 1, j));
-  const cx<T> rR = rb.x(i, j) - (A_x<T>(r, w, i, j) + mu * M_x<T>(r, L, i, j));
-  const cx<T> rB = rb.y(i, j - 1) - (A_y<T>(r, w, i, j - 1) + mu * M_y<T>(r, L, i, j - 1));
-  const cx<T> rT = rb.y(i, j) - (A_y<T>(r, w, i, j) + mu * M_y<T>(r, L, i, j));
-  const T m1 = T(2.0 / 3.0) * L.mx, m2 = T(2.0 / 3.0) * L.my;
-  const cx<T> s0 = (T(1) / (mu * T(2) * (m1 + m2))) * (rL - rR + rB - rT);
-  const cx<T> ya = rL + rR, yb = rB + rT, yc = m2 * (rL - rR) + m1 * (rT - rB);
+__device__ __forceinline__ void edge_smooth_at(const Lvl<T>& L, const W& w, const T* k3, const PatchCoef<T>& pc,
+                                               const Ph<T>& p, const R& r, const RB& rb, cx<T>* X, int i, int j) {
+  // ghost coordinates
+  const cx<T> xL = r.x(i - 1, j), xR = r.x(i, j), xLu = r.x(i - 1, j + 1), xRu = r.x(i, j + 1),
+              xLd = r.x(i - 1, j - 1), xRd = r.x(i, j - 1);
+  const cx<T> yB = r.y(i, j - 1), yT = r.y(i, j), yBl = r.y(i - 1, j - 1), yTl = r.y(i - 1, j),
+              yBr = r.y(i + 1, j - 1), yTr = r.y(i + 1, j);
+  const cx<T> hNE = w(i, j) * ((xRu - xR) - (yTr - yT)), hNW = w(i - 1, j) * ((xLu - xL) - (yT - yTl));
+  const cx<T> hSE = w(i, j - 1) * ((xR - xRd) - (yBr - yB)), hSW = w(i - 1, j - 1) * ((xL - xLd) - (yB - yBl));
+  const cx<T> rL = rb.x(i - 1, j) - ((hSW - hNW) + pc.ux * (T(4) * xL + (xLu + xLd)));
+  const cx<T> rR = rb.x(i, j) - ((hSE - hNE) + pc.ux * (T(4) * xR + (xRu + xRd)));
+  const cx<T> rB = rb.y(i, j - 1) - ((hSE - hSW) + pc.uy * (T(4) * yB + (yBr + yBl)));
+  const cx<T> rT = rb.y(i, j) - ((hNE - hNW) + pc.uy * (T(4) * yT + (yTr + yTl)));
   const long N = (long)L.n * L.m, e = (long)j * L.n + i;
-  const T K00 = k3[e], K01 = k3[N + e], K02 = k3[2 * N + e], K11 = k3[3 * N + e], K12 = k3[4 * N + e],
-          K22 = k3[5 * N + e];
-  const cx<T> za = K00 * ya + K01 * yb + K02 * yc;
-  const cx<T> zb = K01 * ya + K11 * yb + K12 * yc;
-  const cx<T> zc = K02 * ya + K12 * yb + K22 * yc;
-  const cx<T> dL = s0 + za + m2 * zc, dR = za - m2 * zc - s0;
-  const cx<T> dB = s0 + zb - m1 * zc, dT = zb + m1 * zc - s0;
+  cx<T> dL, dR, dB, dT;
+  patch_solve<T>(pc, k3[e], k3[N + e], k3[2 * N + e], k3[3 * N + e], k3[4 * N + e], k3[5 * N + e], rL, rR, rB, rT, dL,
+                 dR, dB, dT);
   cx<T>* Xx = X;
   cx<T>* Xy = X + N;
-  Xx[e] = Xx[e] + dR;
-  Xy[e] = Xy[e] + dT;
+  Xx[e] = xR + dR;
+  Xy[e] = yT + dT;
   // a ghost-coordinate change d of an edge read as conj(alpha) x is alpha d in storage
-  if (i > 0) Xx[e - 1] = Xx[e - 1] + dL;
+  if (i > 0) Xx[e - 1] = xL + dL;
   else Xx[(long)j * L.n + L.n - 1] = Xx[(long)j * L.n + L.n - 1] + cmul(p.al, dL);
-  if (j > 0) Xy[e - L.n] = Xy[e - L.n] + dB;
+  if (j > 0) Xy[e - L.n] = yB + dB;
   else Xy[(long)(L.m - 1) * L.n + i] = Xy[(long)(L.m - 1) * L.n + i] + cmul(p.be, dB);
 }
 
@@ -206,76 +232,6 @@ __device__ __forceinline__ void restrict_edge_at(const R& rf, int I, int J, cx<T
        T(0.25) * (rf.x(i, j + 1) + rf.x(i + 1, j + 1) + rf.x(i, j - 1) + rf.x(i + 1, j - 1));
   vy = T(0.5) * (rf.y(i, j) + rf.y(i, j + 1)) +
        T(0.25) * (rf.y(i + 1, j) + rf.y(i + 1, j + 1) + rf.y(i - 1, j) + rf.y(i - 1, j + 1));
-}
-
-// ---- coarsest level ----------------------------------------------------------
-
-// Solve L L^* x = b with the lower Cholesky factor Lf (column-major n x n), by one
-// warp (all 32 lanes call it); x and b may not alias.
-template <class T>
-__device__ __forceinline__ void chol_solve_warp(const cx<T>* Lf, int n, const cx<T>* b, cx<T>* x, int lane) {
-  // forward: L y = b  (y stored in x)
-  for (int i = 0; i < n; ++i) {
-    cx<T> acc = czero<T>();
-    for (int k = lane; k < i; k += 32) acc = acc + cmul(Lf[(long)k * n + i], x[k]);
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-    }
-    if (lane == 0) {
-      const T d = Lf[(long)i * n + i].x;
-      const cx<T> v = b[i] - acc;
-      x[i] = mk<T>(v.x / d, v.y / d);
-    }
-    __syncwarp();
-  }
-  // backward: L^* x = y
-  for (int i = n - 1; i >= 0; --i) {
-    cx<T> acc = czero<T>();
-    for (int k = i + 1 + lane; k < n; k += 32) acc = acc + cmulc(Lf[(long)i * n + k], x[k]);
-    for (int o = 16; o > 0; o >>= 1) {
-      acc.x += __shfl_xor_sync(0xffffffffu, acc.x, o);
-      acc.y += __shfl_xor_sync(0xffffffffu, acc.y, o);
-    }
-    if (lane == 0) {
-      const T d = Lf[(long)i * n + i].x;
-      const cx<T> v = x[i] - acc;
-      x[i] = mk<T>(v.x / d, v.y / d);
-    }
-    __syncwarp();
-  }
-}
-
-// The same solve with the factor in shared memory at leading dimension ld (n + 1
-// keeps both a column and a row of it free of bank conflicts), both triangular
-// sweeps in column order: once x_k is known, its multiple of column k of L (row
-// k of L^*) leaves the remaining right-hand side, so a step is one division and
-// one strided update with no reduction.
-template <class T>
-__device__ __forceinline__ void chol_solve_warp_cols(const cx<T>* Lf, int ld, int n, const cx<T>* b, cx<T>* x,
-                                                     int lane) {
-  for (int j = lane; j < n; j += 32) x[j] = b[j];
-  __syncwarp();
-  // forward: L y = b  (y stored in x)
-  for (int k = 0; k < n; ++k) {
-    const T d = Lf[k * ld + k].x;
-    const cx<T> v = x[k];
-    const cx<T> y = mk<T>(v.x / d, v.y / d);
-    for (int j = k + 1 + lane; j < n; j += 32) x[j] = x[j] - cmul(Lf[k * ld + j], y);
-    __syncwarp();
-    if (lane == 0) x[k] = y;
-    __syncwarp();
-  }
-  // backward: L^* x = y, (L^*)(i,k) = conj(L(k,i)) = conj(Lf[i ld + k])
-  for (int k = n - 1; k >= 0; --k) {
-    const T d = Lf[k * ld + k].x;
-    const cx<T> v = x[k];
-    const cx<T> xk = mk<T>(v.x / d, v.y / d);
-    for (int i = lane; i < k; i += 32) x[i] = x[i] - cmulc(Lf[i * ld + k], xk);
-    __syncwarp();
-    if (lane == 0) x[k] = xk;
-    __syncwarp();
-  }
 }
 
 }  // namespace pbs

@@ -98,7 +98,7 @@ __global__ void __launch_bounds__(kFineMaxThreads) k_node_down(Lvl<T> L, int nc,
       for_colour<T>(q, lo - 2 - e, lo + FT + 1 + e, oa, ob, [&](int a, int bb) {
         const int k = bb * W + a;
         const cx<T> res = sb[k] - P_at<T>(rs, L, oa + a, ob + bb);
-        sx[k] = sx[k] + (T(1) / P_diag<T>(L)) * res;
+        sx[k] = sx[k] + L.pinv * res;
       });
       __syncthreads();
     }
@@ -162,7 +162,7 @@ __global__ void __launch_bounds__(kFineMaxThreads) k_node_up(Lvl<T> L, int nc, i
       for_colour<T>(q, lo - e, lo + FT + e, oa, ob, [&](int a, int bb) {
         const int k = bb * W + a;
         const cx<T> res = sb[k] - P_at<T>(rs, L, oa + a, ob + bb);
-        sx[k] = sx[k] + (T(1) / P_diag<T>(L)) * res;
+        sx[k] = sx[k] + L.pinv * res;
       });
       __syncthreads();
     }
@@ -249,7 +249,7 @@ __global__ void __launch_bounds__(NT) k_node_down_rb(Lvl<float> L, int nc, int m
   const cx<T>* b = B + c * ldb;
   const cx<T>* x0 = X0 ? X0 + c * ld0 : nullptr;
   const bool in = oa >= 0 && ob >= 0 && oa + W <= L.n && ob + W <= L.m;
-  const T inv = T(1) / P_diag<T>(L);
+  const T inv = L.pinv;
   int bu[KB], bv[KB];
   cx<T> xr[KB][4], br[KB][4];
 #pragma unroll
@@ -344,7 +344,7 @@ __global__ void __launch_bounds__(NT) k_node_up_rb(Lvl<float> L, int nc, int mc,
   const cx<T>* xc = Xc + c * ldc;
   const bool in = oa >= 0 && ob >= 0 && oa + W <= L.n && ob + W <= L.m;
   const bool cin = ca >= 0 && cb >= 0 && ca + H + 1 <= nc && cb + H + 1 <= mc;
-  const T inv = T(1) / P_diag<T>(L);
+  const T inv = L.pinv;
   int bu[KB], bv[KB];
   cx<T> xr[KB][4], br[KB][4];
 #pragma unroll
