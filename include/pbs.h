@@ -38,7 +38,8 @@
  *  - PBS_TUNE_CACHE=<file>: where tuned choices are kept (default
  *    $HOME/.cache/pbs_tune.json); PBS_TUNE_FORCE=<prefix>=<i>,...: choice i for
  *    every tuning key with that prefix (tests);
- *  - PBS_GRAM=tc: offer the tensor-core Gram kernel to the tuner;
+ *  - PBS_GRAM=tc: the mixed policy's Gram on the tensor cores for every width
+ *    (default: from nine trial columns on);
  *  - PBS_GRAPHS=0: no CUDA-graph replays of the multigrid sequences;
  *  - PBS_VERBOSE: per-iteration traces on stderr (synchronises the stream).
  */

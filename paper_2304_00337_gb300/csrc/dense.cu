@@ -710,28 +710,31 @@ __global__ void __launch_bounds__(256, 3) k_gram_df(Lvl<df> L, WtsDF w, MassFact
   }
 }
 
-// sum partials in fixed order; write full Hermitian q x q (column-major) per group
-__global__ void k_gram_finalize(const double2* __restrict__ part, int npart, int q, double2* __restrict__ GM,
-                                double2* __restrict__ GA) {
-  const int g = blockIdx.y;
-  const int ne = q * (q + 1) / 2;
-  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < 2 * ne; e += gridDim.x * blockDim.x) {
-    double2 s = make_double2(0, 0);
-    for (int pp = 0; pp < npart; ++pp) {
-      const double2 v = part[((long)g * npart + pp) * 2 * ne + e];
-      s.x += v.x;
-      s.y += v.y;
-    }
-    const int ee = e < ne ? e : e - ne;
-    double2* G = (e < ne ? GM : GA) + (long)g * q * q;
-    int bi = int((sqrt(8.0 * ee + 1.0) - 1.0) * 0.5);
-    while ((bi + 1) * (bi + 2) / 2 <= ee) ++bi;
-    while (bi * (bi + 1) / 2 > ee) --bi;
-    const int ai = ee - bi * (bi + 1) / 2;
-    if (ai == bi) s.y = 0.0;
-    G[ai + (long)bi * q] = s;
-    G[bi + (long)ai * q] = conj(s);
-  }
+// Sum of the partials in a fixed order, written as full Hermitian q x q (column-major) per group: 8
+// threads share an entry (every eighth partial each), the 8 sums added in order.  (One thread per
+// entry left a chain of npart FP64 additions on four SMs: 65 us for 304 partials at q = 30.)
+constexpr int kFinEntries = 32;
+__global__ void __launch_bounds__(8 * kFinEntries) k_gram_finalize(const double2* __restrict__ part, int npart, int q,
+                                                                   double2* __restrict__ GM, double2* __restrict__ GA) {
+  __shared__ double2 red[8][kFinEntries];
+  const int g = blockIdx.y, ne = q * (q + 1) / 2, l = threadIdx.x % kFinEntries, w = threadIdx.x / kFinEntries;
+  const int e = blockIdx.x * kFinEntries + l;
+  double2 s = make_double2(0, 0);
+  if (e < 2 * ne)
+    for (int pp = w; pp < npart; pp += 8) s = s + part[((long)g * npart + pp) * 2 * ne + e];
+  red[w][l] = s;
+  __syncthreads();
+  if (w != 0 || e >= 2 * ne) return;
+  for (int k = 1; k < 8; ++k) s = s + red[k][l];
+  const int ee = e < ne ? e : e - ne;
+  double2* G = (e < ne ? GM : GA) + (long)g * q * q;
+  int bi = int((sqrtf(8.0f * ee + 1.0f) - 1.0f) * 0.5f);
+  while ((bi + 1) * (bi + 2) / 2 <= ee) ++bi;
+  while (bi * (bi + 1) / 2 > ee) --bi;
+  const int ai = ee - bi * (bi + 1) / 2;
+  if (ai == bi) s.y = 0.0;
+  G[ai + (long)bi * q] = s;
+  G[bi + (long)ai * q] = conj(s);
 }
 
 // ---- small dense Rayleigh-Ritz (one block) -------------------------------
@@ -1744,26 +1747,31 @@ int group_bucket(int ngroups) {
   return b;
 }
 
+// Where the mixed policy's Gram runs on the tensor cores (gram_tc.cu) instead of k_gram_df: from nine
+// columns on (one GB300, one group, ms on the tensor cores / in double-float: 256 x 256, q = 12
+// 0.12 / 0.17, q = 30 0.15 / 0.36, q = 42 0.32 / 0.75, q = 96 0.68 / 4.6; 1024 x 1024, q = 12
+// 0.99 / 1.5, q = 30 1.27 / 4.1, q = 48 4.2 / 11.4; 64 x 64, q = 30 0.055 / 0.078), and while the
+// weights' square roots span at most 2^8 (the headroom of its fixed-point curls).
+bool gram_tc_rule(const Level& L, int q) {
+  if (!L.sw || !(L.wmin * 65536.0 >= L.wmax)) return false;
+  return q >= 9 || gram_on_tensor_cores();
+}
+
 void gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
                  double2* d_partials, long partial_capacity, bool dfa, cudaStream_t s) {
   if (q <= 0 || ngroups <= 0) return;
   if (q > kMaxTrial) fail(PBS_EINVAL, "trial block too wide");
   const int ne = q * (q + 1) / 2;
   const int np0 = gram_partials(L.N(), ngroups);
-  // variants: the kernel (tensor cores or double-float, mixed policy) and the number
-  // of partial blocks per group; the autotuner picks among them on first use
+  // variants: the number of partial blocks per group and (double-float) the row stride of the
+  // staged arrays; the autotuner picks among them on first use
   struct Variant {
-    int kernel;  // 0: FP64, 1: double-float, 2: tensor cores
+    int kernel;  // 0: FP64, 1: double-float
     int npart;
     bool pad;  // double-float kernel: bank-spread row stride of the staged arrays
   };
-  Variant var[6];
+  Variant var[4];
   int nvar = 0;
-  if (dfa && gram_tc_supported(q) && gram_on_tensor_cores()) {
-    // offered first: with tuning off (PBS_TUNE=0) the tensor-core kernel runs
-    var[nvar++] = {2, np0, false};
-    var[nvar++] = {2, 2 * np0, false};
-  }
   const int kern = dfa ? 1 : 0;
   var[nvar++] = {kern, np0, false};
   var[nvar++] = {kern, 2 * np0, false};
@@ -1771,13 +1779,28 @@ void gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngr
     var[nvar++] = {kern, np0, true};
     var[nvar++] = {kern, 2 * np0, true};
   }
+  const std::string key = std::string(dfa ? "gram_df" : "gram") + std::to_string(nvar) + "|" + std::to_string(L.n) + "x" +
+                          std::to_string(L.m) + "|q" + std::to_string(q) + "|g" +
+                          std::to_string(group_bucket(ngroups)) + "|" + device_tag();
+  // flops: three complex MACs per entry and node
+  const double work = 8.0 * ne * 3.0 * L.N() * ngroups;
+  if (dfa && gram_tc_rule(L, q) && !tune_forced(key)) {
+    // (the scratch for the exponents is part of every partials buffer)
+    const long room = (partial_capacity - (long)(gram_tc_scratch(q, ngroups) / sizeof(double2)) - 1) / (2L * ngroups * ne);
+    const int np = (int)std::min<long>(gram_tc_partials(L.n, L.m, q, ngroups), room);
+    if (np < 1) fail(PBS_EINVAL, "gram partials buffer too small");
+    const long used = (long)ngroups * np * 2 * ne;
+    timer_begin(KC_GRAM, s, work);
+    gram_tc(L, d_ph, roles, q, ngroups, np, d_partials, reinterpret_cast<int*>(d_partials + used), s);
+    k_gram_finalize<<<dim3((2 * ne + kFinEntries - 1) / kFinEntries, ngroups), 8 * kFinEntries, 0, s>>>(d_partials, np, q, GM, GA);
+    timer_end(KC_GRAM, s);
+    PBS_LAUNCHED();
+    return;
+  }
   auto fits = [&](const Variant& v) { return (long)ngroups * v.npart * 2 * ne <= partial_capacity; };
   if (!fits(var[0])) fail(PBS_EINVAL, "gram partials buffer too small");
   auto launch = [&](const Variant& v) {
-    if (v.kernel == 2) {
-      gram_tc(L, d_ph, roles, q, ngroups, v.npart, d_partials, s);
-      count_df_launch();
-    } else if (v.kernel == 1) {
+    if (v.kernel == 1) {
       gram_df_dispatch<kGdTile>(L, d_ph, roles, q, ngroups, v.npart, v.pad, d_partials, s);
       count_df_launch();
     } else {
@@ -1791,31 +1814,27 @@ void gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngr
                                                               d_partials, v.npart);
     }
     PBS_LAUNCHED();
-    k_gram_finalize<<<dim3((2 * ne + 255) / 256, ngroups), 256, 0, s>>>(d_partials, v.npart, q, GM, GA);
+    k_gram_finalize<<<dim3((2 * ne + kFinEntries - 1) / kFinEntries, ngroups), 8 * kFinEntries, 0, s>>>(d_partials, v.npart, q, GM, GA);
     PBS_LAUNCHED();
   };
   int pick = 0;
   if (nvar > 1) {
-    const std::string key = std::string(dfa ? "gram_df" : "gram") + std::to_string(nvar) + "|" +
-                            std::to_string(L.n) + "x" + std::to_string(L.m) + "|q" + std::to_string(q) + "|g" +
-                            std::to_string(group_bucket(ngroups)) + "|" + device_tag();
     // a candidate whose partial sums do not fit the buffer runs the first one instead
     pick = tune_pick(key, nvar, [&](int c) { launch(fits(var[c]) ? var[c] : var[0]); }, s);
     if (!fits(var[pick])) pick = 0;
   }
-  timer_begin(KC_GRAM, s, 8.0 * ne * 3.0 * L.N() * ngroups);  // flops: three complex MACs per entry and node
+  timer_begin(KC_GRAM, s, work);
   launch(var[pick]);
   timer_end(KC_GRAM, s);
 }
 
 long gram_partials_size(long rows, int q, int ngroups) {
-  // partial sums for up to twice the default split (a tuning candidate)
-  return 2L * ngroups * gram_partials(rows, ngroups) * q * (q + 1);
+  // partial sums for up to twice the default split (a tuning candidate); the tensor-core kernel has
+  // no more (gram_groups falls back where it had), and its exponents follow them
+  return 2L * ngroups * gram_partials(rows, ngroups) * q * (q + 1) + (long)(gram_tc_scratch(q, ngroups) / sizeof(double2)) + 1;
 }
 
 bool gram_on_tensor_cores() {
-  // PBS_GRAM=tc offers the tensor-core kernel to the autotuner (opt-in); the default
-  // is the double-float kernel
   static const bool tc = [] {
     const char* v = std::getenv("PBS_GRAM");
     return v && std::strcmp(v, "tc") == 0;

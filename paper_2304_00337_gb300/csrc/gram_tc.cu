@@ -1,341 +1,597 @@
-// Block Gram matrices on the tensor cores (the mixed policy's Gram, Section 4).
+// Block Gram matrices of the mixed policy on the tensor cores (tcgen05, accumulators in TMEM).
 //
-// GM = S^* M S and GA = (C S)^* W (C S) are sums over the mesh of products of
-// values that need about 2^-47 relative accuracy (the double-float kernel's level).
-// Written with real operands, X = [Re u | Im u] and Y = [Re v | Im v] (u = S,
-// v = M S for GM; u = C S, v = W C S for GA), both products are P = X^T Y over
-// the rows (edges, or cells):
-//   G_re[a][b] = P[a][b] + P[h+a][h+b],   G_im[a][b] = P[a][h+b] - P[h+a][b]
-// (h = the padded half width).  P is evaluated with the splitting of Ozaki,
-// Ogita, Oishi and Rump (2012): every value, scaled by a power of two 2^-e
-// shared by its column over the chunk's rows, is written as a sum of six
-// bfloat16 slices, x = sum_i X_i, X_i = x_i 2^-8(i+1) with integer digits x_i
-// (|x_0| <= 256, |x_i| <= 128 after rounding to nearest), so that every slice
-// product X_i Y_j is exact in FP32 and a sum of 64 of them stays exact as long as
-// i + j <= 2.  The tensor cores (mma.sync m16n8k16, bf16 in, FP32 accumulate)
-// form the 21 slice products with i + j <= 5: the leading groups (i + j = 0, 1,
-// 2) in exact FP32 accumulators, the rest (whose rounding is 2^-24 of terms
-// already 2^-24 smaller) in one plain FP32 accumulator, all folded into
-// double-float sums after every chunk.  The dropped products (i + j >= 6)
-// and the slicing leave about 2^-48 of the scaled magnitudes per term.
+// The sums of k_gram_df (dense.cu) - GM = S^* M S through the bidiagonal factor of the mass matrix
+// and GA = (C S)^* W (C S) - are products P = V V^T of real operands V, rows (trial column,
+// component), columns mesh nodes:
+//   GM: v = z_x and z_y, z_x = sqrt(mx)(alpha x(i,j) + beta x(i,j+1)), z_y likewise along i;
+//   GA: v = sqrt(w) curl.
+// Each operand value is brought to a fixed-point integer of 48 bits, relative to a power of two
+// that bounds its trial column (k_gram_exponents), and cut into six signed 8-bit digits, held as
+// binary16 integers.  A digit product is exact in the tensor core's FP32 sums: P = sum over digit
+// pairs i + j <= 5, and those with i odd and i + j = 6, of P_ij 2^{-8(i+j)} (the error-free
+// splitting of Ozaki, Ogita, Oishi and Rump, 2012; the squares of digit 3 do not average out on
+// the diagonal, so they are kept).  256 nodes add at most 2 x 512 x 2^14 = 2^24 to a sum of equal i + j <= 3, so FP32 sums
+// of 256 nodes are exact; they are then taken out of TMEM and added up as 64-bit integers.  The
+// only rounding is that of the 48-bit operands (2^-47 of the column's largest value; the
+// double-float kernel rounds each value to 2^-47 of itself, and its curls to 2^-47 of the edge
+// values they are differences of) and of the dropped pairs, whose signs are random.
 //
-// The scale of a column is a power of two above its largest magnitude over the
-// chunk's rows, so each value keeps about 48 bits relative to its chunk's largest
-// one (as the double-float kernel keeps 48 bits of every value); the curls of a
-// smooth field are far smaller than the field itself, and a scale taken from a
-// bound such as 4 max|u| would cost them a dozen bits.
+// Digits come from integers, not from double-float: FP64 input is shifted into 64-bit fixed point
+// (the curl's differences are then exact), multiplied by 63-bit constants, and a byte permutation
+// with the exponent byte of 1024 turns a digit into a binary16 number.  About 200 integer
+// instructions per node, column and matrix against 79 floating-point ones per node and entry of
+// the matrix (q (q + 1) / 2 of them) in k_gram_df.
 //
-// A block takes one product (GM or GA) of one group over a contiguous range of
-// nodes, staging chunks of 16 nodes (the stencils M s and C s in double-float, as
-// in the double-float kernel), then their slices, in shared memory; each warp multiplies
-// one 16-row strip of P against up to NT 8-column tiles.  Tiles holding only
-// entries below the diagonal of each of the four h x h blocks of P are skipped
-// (the Gram matrices are Hermitian).
-#include <cuda_bf16.h>
-
+// One CTA per SM (shared memory) owns a pair (I <= J) of 32-column blocks of GM or of GA (blockIdx.z)
+// and every npart-th chunk of 32 nodes x 8 mesh rows.  16 producer warps fill a ring of 32-node stages; one
+// thread of a 17th warp issues the MMAs (A = two digits of block I, 128 rows; B = up to four
+// digits of block J, 64 rows each; K-major, no swizzle); after each chunk the producers read
+// TMEM.  Accumulator D_t (t = 0 .. 5, 128 rows x 64 columns) holds the pairs i + j = t of even i in
+// rows 0-63 and i + j = t + 1 of odd i in rows 64-127: A = digits (2 u, 2 u + 1), B = digit t - 2 u.
+// For I = J the product is symmetric, even-odd pairs are the transposes of odd-even ones, and the
+// rows 0-63 of odd t are not used.
 #include <algorithm>
 #include <cmath>
-#include <vector>
+#include <cstdlib>
+#include <cstring>
 
 #include "internal.h"
-#include "mgpoint.cuh"
+#include "tc.cuh"
 
 namespace pbs {
+
 namespace {
 
-constexpr int kTcNodes = 16;               // nodes per staged chunk
-constexpr int kTcSlices = 6;               // bf16 slices per value
-constexpr int kTcMaxHalf = 48;             // padded half width h (q <= 48)
-constexpr int kTcMaxTasks = 16;            // warps per block
-constexpr int kTcRowsGM = 2 * kTcNodes;    // GM rows per chunk: x-edge and y-edge of every node
-constexpr int kTcStride = kTcRowsGM + 8;   // shared row stride (bf16): 80 bytes, conflict-free ldmatrix
+constexpr int kProducers = 512;            // producer and epilogue threads (16 warps)
+constexpr int kThreads = kProducers + 32;  // and the warp whose first lane issues the MMAs
+constexpr int kCols = 32;                  // trial columns per block: 64 operand rows
+constexpr int kSlices = 6;
+constexpr int kRows = 64 * kSlices;        // operand rows of a block in shared memory, digit-major
+constexpr int kChunk = 256, kStage = 32;   // nodes per TMEM sum, per ring stage
+constexpr int kOctet = kRows * 16;         // bytes of 8 nodes of a block's rows
+constexpr int kArray = kStage / 8 * kOctet;
+constexpr int kSmem = 196608 + 1024;       // ring and barriers
+constexpr unsigned kTmemCols = 512;
 
-// One warp's share of P: rows [16 mt, 16 mt + 16) and the 8-column tiles nt[0..nn).
-constexpr int kTcMaxNT = 4;
-struct TcTask {
-  unsigned char mt, nn, nt[kTcMaxNT];
+// ---- fixed point ----------------------------------------------------------------
+// A factor 0 <= f < 1 as (hi + lo 2^-31) 2^-31.
+struct Fix {
+  int hi, lo;
 };
-struct TcTasks {
-  TcTask t[kTcMaxTasks];
-  int count;
-};
+inline Fix make_fix(double f) {
+  Fix r;
+  const double s = f * 2147483648.0;
+  r.hi = (int)s;
+  r.lo = (int)((s - (double)r.hi) * 2147483648.0);
+  return r;
+}
+// v 2^{52 - E}, |v| < 2^E, E > kMinExp, truncated to an integer.  (Zero and subnormals, exponent
+// field 0, are shifted out whole.)
+__device__ __forceinline__ long long to_fixed(double v, int E) {
+  const int hi = __double2hiint(v), sh = min(E + 1023 - ((hi >> 20) & 0x7FF), 63);  // at least 1
+  const unsigned long long m =
+      (((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(v)) >> sh;
+  const long long s = (long long)(hi >> 31);
+  return ((long long)m ^ s) - s;
+}
+// Operand digits of 16 z + bias with z = X f / 32 (+ Y g / 32), |z| < 0.99 2^47, rounded to the nearest
+// integer: six bytes that carry 0x80 too much each.  h f.hi and the two high products are exact to
+// a few units of 2^-4.
+constexpr long long kDigitBias = 0x808080808080ll * 16 + 8;
+__device__ __forceinline__ unsigned long long digits1(long long X, Fix f) {
+  const int h = (int)(X >> 32);
+  const long long t = (long long)h * f.hi + kDigitBias + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
+  return (unsigned long long)(t + 2 * (long long)__mulhi(h, f.lo)) >> 4;
+}
+__device__ __forceinline__ unsigned long long digits2(long long X, Fix f, long long Y, Fix g) {
+  const int h = (int)(X >> 32), k = (int)(Y >> 32);
+  const long long t = (long long)h * f.hi + ((long long)k * g.hi + kDigitBias);
+  const unsigned l = __umulhi((unsigned)X, (unsigned)f.hi) + __umulhi((unsigned)Y, (unsigned)g.hi);  // below 2^32
+  return (unsigned long long)(t + (long long)l + 2 * (long long)(__mulhi(h, f.lo) + __mulhi(k, g.lo))) >> 4;
+}
 
-__device__ __forceinline__ const double2* tc_col(const Roles& R, int g, int a) {
+// Operand values of two neighbouring nodes and one component (biased digits b0, b1): stores digit s
+// of both at base + 1024 s (64 rows of 16 bytes) as two binary16 integers -128 .. 127.  A byte next to
+// the byte 0x64 is the binary16 number 1024 + byte.
+__device__ __forceinline__ void store_digits(unsigned base, unsigned long long b0, unsigned long long b1) {
+  const unsigned l0 = (unsigned)b0, h0 = (unsigned)(b0 >> 32), l1 = (unsigned)b1, h1 = (unsigned)(b1 >> 32);
+  const __half2 bias = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1024 + 128
+  auto put = [&](int s, unsigned two) {
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&two), bias);
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(base + 1024u * s), "r"(*reinterpret_cast<const unsigned*>(&d)) : "memory");
+  };
+  // (byte i, byte i + 1 of both words), then each pair with the exponent byte
+  const unsigned t45 = __byte_perm(h0, h1, 0x5140), t23 = __byte_perm(l0, l1, 0x7362), t01 = __byte_perm(l0, l1, 0x5140);
+  put(0, __byte_perm(t45, 0x64646464u, 0x4342));
+  put(1, __byte_perm(t45, 0x64646464u, 0x4140));
+  put(2, __byte_perm(t23, 0x64646464u, 0x4342));
+  put(3, __byte_perm(t23, 0x64646464u, 0x4140));
+  put(4, __byte_perm(t01, 0x64646464u, 0x4342));
+  put(5, __byte_perm(t01, 0x64646464u, 0x4140));
+}
+
+// Bloch continuation of a value across the level's boundary, out of line: its FP64 products are
+// otherwise evaluated (predicated) for every value, and the FP64 pipe is narrow.
+__device__ __noinline__ double2 rotate(double2 v, double2 phase) { return cmul(v, phase); }
+
+__device__ __forceinline__ const double2* trial_col(const Roles& R, int g, int a) {
   const int r = a / R.pr;
   const double2* base = r == 0 ? R.b[0] : (r == 1 ? R.b[1] : R.b[2]);
   return base + ((long)g * R.pr + a % R.pr) * R.ld;
 }
 
-__device__ __forceinline__ void mma_bf16(float (&c)[4], const unsigned (&a)[4], unsigned b0, unsigned b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
-      "{%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+// x-edges of two neighbouring nodes (i even; i + 1 on the same mesh row) on mesh row j <= m, y-edges of
+// the two and the next node on row j < m; Bloch-continued.
+struct PairX {
+  double2 v[2];
+};
+struct PairY {
+  double2 v[3];
+};
+__device__ __forceinline__ PairX load_x(const double2* __restrict__ X, int i, int j, int n, int m, const double2& be,
+                                        bool in) {
+  PairX p;
+  p.v[0] = p.v[1] = make_double2(0.0, 0.0);
+  if (in) {
+    const double2* a = X + (long)(j == m ? 0 : j) * n + i;
+    p.v[0] = a[0];
+    p.v[1] = a[1];
+    if (j == m) {
+      p.v[0] = rotate(p.v[0], be);
+      p.v[1] = rotate(p.v[1], be);
+    }
+  }
+  return p;
 }
-__device__ __forceinline__ void ldsm_x4(unsigned (&r)[4], const void* p) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];\n"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
-               : "r"(s));
-}
-__device__ __forceinline__ void ldsm_x2(unsigned& r0, unsigned& r1, const void* p) {
-  const unsigned s = (unsigned)__cvta_generic_to_shared(p);
-  asm volatile("ldmatrix.sync.aligned.m8n8.x2.shared.b16 {%0,%1}, [%2];\n" : "=r"(r0), "=r"(r1) : "r"(s));
+__device__ __forceinline__ PairY load_y(const double2* __restrict__ Y, int i, int j, int n, const double2& al, bool in) {
+  PairY p;
+  p.v[0] = p.v[1] = p.v[2] = make_double2(0.0, 0.0);
+  if (in) {
+    const double2* a = Y + (long)j * n;
+    p.v[0] = a[i];
+    p.v[1] = a[i + 1];
+    p.v[2] = a[i + 2 == n ? 0 : i + 2];
+    if (i + 2 == n) p.v[2] = rotate(p.v[2], al);
+  }
+  return p;
 }
 
-// 2^k as a float (k within the normal range), exact
-__device__ __forceinline__ float pow2f(int k) { return __int_as_float((k + 127) << 23); }
-
-// Six bf16 slices of a double-float value v with |v| < 2^e: slice i holds
-// x_i 2^(e - 8(i+1)) relative to the unscaled value; stored without the 2^e
-// (which the block applies to P at the end).
-__device__ __forceinline__ void split_store(df v, int e, __nv_bfloat16* dst, int slice_stride) {
-  const float sc = pow2f(8 - e);  // scaled by 2^-e, times 256 for the first digit
-  float hi = v.hi * sc, lo = v.lo * sc;
+// Exponents of the operands of every trial column: E[2 c] with |x|, |y| < 2^E, E[2 c + 1] with
+// sqrt(w) |curl| < 0.99 2^E (c = g q + column; kExpInf where a value is not finite; very negative
+// for a column of zeros).  A bound needs few bits: the curl is formed in binary32 from the leading
+// 21 bits of its edge values, 2^-18 of which is added to it (the digits then still reach 2^-60 of
+// the edge values, below their FP64 rounding).  A block of edge values outside the binary32 range
+// gives the bound without cancellation.  One pass over the block, bound by memory: 8 rows per thread, two
+// nodes wide, the upper row's x-edges carried to the next.
+constexpr int kExpThreads = 256, kExpTile = 64;  // a block's tile: 64 nodes x 64 mesh rows
+__global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, const double* __restrict__ ph, Roles roles, int q,
+                                                                const uint2* __restrict__ sw, int sw_exp,
+                                                                int* __restrict__ E) {
+  __shared__ int red[2][kExpThreads / 32];
+  const int col = blockIdx.y, g = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
+  const int tx = (n + kExpTile - 1) / kExpTile, by = blockIdx.x / tx, bx = blockIdx.x - by * tx;
+  const double2* X = trial_col(roles, g, col);
+  const double2* Y = X + (long)n * m;
+  const Ph<double> p = load_ph<double>(ph, g);
+  const int i = bx * kExpTile + 2 * lane, j0 = by * kExpTile + 8 * (tid >> 5);
+  const bool in = i < n;
+  int top = 0;          // largest high word (sign off): the exponent of the largest value
+  float cmax = 0.0f;    // largest 2^-sw_exp sqrt(w) (|c| + 2^-18 of the values), binary32 range only
+  auto lead = [&](double d) {
+    const int hi = __double2hiint(d), a = hi & 0x7FFFFFFF;
+    top = max(top, a);
+    const int f = a < (900 << 20) ? 0 : (a - (896 << 20)) << 3;
+    return __int_as_float((hi & 0x80000000) | f);
+  };
+  float x0[2][2];
+  {
+    const PairX v = load_x(X, i, j0, n, m, p.be, in && j0 < m);
 #pragma unroll
-  for (int i = 0; i < kTcSlices; ++i) {
-    const float d = rintf(hi);
-    // true slice value d 2^-8(i+1): exact in bf16 (|d| <= 256 is an 8-bit integer times a power of two)
-    dst[i * slice_stride] = __float2bfloat16_rn(d * pow2f(-8 * (i + 1)));
-    const df r = quick_two_sum(hi - d, lo);  // hi - d is exact
-    hi = r.hi * 256.0f;
-    lo = r.lo * 256.0f;
+    for (int k = 0; k < 2; ++k) {
+      x0[k][0] = lead(v.v[k].x);
+      x0[k][1] = lead(v.v[k].y);
+    }
+  }
+  for (int j = j0; j < min(j0 + 8, m); ++j) {
+    const PairX v = load_x(X, i, j + 1, n, m, p.be, in);
+    const PairY u = load_y(Y, i, j, n, p.al, in);
+    float y[3][2];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      y[k][0] = lead(u.v[k].x);
+      y[k][1] = lead(u.v[k].y);
+    }
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      const float s = in ? (float)sw[(long)j * n + i + k].x : 0.0f;
+#pragma unroll
+      for (int c = 0; c < 2; ++c) {
+        const float x1 = lead(c ? v.v[k].y : v.v[k].x);
+        const float d = fabsf((x1 - x0[k][c]) - (y[k + 1][c] - y[k][c]));
+        const float e = fmaxf(fmaxf(fabsf(x1), fabsf(x0[k][c])), fmaxf(fabsf(y[k + 1][c]), fabsf(y[k][c])));
+        cmax = fmaxf(cmax, s * fmaf(e, 0x1p-18f, d));
+        x0[k][c] = x1;
+      }
+    }
+  }
+  // high words order like the values, bits of non-negative floats too
+  const int t = __reduce_max_sync(0xffffffffu, top);
+  const int c = __reduce_max_sync(0xffffffffu, __float_as_int(cmax));
+  if (lane == 0) {
+    red[0][tid >> 5] = t;
+    red[1][tid >> 5] = c;
+  }
+  __syncthreads();
+  if (tid != 0) return;
+  int hi = 0, cb = 0;
+  for (int w = 0; w < kExpThreads / 32; ++w) {
+    hi = max(hi, red[0][w]);
+    cb = max(cb, red[1][w]);
+  }
+  const int e = hi >> 20;
+  if (e == 0) return;
+  int ex = e - 1022, ez;
+  if (e == 0x7FF) {
+    ex = ez = kExpInf;
+  } else if (e < 920 || e > 1140) {
+    ez = ex + sw_exp + 3;  // |c| <= 4 2^ex
+  } else {
+    // sw holds 31 bits; 2 % for the roundings and the margin; a block without curl counts as tiny
+    const float v = __int_as_float(cb) * (1.02f * 0x1p-31f);
+    ez = v > 0.0f ? ilogbf(v) + 1 + sw_exp : ex + sw_exp - 18;
+  }
+  int* Ec = E + 2 * ((long)g * q + col);
+  atomicMax(Ec, ex);
+  atomicMax(Ec + 1, ez);
+}
+
+struct GramArgs {
+  int n, m;
+  long N;
+  Fix ax, bx, ay, by;  // mass factor over kappa
+  double kappa2;
+  const uint2* sw;
+  int sw_exp;
+  const double* ph;
+  Roles roles;
+  int q;
+  const int* E;
+  double2* part;
+  int npart;
+};
+
+// One producer warp's part of a chunk (tile of 32 nodes x 8 mesh rows from (i0, j0)): per stage one
+// mesh row, 8 nodes of it (this lane's two from i), the colgroup of `blocks` 32-column blocks.  The
+// fixed-point x-edges of a row are those one row up of the row before: read and converted once.
+// `wait` blocks until the stage's place in the ring is free and returns it, `ready` hands it on.
+template <bool MASS, int BLOCKS, class Wait, class Ready>
+__device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* const (&Xc)[2], const int (&Ex)[2],
+                                              const int (&Ez)[2], const bool (&on)[2], const Ph<double>& p, int i, int j0,
+                                              unsigned place, Wait&& wait, Ready&& ready) {
+  const bool col_in = i < A.n;
+  long long xf[BLOCKS][2][2];  // x-edges of the current row: block, node, component
+  PairX nx;                    // loads of the next step (a single block's; two blocks load as they go)
+  PairY ny;
+#pragma unroll
+  for (int b = 0; b < BLOCKS; ++b) {
+    const PairX v = load_x(Xc[b], i, j0, A.n, A.m, p.be, on[b] && col_in && j0 < A.m);
+#pragma unroll
+    for (int k = 0; k < 2; ++k) {
+      xf[b][k][0] = to_fixed(v.v[k].x, Ex[b]);
+      xf[b][k][1] = to_fixed(v.v[k].y, Ex[b]);
+    }
+  }
+  if (BLOCKS == 1) {
+    const bool in = on[0] && col_in && j0 < A.m;
+    nx = load_x(Xc[0], i, j0 + 1, A.n, A.m, p.be, in);
+    ny = load_y(Xc[0] + A.N, i, j0, A.n, p.al, in);
+  }
+  for (int s = 0; s < kChunk / kStage; ++s) {
+    const int j = j0 + s;
+    const bool row_in = col_in && j < A.m;
+    uint2 w[2];
+    if (!MASS) {
+#pragma unroll
+      for (int k = 0; k < 2; ++k) w[k] = row_in ? A.sw[(long)j * A.n + i + k] : make_uint2(0, 0);
+    }
+    const unsigned dst = wait() + place;
+#pragma unroll
+    for (int b = 0; b < BLOCKS; ++b) {
+      if (BLOCKS == 2) {
+        nx = load_x(Xc[b], i, j + 1, A.n, A.m, p.be, on[b] && row_in);
+        ny = load_y(Xc[b] + A.N, i, j, A.n, p.al, on[b] && row_in);
+      }
+      long long x1[2][2], y[3][2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        x1[k][0] = to_fixed(nx.v[k].x, Ex[b]);
+        x1[k][1] = to_fixed(nx.v[k].y, Ex[b]);
+      }
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        y[k][0] = to_fixed(ny.v[k].x, Ex[b]);
+        y[k][1] = to_fixed(ny.v[k].y, Ex[b]);
+      }
+      if (BLOCKS == 1) {
+        const bool in = on[0] && col_in && j + 1 < A.m && s + 1 < kChunk / kStage;
+        nx = load_x(Xc[0], i, j + 2, A.n, A.m, p.be, in);
+        ny = load_y(Xc[0] + A.N, i, j + 1, A.n, p.al, in);
+      }
+      const unsigned at = dst + b * kArray;
+      const int sh = Ex[b] + A.sw_exp - Ez[b];
+#pragma unroll
+      for (int im = 0; im < 2; ++im) {
+        // (a row or column outside the level leaves zeros: its loads were zero, and the last row's
+        // carried x-edges are not used)
+        if (MASS) {
+          const long long u0 = row_in ? xf[b][0][im] : 0, u1 = row_in ? xf[b][1][im] : 0;
+          store_digits(at + im * 512, digits2(u0, A.ax, x1[0][im], A.bx), digits2(u1, A.ax, x1[1][im], A.bx));
+          store_digits(at + BLOCKS * kArray + im * 512, digits2(y[0][im], A.ay, y[1][im], A.by),
+                       digits2(y[1][im], A.ay, y[2][im], A.by));
+        } else {
+          unsigned long long z[2];
+#pragma unroll
+          for (int k = 0; k < 2; ++k) {
+            const long long d = (x1[k][im] - xf[b][k][im]) - (y[k + 1][im] - y[k][im]);
+            const long long e = sh >= 0 ? (long long)((unsigned long long)d << min(sh, 62)) : d >> min(-sh, 62);
+            z[k] = digits1(e, Fix{(int)w[k].x, (int)w[k].y});
+          }
+          store_digits(at + im * 512, z[0], z[1]);
+        }
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        xf[b][k][0] = x1[k][0];
+        xf[b][k][1] = x1[k][1];
+      }
+    }
+    ready();
   }
 }
 
-// exponent e with |v| < 2^e for every double-float v whose leading part is at most
-// m in magnitude (|v| <= m (1 + 2^-23)); 0 for an all-zero column.  Clamped so that
-// the float scalings by 2^(8-e) and 2^(ex+ey) stay in range.
-__device__ __forceinline__ int chunk_exp(float m) {
-  if (!(m > 0.0f)) return 0;
-  int e;
-  frexpf(m * 1.0000002f, &e);
-  return max(-60, min(60, e));
-}
+__global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
+  extern __shared__ unsigned char ring[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int g = blockIdx.y, nb = (A.q + kCols - 1) / kCols, npair = nb * (nb + 1) / 2;
+  const bool mass = (int)blockIdx.z < npair;  // GM first: its CTAs take twice as long
+  int I = 0, J = (int)blockIdx.z % npair;     // pair index -> (I <= J), J-major
+  {
+    int j = 0;
+    while ((j + 1) * (j + 2) / 2 <= J) ++j;
+    I = J - j * (j + 1) / 2;
+    J = j;
+  }
+  const bool diag = I == J;
+  const int arrays = mass ? 2 : 1, blocks = diag ? 1 : 2;
+  const int stage_bytes = arrays * blocks * kArray;  // array-major, block I then block J
+  const int nstage = min(8, 196608 / stage_bytes);
+  const unsigned ring0 = smem_u32(ring), bars = ring0 + 196608;
+  const unsigned full = bars, empty = bars + 64, done = bars + 128, tfree = bars + 136;
+  volatile int* abort = reinterpret_cast<volatile int*>(ring + 196608 + 144);
+  unsigned* tmem_slot = reinterpret_cast<unsigned*>(ring + 196608 + 148);
+  if (tid == 0) {
+    for (int s = 0; s < nstage; ++s) {
+      mbar_init(full + 8 * s, kProducers / 32);
+      mbar_init(empty + 8 * s, 1);
+    }
+    mbar_init(done, 1);
+    mbar_init(tfree, kProducers / 32);
+    *abort = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  // rows of absent columns stay zero
+  for (int t = tid; t < 196608 / 16; t += kThreads) reinterpret_cast<int4*>(ring)[t] = make_int4(0, 0, 0, 0);
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  if (warp == kProducers / 32) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(tmem_slot)), "r"(kTmemCols)
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const unsigned tmem = *tmem_slot;
+  const int tx = (A.n + kStage - 1) / kStage, nchunk = tx * ((A.m + 7) / 8), first = blockIdx.x;
+  const int mine = first < nchunk ? (nchunk - first + A.npart - 1) / A.npart : 0;
+  constexpr int kStages = kChunk / kStage;
 
-// grid: (npart, ngroups, 2); blockIdx.z = 0: GM, 1: GA.  H = padded half width.
-// Every chunk is scaled on its own: the largest magnitude of each operand column over
-// the chunk's rows sets its power of two, so the slices carry the chunk's own values
-// to 2^-48 (the accuracy of the double-float kernel's terms), and the chunk's slice
-// products are folded into the double-float sums with that chunk's scales.
-template <int H, int NT>
-__global__ void __launch_bounds__(NT == 3 ? kTcMaxTasks * 32 : 384) k_gram_tc(Lvl<df> L, WtsDF w, const double* ph,
-                                                                            Roles roles, int q, TcTasks tasks,
-                                                                            double2* __restrict__ part, int npart) {
-  extern __shared__ float4 tc_sm[];
-  constexpr int W2 = 2 * H;           // real columns of X and Y
-  constexpr int SL = W2 * kTcStride;  // bf16 elements of one slice of one operand
-  __nv_bfloat16* sX = reinterpret_cast<__nv_bfloat16*>(tc_sm);  // [slice][W2][stride]
-  __nv_bfloat16* sY = sX + kTcSlices * SL;
-  dcx* su = reinterpret_cast<dcx*>(sY + kTcSlices * SL);  // [a][row] chunk values (X operand)
-  dcx* sv = su + H * kTcRowsGM;                            // [a][row] (Y operand)
-  __shared__ int ex[kTcMaxHalf], ey[kTcMaxHalf];
-  const int g = blockIdx.y, prod = blockIdx.z;
-  const int tid = threadIdx.x, nt = blockDim.x, lane = tid & 31, warp = tid >> 5;
-  const Ph<df> p = load_ph<df>(ph, g);
-  const long N = (long)L.n * L.m;
-  const long nchunks = (N + kTcNodes - 1) / kTcNodes;
-  const long per = (nchunks + npart - 1) / npart;
-  const long c_begin = blockIdx.x * per, c_end = min(nchunks, c_begin + per);
-  const long r_end = min(N, c_end * kTcNodes);
-  const int rows = prod == 0 ? kTcRowsGM : kTcNodes;  // rows per chunk
-  // padding columns (a >= q) stay zero in every slice
-  for (int t = tid; t < 2 * kTcSlices * SL; t += nt) sX[t] = __float2bfloat16_rn(0.0f);
-
-  const bool active = warp < tasks.count;
-  TcTask tk{0, 0, {0, 0, 0, 0}};
-  if (active) tk = tasks.t[warp];
-  df sum[NT][4];  // P entries of the warp's tiles
+  long long acc[16];  // this thread's sums: row lane + 32 (warp & 3) of the pair, 16 columns from 16 (warp >> 2)
 #pragma unroll
-  for (int t = 0; t < NT; ++t)
-#pragma unroll
-    for (int k = 0; k < 4; ++k) sum[t][k] = df_zero();
+  for (int k = 0; k < 16; ++k) acc[k] = 0;
 
-  for (long ch = c_begin; ch < c_end; ++ch) {
-    const long r0 = ch * kTcNodes;
-    __syncthreads();  // the previous chunk's slices and scales are no longer read
-    // 1. the chunk's operand values (stencils in double-float)
-    for (int t = tid; t < q * kTcNodes; t += nt) {
-      const int a = t / kTcNodes, rr = t % kTcNodes;
-      const long node = r0 + rr;
-      const dcx z = dcx_make(df_zero(), df_zero());
-      dcx u0 = z, u1 = z, v0 = z, v1 = z;
-      if (node < r_end) {
-        const int i = int(node % L.n), j = int(node / L.n);
-        const ERdD<df> rd{tc_col(roles, g, a), L.n, L.m, p};
-        if (prod == 0) {
-          u0 = rd.x(i, j);
-          u1 = rd.y(i, j);
-          v0 = M_x<df>(rd, L, i, j);
-          v1 = M_y<df>(rd, L, i, j);
-        } else {
-          u0 = curl_at<df>(rd, i, j);
-          v0 = w(i, j) * u0;
+  if (warp == kProducers / 32) {
+    if (lane == 0) {
+      int st = 0;
+      unsigned par = 0;
+      for (int c = 0; c < mine; ++c) {
+        if (c > 0) {
+          mbar_wait(tfree, (c - 1) & 1, abort);
+          tc_fence_after();
         }
-      }
-      if (prod == 0) {
-        su[a * kTcRowsGM + 2 * rr] = u0;
-        su[a * kTcRowsGM + 2 * rr + 1] = u1;
-        sv[a * kTcRowsGM + 2 * rr] = v0;
-        sv[a * kTcRowsGM + 2 * rr + 1] = v1;
-      } else {
-        su[a * kTcRowsGM + rr] = u0;
-        sv[a * kTcRowsGM + rr] = v0;
-      }
-    }
-    __syncthreads();
-    // 2. column scales of the chunk: one warp per operand column (rows <= 32 = lanes)
-    for (int c = warp; c < 2 * q; c += nt / 32) {
-      const dcx* col = (c < q ? su : sv) + (c % q) * kTcRowsGM;
-      float m = 0.0f;
-      if (lane < rows) m = fmaxf(fabsf(col[lane].x.hi), fabsf(col[lane].y.hi));
-      for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-      if (lane == 0) (c < q ? ex : ey)[c % q] = chunk_exp(m);
-    }
-    for (int a = q + tid; a < H; a += nt) {
-      ex[a] = 0;
-      ey[a] = 0;
-    }
-    __syncthreads();
-    // 3. slices
-    for (int t = tid; t < q * rows; t += nt) {
-      const int a = t / rows, r = t % rows;
-      const dcx u = su[a * kTcRowsGM + r], v = sv[a * kTcRowsGM + r];
-      split_store(u.x, ex[a], sX + a * kTcStride + r, SL);
-      split_store(u.y, ex[a], sX + (H + a) * kTcStride + r, SL);
-      split_store(v.x, ey[a], sY + a * kTcStride + r, SL);
-      split_store(v.y, ey[a], sY + (H + a) * kTcStride + r, SL);
-    }
-    __syncthreads();
-    // 4. slice products on the tensor cores, folded with the chunk's scales
-    if (active) {
-      float acc[4][NT][4];  // [group: i+j = 0, 1, 2, >= 3][tile][fragment]
+        for (int s = 0; s < kStages; ++s) {
+          mbar_wait(full + 8 * st, par, abort);
+          tc_fence_after();
+          for (int ar = 0; ar < arrays; ++ar) {
+            const unsigned a0 = ring0 + st * stage_bytes + ar * blocks * kArray, b0 = diag ? a0 : a0 + kArray;
 #pragma unroll
-      for (int s2 = 0; s2 < 4; ++s2)
-#pragma unroll
-        for (int t = 0; t < NT; ++t)
-#pragma unroll
-          for (int k = 0; k < 4; ++k) acc[s2][t][k] = 0.0f;
-      for (int k0 = 0; k0 < rows; k0 += 16) {
-        unsigned A[kTcSlices][4];
-#pragma unroll
-        for (int i = 0; i < kTcSlices; ++i)
-          ldsm_x4(A[i], sX + i * SL + (16 * tk.mt + (lane & 15)) * kTcStride + k0 + (lane >> 4) * 8);
-#pragma unroll
-        for (int j = 0; j < kTcSlices; ++j) {
-#pragma unroll
-          for (int t = 0; t < NT; ++t) {
-            if (t >= tk.nn) break;
-            unsigned b0, b1;
-            ldsm_x2(b0, b1, sY + j * SL + (8 * tk.nt[t] + (lane & 7)) * kTcStride + k0 + ((lane >> 3) & 1) * 8);
-#pragma unroll
-            for (int i = 0; i + j < kTcSlices; ++i) {
-              const int grp = i + j < 3 ? i + j : 3;
-              mma_bf16(acc[grp][t], A[i], b0, b1);
+            for (int ks = 0; ks < kStage / 16; ++ks) {
+              const unsigned a = a0 + 2 * ks * kOctet, b = b0 + 2 * ks * kOctet;
+              const unsigned acm = !(s == 0 && ar == 0 && ks == 0);
+              // D_t (64 columns each) += (digits 2 u, 2 u + 1 of I) x (digit t - 2 u of J)
+              tc_mma(tmem, tc_desc(a, kOctet), tc_desc(b, kOctet), tc_idesc(256), acm);
+              tc_mma(tmem + 256, tc_desc(a, kOctet), tc_desc(b + 4 * 1024, kOctet), tc_idesc(128), acm);
+              tc_mma(tmem + 128, tc_desc(a + 2048, kOctet), tc_desc(b, kOctet), tc_idesc(256), 1);
+              tc_mma(tmem + 256, tc_desc(a + 4096, kOctet), tc_desc(b, kOctet), tc_idesc(128), 1);
             }
           }
+          tc_commit(empty + 8 * st);
+          if (++st == nstage) {
+            st = 0;
+            par ^= 1;
+          }
+        }
+        tc_commit(done);
+      }
+      // the last commits have to land before the barriers' memory goes away
+      if (mine > 0) mbar_wait(done, (mine - 1) & 1, abort);
+    }
+    __syncwarp();
+  } else {
+    const Ph<double> p = load_ph<double>(A.ph, g);
+    const int octet = warp & 3, sub = lane & 3;  // 8 nodes of the stage, 2 of them this lane's
+    // trial columns of this lane: colgroup (warp >> 2) of block I, and of block J
+    const double2* Xc[2];
+    int Ex[2], Ez[2];
+    bool on[2];
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const int cl = (warp >> 2) * 8 + (lane >> 2), col = (b ? J : I) * kCols + cl;
+      on[b] = b < blocks && col < A.q;
+      Xc[b] = trial_col(A.roles, g, on[b] ? col : 0);
+      Ex[b] = Ez[b] = 0;
+      if (on[b]) {
+        const int e0 = A.E[2 * ((long)g * A.q + col)], e1 = A.E[2 * ((long)g * A.q + col) + 1];
+        on[b] = e0 > kMinExp && e0 < kExpInf;  // zero columns stay zero, non-finite ones are marked at the end
+        Ex[b] = e0;
+        Ez[b] = e1;
+      }
+    }
+    const bool any = __any_sync(0xffffffffu, on[0] || on[1]);
+    int st = 0;
+    unsigned par = 1;  // the ring starts empty
+    auto wait = [&] {
+      mbar_wait(empty + 8 * st, par, abort);
+      return ring0 + st * stage_bytes;
+    };
+    auto ready = [&] {
+      asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+      __syncwarp();
+      if (lane == 0) mbar_arrive(full + 8 * st);
+      if (++st == nstage) {
+        st = 0;
+        par ^= 1;
+      }
+    };
+    const unsigned place = octet * kOctet + (warp >> 2) * 128 + lane * 4;
+    for (int c = 0; c < mine; ++c) {
+      const int t = first + c * A.npart, j0 = t / tx * 8, i = (t - t / tx * tx) * kStage + octet * 8 + sub * 2;
+      if (!any) {
+        for (int s = 0; s < kStages; ++s) {
+          wait();
+          ready();
+        }
+      } else if (mass) {
+        if (diag) produce_chunk<true, 1>(A, Xc, Ex, Ez, on, p, i, j0, place, wait, ready);
+        else produce_chunk<true, 2>(A, Xc, Ex, Ez, on, p, i, j0, place, wait, ready);
+      } else {
+        if (diag) produce_chunk<false, 1>(A, Xc, Ex, Ez, on, p, i, j0, place, wait, ready);
+        else produce_chunk<false, 2>(A, Xc, Ex, Ez, on, p, i, j0, place, wait, ready);
+      }
+      // the chunk's sums: rows 0-63 belong to even digits of I, rows 64-127 to odd ones
+      mbar_wait(done, c & 1, abort);
+      __syncwarp();
+      tc_fence_after();
+      const unsigned ta = tmem + ((unsigned)(warp & 3) << 21) + 16 * (warp >> 2);
+      const bool odd = (warp & 2) != 0;
+      // weights of D_t in the 64-bit sum: 2^(32 - 8 t); on the diagonal odd t count on odd rows
+      // only, halved (their product is symmetric there)
+      for (int t = 0; t < 6; ++t) {
+        float d[16];
+        tc_ld16(ta + 64 * t, d);
+        if (diag && (t & 1) && !odd) continue;
+        const int sh = 32 - 8 * t - (diag && (t & 1) ? 1 : 0);  // t = 5: -8 or -9
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          const long long v = (long long)__float2int_rn(d[k]);
+          acc[k] += sh >= 0 ? (long long)((unsigned long long)v << sh) : (v + (1 << (-sh - 1))) >> -sh;
         }
       }
-      // the groups i + j <= 2 are exact; the rest carries 2^-24 of its (2^-24 smaller) value
-#pragma unroll
-      for (int t = 0; t < NT; ++t) {
-        if (t >= tk.nn) break;
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          const int row = 16 * tk.mt + (lane >> 2) + (k >= 2 ? 8 : 0);
-          const int col = 8 * tk.nt[t] + 2 * (lane & 3) + (k & 1);
-          const float sc = pow2f(ex[row % H] + ey[col % H]);
-#pragma unroll
-          for (int s2 = 0; s2 < 4; ++s2) sum[t][k] = sum[t][k] + df_make(acc[s2][t][k] * sc, 0.0f);
-        }
-      }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(tfree);
     }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == kProducers / 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+  // the sums of the pair as doubles, in the ring's memory: S[half][row 0-63][column 0-63]
+  double* S = reinterpret_cast<double*>(ring);
+  if (warp < kProducers / 32) {
+    const int rr = 32 * (warp & 3) + lane;
+#pragma unroll
+    for (int k = 0; k < 16; ++k) S[rr * 65 + 16 * (warp >> 2) + k] = (double)acc[k];
   }
   __syncthreads();
-  // 5. P in shared memory as FP64, then the partial sums
-  double* Ps = reinterpret_cast<double*>(tc_sm);  // [W2][W2]
-  if (active) {
-#pragma unroll
-    for (int t = 0; t < NT; ++t) {
-      if (t >= tk.nn) break;
-#pragma unroll
-      for (int k = 0; k < 4; ++k) {
-        const int row = 16 * tk.mt + (lane >> 2) + (k >= 2 ? 8 : 0);
-        const int col = 8 * tk.nt[t] + 2 * (lane & 3) + (k & 1);
-        Ps[row * W2 + col] = df_to(sum[t][k]);
-      }
+  const int ne = A.q * (A.q + 1) / 2;
+  double2* out = A.part + ((long)g * A.npart + blockIdx.x) * 2 * ne + (mass ? 0 : ne);
+  const bool bad = *abort != 0;
+  for (int t = tid; t < kCols * kCols; t += kThreads) {
+    const int a = t % kCols, b = t / kCols, ca = I * kCols + a, cb = J * kCols + b;
+    if (ca > cb || cb >= A.q) continue;
+    const int ea = A.E[2 * ((long)g * A.q + ca) + (mass ? 0 : 1)], eb = A.E[2 * ((long)g * A.q + cb) + (mass ? 0 : 1)];
+    auto sum = [&](int r, int c) {
+      const double even = S[r * 65 + c], odd = S[(64 + r) * 65 + c];
+      return even + 0x1p-8 * (diag ? odd + S[(64 + c) * 65 + r] : odd);
+    };
+    double2 v = make_double2(sum(a, b) + sum(32 + a, 32 + b), sum(a, 32 + b) - sum(32 + a, b));
+    if (ea <= kMinExp || eb <= kMinExp) {
+      v = make_double2(0.0, 0.0);
+    } else {
+      const double s = mass ? A.kappa2 : 1.0;
+      v = make_double2(s * scalbn(v.x, ea + eb - 46), s * scalbn(v.y, ea + eb - 46));
     }
+    if (bad || ea == kExpInf || eb == kExpInf) v = make_double2(nan(""), nan(""));
+    out[cb * (cb + 1) / 2 + ca] = v;
   }
-  __syncthreads();
-  const int ne = q * (q + 1) / 2;
-  double2* pm = part + ((long)g * npart + blockIdx.x) * 2 * ne + (prod == 0 ? 0 : ne);
-  for (int e = tid; e < ne; e += nt) {
-    int b = int((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
-    while ((b + 1) * (b + 2) / 2 <= e) ++b;
-    while (b * (b + 1) / 2 > e) --b;
-    const int a = e - b * (b + 1) / 2;
-    const double re = Ps[a * W2 + b] + Ps[(H + a) * W2 + H + b];
-    const double im = Ps[a * W2 + H + b] - Ps[(H + a) * W2 + b];
-    pm[e] = make_double2(re, im);
-  }
-}
-
-// Warp tasks for a padded half width h: the 16-row strips of P and, per strip, the
-// 8-column tiles holding entries a <= b (a < q, b < q) of a block.
-TcTasks make_tasks(int h, int q, int per_task) {
-  TcTasks T{};
-  const int w2 = 2 * h;
-  for (int mt = 0; mt < w2 / 16; ++mt) {
-    const int a0 = (16 * mt) % h;
-    if (a0 >= q) continue;
-    std::vector<int> cols;
-    for (int ntl = 0; ntl < w2 / 8; ++ntl) {
-      const int b0 = (8 * ntl) % h;
-      if (b0 >= q || a0 > b0 + 7) continue;
-      cols.push_back(ntl);
-    }
-    for (size_t s = 0; s < cols.size(); s += per_task) {
-      if (T.count >= kTcMaxTasks) fail(PBS_EINVAL, "tensor-core Gram: too many tiles");
-      TcTask& t = T.t[T.count++];
-      t.mt = (unsigned char)mt;
-      t.nn = (unsigned char)std::min<size_t>(per_task, cols.size() - s);
-      for (int u = 0; u < t.nn; ++u) t.nt[u] = (unsigned char)cols[s + u];
-    }
-  }
-  return T;
-}
-
-template <int H> size_t tc_smem() {
-  const size_t slices = 2ull * kTcSlices * 2 * H * kTcStride * sizeof(__nv_bfloat16);
-  const size_t stage = 2ull * H * kTcRowsGM * sizeof(dcx);
-  const size_t pmat = (size_t)(2 * H) * (2 * H) * sizeof(double);
-  return std::max(slices + stage, pmat);
-}
-
-template <int H, int NT>
-void launch_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
-               cudaStream_t s) {
-  static PerDeviceOnce once;
-  once([] {
-    PBS_CUDA(cudaFuncSetAttribute(k_gram_tc<H, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tc_smem<H>()));
-  });
-  const TcTasks tasks = make_tasks(H, q, NT);
-  k_gram_tc<H, NT><<<dim3(npart, ngroups, 2), 32 * tasks.count, tc_smem<H>(), s>>>(
-      L.lvl<df>(), L.wts_df(), d_ph, roles, q, tasks, d_partials, npart);
 }
 
 }  // namespace
 
-bool gram_tc_supported(int q) { return q >= 1 && q <= kTcMaxHalf; }
+// Partial sums per group: enough CTAs for a few waves of one per SM, at most 128 chunks each (the
+// 64-bit sums then cannot overflow).
+int gram_tc_partials(int n, int m, int q, int ngroups) {
+  const int nb = (q + kCols - 1) / kCols, per = nb * (nb + 1);  // CTAs per group and partial block
+  const long chunks = (long)((n + kStage - 1) / kStage) * ((m + 7) / 8);
+  long np = (4L * 152 + (long)per * ngroups - 1) / ((long)per * ngroups);
+  np = std::max(np, (chunks + 127) / 128);
+  return (int)std::max<long>(1, std::min(np, chunks));
+}
+
+size_t gram_tc_scratch(int q, int ngroups) { return 2 * sizeof(int) * (size_t)q * ngroups; }
 
 void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
-             cudaStream_t s) {
-  if (q <= 16) launch_tc<16, 3>(L, d_ph, roles, q, ngroups, npart, d_partials, s);
-  else if (q <= 32) launch_tc<32, 3>(L, d_ph, roles, q, ngroups, npart, d_partials, s);
-  else if (q <= 48) launch_tc<48, 4>(L, d_ph, roles, q, ngroups, npart, d_partials, s);
-  else fail(PBS_EINVAL, "tensor-core Gram: q > 48");
+             int* d_exps, cudaStream_t s) {
+  static PerDeviceOnce once;
+  once([] { PBS_CUDA(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)); });
+  // every byte 0x80: below -kExpInf
+  PBS_CUDA(cudaMemsetAsync(d_exps, 0x80, gram_tc_scratch(q, ngroups), s));
+  const unsigned tiles = ((L.n + kExpTile - 1) / kExpTile) * ((L.m + kExpTile - 1) / kExpTile);
+  k_gram_exponents<<<dim3(tiles, q, ngroups), kExpThreads, 0, s>>>(L.n, L.m, d_ph, roles, q, L.sw, L.sw_exp, d_exps);
+  PBS_LAUNCHED();
+  // the mass factor relative to kappa, so that |z| < 0.99 times the bound of the edge values
+  const double r3 = 1.0 / std::sqrt(3.0), al = 0.5 * (1.0 + r3), be = 0.5 * (1.0 - r3);
+  const double sx = std::sqrt(L.h2 / L.h1), sy = std::sqrt(L.h1 / L.h2), kappa = std::max(sx, sy) / 0.99;
+  GramArgs a{};
+  a.n = L.n;
+  a.m = L.m;
+  a.N = L.N();
+  a.ax = make_fix(sx * al / kappa);
+  a.bx = make_fix(sx * be / kappa);
+  a.ay = make_fix(sy * al / kappa);
+  a.by = make_fix(sy * be / kappa);
+  a.kappa2 = kappa * kappa;
+  a.sw = L.sw;
+  a.sw_exp = L.sw_exp;
+  a.ph = d_ph;
+  a.roles = roles;
+  a.q = q;
+  a.E = d_exps;
+  a.part = d_partials;
+  a.npart = npart;
+  const int nb = (q + kCols - 1) / kCols;
+  k_gram_tc<<<dim3(npart, ngroups, nb * (nb + 1)), kThreads, kSmem, s>>>(a);
+  PBS_LAUNCHED();
 }
 
 }  // namespace pbs

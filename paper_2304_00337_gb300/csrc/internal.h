@@ -56,7 +56,9 @@ struct Level {
   double* k3_64 = nullptr;   // per node: 6 entries of the inverse 3x3 patch block, SoA [6][N]
   float* k3_32 = nullptr;
   float2* wdf = nullptr;     // level 0: w = (1/eps) / (h1 h2) as double-float (hi, lo) per cell
-  double wmax = 0;           // level 0: the largest w
+  uint2* sw = nullptr;       // level 0: sqrt(w) 2^-sw_exp < 1 per cell in 62-bit fixed point (two 31-bit words)
+  int sw_exp = 0;
+  double wmax = 0, wmin = 0;  // level 0: the largest and smallest w
   long N() const { return (long)n * m; }
   WtsDF wts_df() const { return WtsDF{wdf, n, m}; }
   long D() const { return 2L * n * m; }
@@ -167,6 +169,7 @@ bool verbose_enabled();  // PBS_VERBOSE set in the environment (diagnostic trace
 // first use (run(c) launches candidate c on stream s; candidates are idempotent),
 // then remembered for the process and in the tuning cache file.
 int tune_pick(const std::string& key, int ncand, const std::function<void(int)>& run, cudaStream_t s);
+bool tune_forced(const std::string& key);  // PBS_TUNE_FORCE names a prefix of the key
 std::string device_tag();  // device name and SM count, for tuning keys
 
 // ---- hierarchy set-up (mg.cu) ---------------------------------------------
@@ -290,12 +293,13 @@ struct Roles {
 void gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
                  double2* d_partials, long partial_capacity, bool dfa, cudaStream_t s);
 long gram_partials_size(long rows, int q, int ngroups);  // double2 elements
-// The mixed policy's Gram on the tensor cores (gram_tc.cu): the partial sums of
-// gram_groups' double-float kernel for q <= 48, from bf16 slices (Ozaki splitting).
-bool gram_tc_supported(int q);
-bool gram_on_tensor_cores();  // true when the environment sets PBS_GRAM=tc (then offered first)
+// The mixed policy's Gram on the tensor cores (gram_tc.cu): partial sums in the layout of
+// gram_groups, npart per group; d_exps: gram_tc_scratch bytes.
+bool gram_on_tensor_cores();  // the environment sets PBS_GRAM=tc: every width runs there
+int gram_tc_partials(int n, int m, int q, int ngroups);
+size_t gram_tc_scratch(int q, int ngroups);
 void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
-             cudaStream_t s);
+             int* d_exps, cudaStream_t s);
 // Rayleigh-Ritz in coefficient space for ngroups groups: C (q x p per group), theta (p per
 // group), status in d_info[8 g], scratch small_rr_scratch(q) bytes per group; dfa selects
 // double-float (mixed policy) instead of FP64 arithmetic

@@ -54,8 +54,17 @@ __global__ void k_weights_df(const double* __restrict__ winv, double scale, floa
   w[t] = make_float2(v.hi, v.lo);
 }
 
+// sqrt(w) 2^-ex in 62-bit fixed point (two 31-bit words), w = scale / eps
+__global__ void k_weights_sqrt(const double* __restrict__ winv, double scale, double down, uint2* __restrict__ sw, long N) {
+  const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  if (t >= N) return;
+  const double s = sqrt(scale * winv[t]) * down * 2147483648.0, hi = floor(s);
+  sw[t] = make_uint2((unsigned)hi, (unsigned)((s - hi) * 2147483648.0));
+}
+
 __global__ void k_inv_eps(const double* __restrict__ eps, double* __restrict__ w64, float* __restrict__ w32, long N,
-                          int* __restrict__ bad, unsigned long long* __restrict__ wmax) {
+                          int* __restrict__ bad, unsigned long long* __restrict__ wmax,
+                          unsigned long long* __restrict__ wmin) {
   const long t = blockIdx.x * (long)blockDim.x + threadIdx.x;
   if (t >= N) return;
   const double e = eps[t];
@@ -69,6 +78,7 @@ __global__ void k_inv_eps(const double* __restrict__ eps, double* __restrict__ w
   w32[t] = float(1.0 / e);
   // positive doubles order like their bit patterns
   atomicMax(wmax, (unsigned long long)__double_as_longlong(1.0 / e));
+  atomicMin(wmin, (unsigned long long)__double_as_longlong(1.0 / e));
 }
 
 __global__ void k_coarsen_w(const double* __restrict__ wf, int nf, double* __restrict__ wc, float* __restrict__ wc32,
@@ -413,10 +423,11 @@ int num_levels(int n, int m, int coarsest) {
 void build_hierarchy(DevMem& mem, Hierarchy& H, const double* d_eps, int coarsest, cudaStream_t s) {
   H.nlev = num_levels(H.n, H.m, coarsest);
   if (H.nlev < 1) fail(-1, "invalid mesh for the hierarchy");
-  int* d_bad = (int*)mem.alloc(2 * sizeof(unsigned long long));
+  int* d_bad = (int*)mem.alloc(3 * sizeof(unsigned long long));
   unsigned long long* d_wmax = (unsigned long long*)d_bad + 1;
   H.allocs.push_back(d_bad);
   PBS_CUDA(cudaMemsetAsync(d_bad, 0, 2 * sizeof(unsigned long long), s));
+  PBS_CUDA(cudaMemsetAsync(d_wmax + 1, 0xff, sizeof(unsigned long long), s));
   int n = H.n, m = H.m;
   for (int l = 0; l < H.nlev; ++l) {
     Level& L = H.lev[l];
@@ -431,7 +442,7 @@ void build_hierarchy(DevMem& mem, Hierarchy& H, const double* d_eps, int coarses
     L.k3_32 = (float*)mem.alloc(6 * N * sizeof(float));
     H.allocs.insert(H.allocs.end(), {L.winv64, L.winv32, L.k3_64, L.k3_32});
     if (l == 0) {
-      k_inv_eps<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(d_eps, L.winv64, L.winv32, N, d_bad, d_wmax);
+      k_inv_eps<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(d_eps, L.winv64, L.winv32, N, d_bad, d_wmax, d_wmax + 1);
     } else {
       const Level& F = H.lev[l - 1];
       k_coarsen_w<<<dim3((n + kBX - 1) / kBX, (m + kBY - 1) / kBY), dim3(kBX, kBY), 0, s>>>(F.winv64, F.n, L.winv64,
@@ -441,6 +452,8 @@ void build_hierarchy(DevMem& mem, Hierarchy& H, const double* d_eps, int coarses
     if (l == 0) {
       L.wdf = (float2*)mem.alloc(N * sizeof(float2));
       H.allocs.push_back(L.wdf);
+      L.sw = (uint2*)mem.alloc(N * sizeof(uint2));
+      H.allocs.push_back(L.sw);
       k_weights_df<<<(unsigned)((N + 255) / 256), 256, 0, s>>>(L.winv64, 1.0 / (L.h1 * L.h2), L.wdf, N);
       PBS_LAUNCHED();
     }
@@ -452,13 +465,23 @@ void build_hierarchy(DevMem& mem, Hierarchy& H, const double* d_eps, int coarses
     m /= 2;
   }
   int bad = 0;
-  unsigned long long wmax = 0;
+  unsigned long long wlim[2] = {0, 0};
   PBS_CUDA(cudaMemcpyAsync(&bad, d_bad, sizeof(int), cudaMemcpyDeviceToHost, s));
-  PBS_CUDA(cudaMemcpyAsync(&wmax, d_wmax, sizeof(wmax), cudaMemcpyDeviceToHost, s));
+  PBS_CUDA(cudaMemcpyAsync(wlim, d_wmax, sizeof(wlim), cudaMemcpyDeviceToHost, s));
   PBS_CUDA(cudaStreamSynchronize(s));
   if (bad) fail(-1, "eps must be finite and positive");
-  std::memcpy(&H.winv_max, &wmax, sizeof(double));
-  H.lev[0].wmax = H.winv_max / (H.lev[0].h1 * H.lev[0].h2);
+  std::memcpy(&H.winv_max, &wlim[0], sizeof(double));
+  double winv_min = 0.0;
+  std::memcpy(&winv_min, &wlim[1], sizeof(double));
+  {
+    Level& L = H.lev[0];
+    const double scale = 1.0 / (L.h1 * L.h2);
+    L.wmax = H.winv_max * scale;
+    L.wmin = winv_min * scale;
+    std::frexp(std::sqrt(L.wmax) * (1.0 + 1e-9), &L.sw_exp);  // sqrt(wmax) < 2^sw_exp
+    k_weights_sqrt<<<(unsigned)((L.N() + 255) / 256), 256, 0, s>>>(L.winv64, scale, std::ldexp(1.0, -L.sw_exp), L.sw, L.N());
+    PBS_LAUNCHED();
+  }
   const Level& C = H.lev[H.nlev - 1];
   if (C.D() > kMaxCoarseEdges) fail(-1, "coarsest level too large for the dense solve (raise coarsest or use sides with more factors of 2)");
 }

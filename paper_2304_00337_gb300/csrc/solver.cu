@@ -1275,7 +1275,7 @@ double job_bytes(int n, int m, const pbs_opts& o, int nk, size_t budget) {
   double hb = 0.0;
   for (int l = 0; l < nl; ++l) hb += (double)(n >> l) * (m >> l) * (8 + 4 + 48 + 24);
   const double N = (double)n * m, D = 2.0 * N;
-  hb += 8.0 * N + 8.0 * N;  // level-0 double-float weights, device copy of eps
+  hb += 8.0 * N + 8.0 * N + 8.0 * N;  // level-0 double-float weights, their square roots, device copy of eps
   const double Nc = (double)(n >> (nl - 1)) * (m >> (nl - 1)), Dc = 2.0 * Nc;
   const int G = std::max(1, std::min(o.kbatch, nk)), p = o.block, q = 3 * p;
   const double Gp = (double)G * p;

@@ -138,6 +138,12 @@ std::string device_tag() {
   return name;
 }
 
+bool tune_forced(const std::string& key) {
+  for (const auto& f : forced())
+    if (key.compare(0, f.first.size(), f.first) == 0) return true;
+  return false;
+}
+
 int tune_pick(const std::string& key, int ncand, const std::function<void(int)>& run, cudaStream_t s) {
   if (ncand <= 1) return 0;
   for (const auto& f : forced())
