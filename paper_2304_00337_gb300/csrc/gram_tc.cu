@@ -160,9 +160,9 @@ __device__ __forceinline__ PairY load_y(const double2* __restrict__ Y, int i, in
 // sqrt(w) |curl| < 0.99 2^E (c = g q + column; kExpInf where a value is not finite; very negative
 // for a column of zeros).  A bound needs few bits: the curl is formed in binary32 from the leading
 // 21 bits of its edge values, 2^-18 of which is added to it (the digits then still reach 2^-60 of
-// the edge values, below their FP64 rounding).  A block of edge values outside the binary32 range
-// gives the bound without cancellation.  One pass over the block, bound by memory: 8 rows per thread, two
-// nodes wide, the upper row's x-edges carried to the next.
+// the edge values, below their FP64 rounding).  One pass over the block, bound by memory: 8 rows per
+// thread, two nodes wide, the upper row's x-edges carried to the next; a block whose largest value is
+// outside the middle of the binary32 range walks its tile again relative to that value.
 constexpr int kExpThreads = 256, kExpTile = 64;  // a block's tile: 64 nodes x 64 mesh rows
 __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, const double* __restrict__ ph, Roles roles, int q,
                                                                 const uint2* __restrict__ sw, int sw_exp,
@@ -175,70 +175,75 @@ __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, co
   const Ph<double> p = load_ph<double>(ph, g);
   const int i = bx * kExpTile + 2 * lane, j0 = by * kExpTile + 8 * (tid >> 5);
   const bool in = i < n;
-  int top = 0;          // largest high word (sign off): the exponent of the largest value
-  float cmax = 0.0f;    // largest 2^-sw_exp sqrt(w) (|c| + 2^-18 of the values), binary32 range only
-  auto lead = [&](double d) {
-    const int hi = __double2hiint(d), a = hi & 0x7FFFFFFF;
-    top = max(top, a);
-    const int f = a < (900 << 20) ? 0 : (a - (896 << 20)) << 3;
-    return __int_as_float((hi & 0x80000000) | f);
-  };
-  float x0[2][2];
-  {
-    const PairX v = load_x(X, i, j0, n, m, p.be, in && j0 < m);
+  int base = 896, hi = 0, cb = 0;  // binary64 exponent field that becomes binary32's 0
+  for (int pass = 0; pass < 2; ++pass) {
+    int top = 0;        // largest high word (sign off): the exponent of the largest value
+    float cmax = 0.0f;  // largest 2^-sw_exp sqrt(w) (|c| + 2^-18 of the values), relative to 2^(base - 896)
+    auto lead = [&](double d) {
+      const int h = __double2hiint(d), a = h & 0x7FFFFFFF;
+      top = max(top, a);
+      const int f = a < ((base + 4) << 20) ? 0 : (a - (base << 20)) << 3;
+      return __int_as_float((h & 0x80000000) | f);
+    };
+    float x0[2][2];
+    {
+      const PairX v = load_x(X, i, j0, n, m, p.be, in && j0 < m);
 #pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      x0[k][0] = lead(v.v[k].x);
-      x0[k][1] = lead(v.v[k].y);
-    }
-  }
-  for (int j = j0; j < min(j0 + 8, m); ++j) {
-    const PairX v = load_x(X, i, j + 1, n, m, p.be, in);
-    const PairY u = load_y(Y, i, j, n, p.al, in);
-    float y[3][2];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      y[k][0] = lead(u.v[k].x);
-      y[k][1] = lead(u.v[k].y);
-    }
-#pragma unroll
-    for (int k = 0; k < 2; ++k) {
-      const float s = in ? (float)sw[(long)j * n + i + k].x : 0.0f;
-#pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const float x1 = lead(c ? v.v[k].y : v.v[k].x);
-        const float d = fabsf((x1 - x0[k][c]) - (y[k + 1][c] - y[k][c]));
-        const float e = fmaxf(fmaxf(fabsf(x1), fabsf(x0[k][c])), fmaxf(fabsf(y[k + 1][c]), fabsf(y[k][c])));
-        cmax = fmaxf(cmax, s * fmaf(e, 0x1p-18f, d));
-        x0[k][c] = x1;
+      for (int k = 0; k < 2; ++k) {
+        x0[k][0] = lead(v.v[k].x);
+        x0[k][1] = lead(v.v[k].y);
       }
     }
+    for (int j = j0; j < min(j0 + 8, m); ++j) {
+      const PairX v = load_x(X, i, j + 1, n, m, p.be, in);
+      const PairY u = load_y(Y, i, j, n, p.al, in);
+      float y[3][2];
+#pragma unroll
+      for (int k = 0; k < 3; ++k) {
+        y[k][0] = lead(u.v[k].x);
+        y[k][1] = lead(u.v[k].y);
+      }
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const float s = in ? (float)sw[(long)j * n + i + k].x : 0.0f;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+          const float x1 = lead(c ? v.v[k].y : v.v[k].x);
+          const float d = fabsf((x1 - x0[k][c]) - (y[k + 1][c] - y[k][c]));
+          const float e = fmaxf(fmaxf(fabsf(x1), fabsf(x0[k][c])), fmaxf(fabsf(y[k + 1][c]), fabsf(y[k][c])));
+          cmax = fmaxf(cmax, s * fmaf(e, 0x1p-18f, d));
+          x0[k][c] = x1;
+        }
+      }
+    }
+    // high words order like the values, bits of non-negative floats too
+    const int t = __reduce_max_sync(0xffffffffu, top);
+    const int c = __reduce_max_sync(0xffffffffu, __float_as_int(cmax));
+    if (lane == 0) {
+      red[0][tid >> 5] = t;
+      red[1][tid >> 5] = c;
+    }
+    __syncthreads();
+    hi = cb = 0;
+    for (int w = 0; w < kExpThreads / 32; ++w) {
+      hi = max(hi, red[0][w]);
+      cb = max(cb, red[1][w]);
+    }
+    const int e = hi >> 20;
+    if (e == 0 || e == 0x7FF || (e >= 960 && e <= 1080)) break;
+    base = e - 127;
+    __syncthreads();
   }
-  // high words order like the values, bits of non-negative floats too
-  const int t = __reduce_max_sync(0xffffffffu, top);
-  const int c = __reduce_max_sync(0xffffffffu, __float_as_int(cmax));
-  if (lane == 0) {
-    red[0][tid >> 5] = t;
-    red[1][tid >> 5] = c;
-  }
-  __syncthreads();
   if (tid != 0) return;
-  int hi = 0, cb = 0;
-  for (int w = 0; w < kExpThreads / 32; ++w) {
-    hi = max(hi, red[0][w]);
-    cb = max(cb, red[1][w]);
-  }
   const int e = hi >> 20;
   if (e == 0) return;
   int ex = e - 1022, ez;
   if (e == 0x7FF) {
     ex = ez = kExpInf;
-  } else if (e < 920 || e > 1140) {
-    ez = ex + sw_exp + 3;  // |c| <= 4 2^ex
   } else {
     // sw holds 31 bits; 2 % for the roundings and the margin; a block without curl counts as tiny
     const float v = __int_as_float(cb) * (1.02f * 0x1p-31f);
-    ez = v > 0.0f ? ilogbf(v) + 1 + sw_exp : ex + sw_exp - 18;
+    ez = v > 0.0f ? ilogbf(v) + 1 + sw_exp + base - 896 : ex + sw_exp - 18;
   }
   int* Ec = E + 2 * ((long)g * q + col);
   atomicMax(Ec, ex);
