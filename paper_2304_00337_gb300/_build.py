@@ -16,7 +16,7 @@ CSRC = os.path.join(PKG, "csrc")
 INCLUDE = os.path.join(ROOT, "include")
 BUILD = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libpbs.so")
-SOURCES = ["ops.cu", "mg.cu", "dense.cu", "gram_tc.cu", "solver.cu", "householder.cu", "tune.cu"]
+SOURCES = ["ops.cu", "mg.cu", "dense.cu", "gram_tc.cu", "update_tc.cu", "solver.cu", "householder.cu", "tune.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-Xcompiler", "-fvisibility=hidden",
          "--expt-relaxed-constexpr", f"-I{INCLUDE}", f"-I{CSRC}"]

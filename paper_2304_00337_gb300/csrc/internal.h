@@ -290,8 +290,10 @@ struct Roles {
 };
 // Per group g (phases from entry g of d_ph): GM_g = S^* M S, GA_g = (C S)^* W (C S), q x q
 // column-major at GM + g q^2, GA + g q^2.
-void gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
-                 double2* d_partials, long partial_capacity, bool dfa, cudaStream_t s);
+// Returns the exponents of the trial columns (entry 2 (g q + a): |x| < 2^e over column a of group g) if
+// the tensor-core kernel ran, else null; they lie in d_partials, valid until that is written again.
+const int* gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
+                       double2* d_partials, long partial_capacity, bool dfa, cudaStream_t s);
 long gram_partials_size(long rows, int q, int ngroups);  // double2 elements
 // The mixed policy's Gram on the tensor cores (gram_tc.cu): partial sums in the layout of
 // gram_groups, npart per group; d_exps: gram_tc_scratch bytes.
@@ -307,9 +309,16 @@ void small_rr(const double2* GM, const double2* GA, int q, int p, double2* C, do
               int* d_info, int ngroups, bool dfa, cudaStream_t s);
 size_t small_rr_scratch(int q);
 // Y_g[:, j] = sum_i X_g[:, i] C_g[i, j] (+ Z_g[:, j]) for each group
-// (dfa: double-float, for the search direction only; the iterate's update is FP64)
+// (dfa: double-float, for the search direction only; the iterate's update is FP64); d_exps, where
+// given: the columns' exponents, for the tensor cores
 void block_update(Roles X, int q, const double2* C, int ldc, long cgs, double2* Y, long ldy, int p,
-                  const double2* Z, long ldz, long rows, int ngroups, bool dfa, cudaStream_t s);
+                  const double2* Z, long ldz, long rows, int ngroups, bool dfa, const int* d_exps, int egs,
+                  cudaStream_t s);
+// The same on the tensor cores (update_tc.cu): d_exps from gram_groups, the exponent of trial column i of
+// group g at d_exps[g egs + 2 i]; `slices` CTAs per group (the result does not depend on it).
+bool update_tc_takes(int q, int p);
+void update_tc(Roles X, int q, const double2* C, int ldc, long cgs, const int* d_exps, int egs, double2* Y, long ldy, int p,
+               const double2* Z, long ldz, long rows, int ngroups, int slices, cudaStream_t s);
 void random_block(double2* X, long ld, long rows, int ncols, uint64_t seed, cudaStream_t s);
 
 // ---- generalised Householder orthonormalisation (householder.cu) ----------
