@@ -11,12 +11,13 @@
 #include "df32.cuh"
 #include "internal.h"
 #include "mgpoint.cuh"
+#include "strips.cuh"
 
 namespace pbs {
 
 namespace {
 
-constexpr int kBX = 32, kBY = 8, kThreads = kBX * kBY;
+constexpr int kBX = 32, kBY = 8;
 
 inline dim3 grid2(int n, int m, int ncols) { return dim3((n + kBX - 1) / kBX, (m + kBY - 1) / kBY, ncols); }
 
@@ -46,30 +47,6 @@ __device__ __forceinline__ void block_sum2(double& a, double& b) {
 
 __device__ __forceinline__ df shfl_df(df v, int o) {
   return df_make(__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o));
-}
-
-// Block-wide sum of two double-floats (fixed order); result valid in thread 0.
-__device__ __forceinline__ void block_sum2(df& a, df& b) {
-  __shared__ df sa[32], sb[32];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, lane = tid & 31, wid = tid >> 5;
-  for (int o = 16; o > 0; o >>= 1) {
-    a = a + df_make(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o));
-    b = b + df_make(__shfl_xor_sync(0xffffffffu, b.hi, o), __shfl_xor_sync(0xffffffffu, b.lo, o));
-  }
-  if (lane == 0) {
-    sa[wid] = a;
-    sb[wid] = b;
-  }
-  __syncthreads();
-  const int nw = (blockDim.x * blockDim.y + 31) >> 5;
-  if (wid == 0) {
-    a = lane < nw ? sa[lane] : df_zero();
-    b = lane < nw ? sb[lane] : df_zero();
-    for (int o = 16; o > 0; o >>= 1) {
-      a = a + df_make(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o));
-      b = b + df_make(__shfl_xor_sync(0xffffffffu, b.hi, o), __shfl_xor_sync(0xffffffffu, b.lo, o));
-    }
-  }
 }
 
 // partials: [ncols][nblk][2] -> out [ncols][2], fixed order
@@ -107,35 +84,22 @@ MassFactor mass_factor(const Level& L) {
 // The kernels below read and write FP64 blocks; V is the arithmetic: double
 // (plain FP64) or df (double-float on the FP32 pipe, about 2^-47 relative).
 
-template <class V, class W>
-__global__ void k_rayleigh_parts(Lvl<V> L, W w, MassFactor mf, const double* ph, int cpg,
-                                 const double2* __restrict__ X, long ld, double* __restrict__ part) {
+__global__ void k_rayleigh_parts(Lvl<double> L, Wts<double> w, const double* ph, int cpg, const double2* __restrict__ X,
+                                 long ld, double* __restrict__ part) {
   const int i = blockIdx.x * kBX + threadIdx.x, j = blockIdx.y * kBY + threadIdx.y, c = blockIdx.z;
-  V den = V(0.0), num = V(0.0);
-  if constexpr (std::is_same<V, df>::value) {
-    // double-float: e^* M e = |z_x|^2 + |z_y|^2 (factored mass), and plain reads where
-    // the stencil stays inside the level
-    const auto parts = [&](const auto& r) {
-      const dcx x0 = r.x(i, j), x1 = r.x(i, j + 1), y0 = r.y(i, j), y1 = r.y(i + 1, j);
-      den = nrm2(mf.ax * x0 + mf.bx * x1) + nrm2(mf.ay * y0 + mf.by * y1);
-      num = w(i, j) * nrm2(x1 - x0 - y1 + y0);  // curl_at's order
-    };
-    if (i < L.n && j < L.m) {
-      if (inside(i, j, L.n, L.m, 1, 1)) parts(ERdDIn<df>{X + c * ld, L.n, (long)L.n * L.m});
-      else parts(ERdD<df>{X + c * ld, L.n, L.m, load_ph<df>(ph, c / cpg)});
-    }
-  } else if (i < L.n && j < L.m) {
-    const ERdD<V> r{X + c * ld, L.n, L.m, load_ph<V>(ph, c / cpg)};
-    const cx<V> mx = M_x<V>(r, L, i, j), my = M_y<V>(r, L, i, j);
-    const cx<V> ex = r.x(i, j), ey = r.y(i, j);
+  double den = 0.0, num = 0.0;
+  if (i < L.n && j < L.m) {
+    const ERdD<double> r{X + c * ld, L.n, L.m, load_ph<double>(ph, c / cpg)};
+    const double2 mx = M_x<double>(r, L, i, j), my = M_y<double>(r, L, i, j);
+    const double2 ex = r.x(i, j), ey = r.y(i, j);
     den = ex.x * mx.x + ex.y * mx.y + ey.x * my.x + ey.y * my.y;
-    num = w(i, j) * nrm2(curl_at<V>(r, i, j));
+    num = w(i, j) * nrm2(curl_at<double>(r, i, j));
   }
   block_sum2(den, num);
   if (threadIdx.x == 0 && threadIdx.y == 0) {
     const int nblk = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
-    part[((long)c * nblk + b) * 2] = to_double(den);
-    part[((long)c * nblk + b) * 2 + 1] = to_double(num);
+    part[((long)c * nblk + b) * 2] = den;
+    part[((long)c * nblk + b) * 2 + 1] = num;
   }
 }
 
@@ -261,94 +225,19 @@ __global__ void __launch_bounds__(kBX * kBY) k_residual(Lvl<double> L, Wts<doubl
   }
 }
 
-// The same residual for the mixed policy, whose preconditioner reads it in FP32.
-// The curls c = x(i,j+1) - x(i,j) - y(i+1,j) + y(i,j) are formed in FP64: they are
-// where the stencil cancels (neighbouring values of a smooth iterate nearly agree),
-// and their FP64 rounding is the floor every policy shares.  Everything after them -
-// H = w c, the differences of H, the mass stencil and R = A e - lambda M e - is
-// double-float: those steps see the curls and the iterate's values themselves, so a
-// relative rounding of 2^-47 there moves the relative residual by about 2^-47 (H
-// differences: 2^-47 sqrt(lambda_max / lambda), 1e-10 next to Gamma at 1024^2), far
-// below any tolerance.  R is stored rounded to FP32 and the norms |R|^2, |M e|^2 are
-// summed per thread in FP32 and across the block in FP64 (the convergence test needs
-// a few digits of them).  FP64 work: the curls only (about 7 operations per node
-// against about 45 in the all-FP64 kernel).
-template <class Rd>
-__device__ __forceinline__ void residual_tile_mixed(const Lvl<df>& L, const WtsDF& w, const Rd& r, df l,
-                                                    float2* __restrict__ Rc, double& rr, double& mm) {
-  __shared__ dcx Hs[kBY + 1][kBX + 1];  // cell (i0 - 1 + a, j0 - 1 + b) at Hs[b][a]
-  const int tx = threadIdx.x, ty = threadIdx.y;
-  const int i0 = blockIdx.x * kBX, j0 = blockIdx.y * kBY;
-  const int i = i0 + tx, j = j0 + ty;
-  const bool in = i < L.n && j < L.m;
-  if (in) Hs[ty + 1][tx + 1] = w(i, j) * dcx_split(curl_at<double>(r, i, j));
-  if (ty == 0 && i < L.n) Hs[0][tx + 1] = w(i, j0 - 1) * dcx_split(curl_at<double>(r, i, j0 - 1));
-  if (tx == 0 && j < L.m) Hs[ty + 1][0] = w(i0 - 1, j) * dcx_split(curl_at<double>(r, i0 - 1, j));
-  __syncthreads();
-  if (in) {
-    const df sx = L.mx * df(1.0 / 6.0), sy = L.my * df(1.0 / 6.0), four = df(4.0);
-    const dcx x0 = dcx_split(r.x(i, j)), x1 = dcx_split(r.x(i, j + 1)), x2 = dcx_split(r.x(i, j - 1));
-    const dcx y0 = dcx_split(r.y(i, j)), y1 = dcx_split(r.y(i + 1, j)), y2 = dcx_split(r.y(i - 1, j));
-    const dcx mx = sx * (four * x0 + (x1 + x2));
-    const dcx my = sy * (four * y0 + (y1 + y2));
-    const dcx h = Hs[ty + 1][tx + 1], hb = Hs[ty][tx + 1], hl = Hs[ty + 1][tx];
-    const dcx rx = (hb - h) - l * mx;
-    const dcx ry = (h - hl) - l * my;
-    const long N = (long)L.n * L.m, e = (long)j * L.n + i;
-    const float2 fx = make_float2(df_to_float(rx.x), df_to_float(rx.y));
-    const float2 fy = make_float2(df_to_float(ry.x), df_to_float(ry.y));
-    Rc[e] = fx;
-    Rc[N + e] = fy;
-    const float r2 = fmaf(fx.x, fx.x, fmaf(fx.y, fx.y, fmaf(fy.x, fy.x, fy.y * fy.y)));
-    const float mxf = df_to_float(mx.x), mxi = df_to_float(mx.y), myf = df_to_float(my.x), myi = df_to_float(my.y);
-    const float m2 = fmaf(mxf, mxf, fmaf(mxi, mxi, fmaf(myf, myf, myi * myi)));
-    rr = f2d_exact(r2);
-    mm = f2d_exact(m2);
-  }
-}
-
-__global__ void __launch_bounds__(kBX * kBY) k_residual_mixed(Lvl<df> L, WtsDF w, const double* ph, int cpg,
-                                                               const double2* __restrict__ E, float2* __restrict__ R,
-                                                               long ld, const double* __restrict__ lam,
-                                                               double* __restrict__ part) {
-  const int i0 = blockIdx.x * kBX, j0 = blockIdx.y * kBY, c = blockIdx.z;
-  double rr = 0, mm = 0;
-  const df l = df_split(lam[c]);
-  if (i0 >= 1 && j0 >= 1 && i0 + kBX < L.n && j0 + kBY < L.m) {
-    residual_tile_mixed(L, w, ERdIn<double>{E + c * ld, L.n, (long)L.n * L.m}, l, R + c * ld, rr, mm);
-  } else {
-    constexpr int WX = kBX + 1, WY = kBX + 2;
-    __shared__ double2 sx[(kBY + 2) * WX], sy[(kBY + 1) * WY];
-    const int nx = min(kBX, L.n - i0), ny = min(kBY, L.m - j0);
-    const Ph<double> p = load_ph<double>(ph, c / cpg);
-    const double2* Ec = E + c * ld;
-    stage_field(Ec, L.n, L.m, p, i0, j0, WX, kBY + 2, nx, ny + 1, sx);
-    stage_field(Ec + (long)L.n * L.m, L.n, L.m, p, i0, j0, WY, kBY + 1, nx + 1, ny, sy);
-    __syncthreads();
-    residual_tile_mixed(L, w, TileERd<double>{sx, sy, i0 - 1, j0 - 1, WX, WY}, l, R + c * ld, rr, mm);
-  }
-  block_sum2(rr, mm);
-  if (threadIdx.x == 0 && threadIdx.y == 0) {
-    const int nblk = gridDim.x * gridDim.y, b = blockIdx.y * gridDim.x + blockIdx.x;
-    part[((long)c * nblk + b) * 2] = rr;
-    part[((long)c * nblk + b) * 2 + 1] = mm;
-  }
-}
-
 // rhs(i,j) = (L^* M x)(i,j) = (Mx)_x(i-1,j) - (Mx)_x(i,j) + (Mx)_y(i,j-1) - (Mx)_y(i,j),
-// computed in V and stored in T.  A CTA stages the edge values its 32 x 8 nodes
-// read (converted to V once), forms each mass-stencil value once in shared
+// in FP64, stored in T.  A CTA stages the edge values its 32 x 8 nodes read, forms each mass-stencil value once in shared
 // memory, then combines them; the stencil functions and the order of the sums
 // are those of the per-node formula.
-template <class V, class T>
-__global__ void __launch_bounds__(kBX * kBY) k_lift_adj_mass(Lvl<V> L, const double* ph, int cpg,
+template <class T>
+__global__ void __launch_bounds__(kBX * kBY) k_lift_adj_mass(Lvl<double> L, const double* ph, int cpg,
                                                              const double2* __restrict__ X, long ldx,
                                                              cx<T>* __restrict__ Y, long ldy) {
   constexpr int WX = kBX + 1, WY = kBX + 2;
-  __shared__ cx<V> sx[(kBY + 2) * WX];  // x-edges (i0 - 1 + a, j0 - 1 + b)
-  __shared__ cx<V> sy[(kBY + 1) * WY];  // y-edges (i0 - 1 + a, j0 - 1 + b)
-  __shared__ cx<V> mxs[kBY * WX];       // (Mx)_x(i0 - 1 + a, j0 + b)
-  __shared__ cx<V> mys[(kBY + 1) * kBX];  // (Mx)_y(i0 + a, j0 - 1 + b)
+  __shared__ double2 sx[(kBY + 2) * WX];  // x-edges (i0 - 1 + a, j0 - 1 + b)
+  __shared__ double2 sy[(kBY + 1) * WY];  // y-edges (i0 - 1 + a, j0 - 1 + b)
+  __shared__ double2 mxs[kBY * WX];       // (Mx)_x(i0 - 1 + a, j0 + b)
+  __shared__ double2 mys[(kBY + 1) * kBX];  // (Mx)_y(i0 + a, j0 - 1 + b)
   const int i0 = blockIdx.x * kBX, j0 = blockIdx.y * kBY, c = blockIdx.z;
   const int tid = threadIdx.y * kBX + threadIdx.x, nt = kBX * kBY;
   const int nx = min(kBX, L.n - i0), ny = min(kBY, L.m - j0);  // nodes of the tile inside the level
@@ -357,11 +246,11 @@ __global__ void __launch_bounds__(kBX * kBY) k_lift_adj_mass(Lvl<V> L, const dou
   // the values the tile's nodes read: x-edges a <= nx, b <= ny + 1; y-edges a <= nx + 1, b <= ny
   if (i0 >= 1 && j0 >= 1 && i0 + kBX < L.n && j0 + kBY < L.m) {
     for (int t = tid; t < (kBY + 2) * WX; t += nt)
-      sx[t] = ld_as<V>(xc + (long)(j0 - 1 + t / WX) * L.n + (i0 - 1 + t % WX));
+      sx[t] = xc[ (long)(j0 - 1 + t / WX) * L.n + (i0 - 1 + t % WX)];
     for (int t = tid; t < (kBY + 1) * WY; t += nt)
-      sy[t] = ld_as<V>(xc + N + (long)(j0 - 1 + t / WY) * L.n + (i0 - 1 + t % WY));
+      sy[t] = xc[ N + (long)(j0 - 1 + t / WY) * L.n + (i0 - 1 + t % WY)];
   } else {
-    const ERdD<V> r{xc, L.n, L.m, load_ph<V>(ph, c / cpg)};
+    const ERdD<double> r{xc, L.n, L.m, load_ph<double>(ph, c / cpg)};
     for (int t = tid; t < (kBY + 2) * WX; t += nt) {
       const int a = t % WX, b = t / WX;
       if (a <= nx && b <= ny + 1) sx[t] = r.x(i0 - 1 + a, j0 - 1 + b);
@@ -372,19 +261,19 @@ __global__ void __launch_bounds__(kBX * kBY) k_lift_adj_mass(Lvl<V> L, const dou
     }
   }
   __syncthreads();
-  const TileERd<V> tr{sx, sy, i0 - 1, j0 - 1, WX, WY};
+  const TileERd<double> tr{sx, sy, i0 - 1, j0 - 1, WX, WY};
   for (int t = tid; t < kBY * WX; t += nt) {
     const int a = t % WX, b = t / WX;
-    if (a <= nx && b < ny) mxs[t] = M_x<V>(tr, L, i0 - 1 + a, j0 + b);
+    if (a <= nx && b < ny) mxs[t] = M_x<double>(tr, L, i0 - 1 + a, j0 + b);
   }
   for (int t = tid; t < (kBY + 1) * kBX; t += nt) {
     const int a = t % kBX, b = t / kBX;
-    if (a < nx && b <= ny) mys[t] = M_y<V>(tr, L, i0 + a, j0 - 1 + b);
+    if (a < nx && b <= ny) mys[t] = M_y<double>(tr, L, i0 + a, j0 - 1 + b);
   }
   __syncthreads();
   const int a = threadIdx.x, b = threadIdx.y;
   if (a >= nx || b >= ny) return;
-  const cx<V> v = mxs[b * WX + a] - mxs[b * WX + a + 1] + mys[b * kBX + a] - mys[(b + 1) * kBX + a];
+  const double2 v = mxs[b * WX + a] - mxs[b * WX + a + 1] + mys[b * kBX + a] - mys[(b + 1) * kBX + a];
   Y[c * ldy + (long)(j0 + b) * L.n + i0 + a] = mk<T>(narrow<T>(v.x), narrow<T>(v.y));
 }
 
@@ -1634,12 +1523,14 @@ void lift_adj_mass(const Level& L, const double* d_ph, int cpg, const double2* X
                    int ncols, bool dfa, cudaStream_t s) {
   if (ncols <= 0) return;
   timer_begin(KC_LIFT_ADJ_MASK, s, (16.0 * L.D() + 2.0 * sizeof(T) * L.N()) * ncols);
-  const dim3 g = grid2(L.n, L.m, ncols);
   if (dfa) {
-    k_lift_adj_mass<df, T><<<g, dim3(kBX, kBY), 0, s>>>(L.lvl<df>(), d_ph, cpg, X, ldx, Rhs, ldr);
+    const int rows = strip_rows(L.n, L.m);
+    k_lift_adj_mass_strips<T><<<dim3(strip_blocks<30>(L.n, L.m, rows), ncols), 32 * kStripWarps, 0, s>>>(
+        L.lvl<df>(), d_ph, cpg, X, ldx, Rhs, ldr, rows);
     count_df_launch();
-  } else
-    k_lift_adj_mass<double, T><<<g, dim3(kBX, kBY), 0, s>>>(L.lvl<double>(), d_ph, cpg, X, ldx, Rhs, ldr);
+  } else {
+    k_lift_adj_mass<T><<<grid2(L.n, L.m, ncols), dim3(kBX, kBY), 0, s>>>(L.lvl<double>(), d_ph, cpg, X, ldx, Rhs, ldr);
+  }
   timer_end(KC_LIFT_ADJ_MASK, s);
   PBS_LAUNCHED();
 }
@@ -1658,28 +1549,30 @@ void rayleigh_parts(const Level& L, const double* d_ph, int cpg, const double2* 
                     double* d_partials, double* d_out, bool dfa, cudaStream_t s) {
   if (ncols <= 0) return;
   const dim3 g = grid2(L.n, L.m, ncols);
+  const int rows = strip_rows(L.n, L.m), nblk = dfa ? (int)strip_blocks<31>(L.n, L.m, rows) : (int)(g.x * g.y);
   if (dfa) {
-    k_rayleigh_parts<df><<<g, dim3(kBX, kBY), 0, s>>>(L.lvl<df>(), L.wts_df(), mass_factor(L), d_ph, cpg, X, ld,
-                                                     d_partials);
+    k_rayleigh_strips<<<dim3(nblk, ncols), 32 * kStripWarps, 0, s>>>(L.lvl<df>(), L.wts_df(), d_ph, cpg, X, ld, rows,
+                                                                      d_partials);
     count_df_launch();
-  } else
-    k_rayleigh_parts<double><<<g, dim3(kBX, kBY), 0, s>>>(L.lvl<double>(), L.wts<double>(), mass_factor(L), d_ph,
-                                                         cpg, X, ld, d_partials);
+  } else {
+    k_rayleigh_parts<<<g, dim3(kBX, kBY), 0, s>>>(L.lvl<double>(), L.wts<double>(), d_ph, cpg, X, ld, d_partials);
+  }
   PBS_LAUNCHED();
-  k_finalize2<<<ncols, 256, 0, s>>>(d_partials, g.x * g.y, d_out);
+  k_finalize2<<<ncols, 256, 0, s>>>(d_partials, nblk, d_out);
   PBS_LAUNCHED();
 }
 
 void residual_mixed(const Level& L, const double* d_ph, int cpg, const double2* E, float2* R, long ld, int ncols,
                     const double* d_lam, double* d_partials, double* d_out, cudaStream_t s) {
   if (ncols <= 0) return;
-  const dim3 g = grid2(L.n, L.m, ncols);
+  const int rows = strip_rows(L.n, L.m), nblk = (int)strip_blocks<30>(L.n, L.m, rows);
   timer_begin(KC_RESIDUAL, s, 24.0 * L.D() * ncols);  // read E (16 B), write R (8 B) per edge DOF
-  k_residual_mixed<<<g, dim3(kBX, kBY), 0, s>>>(L.lvl<df>(), L.wts_df(), d_ph, cpg, E, R, ld, d_lam, d_partials);
+  k_residual_strips<<<dim3(nblk, ncols), 32 * kStripWarps, 0, s>>>(L.lvl<df>(), L.wts_df(), d_ph, cpg, E, R, ld, d_lam, rows,
+                                                                    d_partials);
   timer_end(KC_RESIDUAL, s);
   PBS_LAUNCHED();
   count_df_launch();
-  k_finalize2<<<ncols, 256, 0, s>>>(d_partials, g.x * g.y, d_out);
+  k_finalize2<<<ncols, 256, 0, s>>>(d_partials, nblk, d_out);
   PBS_LAUNCHED();
 }
 
