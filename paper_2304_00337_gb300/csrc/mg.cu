@@ -36,6 +36,7 @@
 
 #include "internal.h"
 #include "mgpoint.cuh"
+#include "node_strips.cuh"
 #include "nodal_tiles.cuh"
 #include "tail.cuh"
 
@@ -905,32 +906,27 @@ template <class T, int FT> void set_fine_smem() {
                                   (int)fine_smem_cap([](int nu) { return fine_up_smem<T>(FT, nu); })));
   });
 }
-// shared memory of the register-blocked steps (FP32, one sweep per side)
-template <int FT, int NT> void set_fine_rb_smem() {
-  static PerDeviceOnce once;
-  once([] {
-    PBS_CUDA(cudaFuncSetAttribute(k_node_down_rb<FT, NT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)RbDown<FT, NT, 1>::smem));
-    PBS_CUDA(cudaFuncSetAttribute(k_node_up_rb<FT, NT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)RbUp<FT, NT, 1>::smem));
-  });
-}
-// launch shapes of the tiled steps offered to the autotuner: (tile side, threads,
-// register-blocked); the first one fits every level the tiled path takes, the
-// register-blocked ones run FP32 cycles with one sweep per side
+// launch shapes of the fine-level steps offered to the autotuner.  Cycles with one sweep per side run as
+// row strips (ft rows, nt = 0), the others as tiles (side ft, nt threads).  One GB300, down + up step
+// in us, strips of 16 / 32 / 64 rows against the best tile: FP32, 40 columns: 1024 x 1024 449 / 438 /
+// 437, 846; 512 x 512 139 / 146 / 174, 234; 256 x 256 42 / 40 / 57, 65; 128 x 128 24 / 31 / 51, 29;
+// FP64, 20 columns: 512 x 512 1107 / 1160 / 1147, 1549; 128 x 128 121 / 219 / 413, 189.  The first
+// shape fits every level this path takes.
 struct FineShape {
   int ft, nt;
-  bool rb;
 };
-constexpr FineShape kFineShapes[] = {{32, 256, false}, {64, 512, false}, {64, 256, false},
-                                     {32, 256, true},  {64, 512, true},  {32, 128, true}};
-constexpr int kNumFineShapes = 6;
+constexpr FineShape kStripShapes[] = {{16, 0}, {32, 0}, {64, 0}};
+constexpr FineShape kTileShapes[] = {{32, 256}, {64, 512}, {64, 256}};
+constexpr int kNumFineShapes = 3;
 template <class T>
 int fine_shapes(const Level& L, int nu, bool down, FineShape* out) {
   int n = 0;
-  for (const FineShape& f : kFineShapes) {
-    if (f.rb && (!std::is_same<T, float>::value || nu != 1)) continue;
-    const size_t sm = f.rb ? 0 : down ? fine_down_smem<T>(f.ft, nu) : fine_up_smem<T>(f.ft, nu);
+  if (nu == 1) {
+    for (const FineShape& f : kStripShapes) out[n++] = f;
+    return n;
+  }
+  for (const FineShape& f : kTileShapes) {
+    const size_t sm = down ? fine_down_smem<T>(f.ft, nu) : fine_up_smem<T>(f.ft, nu);
     if (fine_fits(L, f.ft) && sm <= kSmemOptIn) out[n++] = f;
   }
   return n;
@@ -968,45 +964,25 @@ void launch_node_up(const Level& L, const Level& C, const KData& K, MgWork<T>& w
   PBS_LAUNCHED();
 }
 
-template <int FT, int NT>
-void launch_node_down_rb(const Level& L, const Level& C, const KData& K, MgWork<float>& w, int l, const float2* b,
-                         const float2* x0, long ld, int ncols, int cpg, cudaStream_t s) {
-  set_fine_rb_smem<FT, NT>();
-  const dim3 grid((L.n + FT - 1) / FT, (L.m + FT - 1) / FT, ncols);
-  k_node_down_rb<FT, NT, 1><<<grid, NT, RbDown<FT, NT, 1>::smem, s>>>(L.lvl<float>(), C.n, C.m, K.d_ph, cpg, b, ld,
-                                                                      x0, ld, w.r[l], L.N(), w.b[l + 1], C.N());
-  PBS_LAUNCHED();
-}
-
-template <int FT, int NT>
-void launch_node_up_rb(const Level& L, const Level& C, const KData& K, MgWork<float>& w, int l, const float2* b,
-                       float2* x, long ld, int ncols, int cpg, cudaStream_t s) {
-  set_fine_rb_smem<FT, NT>();
-  const dim3 grid((L.n + FT - 1) / FT, (L.m + FT - 1) / FT, ncols);
-  k_node_up_rb<FT, NT, 1><<<grid, NT, RbUp<FT, NT, 1>::smem, s>>>(L.lvl<float>(), C.n, C.m, K.d_ph, cpg, b, ld,
-                                                                  w.r[l], L.N(), w.x[l + 1], C.N(), x, ld);
-  PBS_LAUNCHED();
-}
-
-// the register-blocked steps exist in FP32 only (fine_shapes offers them nowhere else)
 template <class T>
-void launch_rb(bool down, const FineShape& f, const Level& L, const Level& C, const KData& K, MgWork<T>& w, int l,
-               const cx<T>* b, const cx<T>* x0, cx<T>* x, long ld, int ncols, int cpg, cudaStream_t s) {
-  if constexpr (std::is_same<T, float>::value) {
-    const bool s32 = f.ft == 32 && f.nt == 256, s64 = f.ft == 64 && f.nt == 512, t32 = f.ft == 32 && f.nt == 128;
-    if (!s32 && !s64 && !t32) fail(-1, "nodal step: no register-blocked kernel for this shape");
-    if (down) {
-      if (s64) launch_node_down_rb<64, 512>(L, C, K, w, l, b, x0, ld, ncols, cpg, s);
-      else if (s32) launch_node_down_rb<32, 256>(L, C, K, w, l, b, x0, ld, ncols, cpg, s);
-      else launch_node_down_rb<32, 128>(L, C, K, w, l, b, x0, ld, ncols, cpg, s);
-    } else {
-      if (s64) launch_node_up_rb<64, 512>(L, C, K, w, l, b, x, ld, ncols, cpg, s);
-      else if (s32) launch_node_up_rb<32, 256>(L, C, K, w, l, b, x, ld, ncols, cpg, s);
-      else launch_node_up_rb<32, 128>(L, C, K, w, l, b, x, ld, ncols, cpg, s);
-    }
-  } else {
-    fail(-1, "nodal step: register-blocked kernels run FP32 only");
-  }
+void launch_node_down_strips(const Level& L, const Level& C, const KData& K, MgWork<T>& w, int l, const cx<T>* b, const cx<T>* x0,
+                             long ld, int ncols, int cpg, int rows, cudaStream_t s) {
+  const dim3 grid(node_strip_blocks<kDownLanes>(L.n, L.m, rows), ncols);
+  if (x0)
+    k_node_down_strips<T, true><<<grid, 32 * kNodeStripWarps, 0, s>>>(L.lvl<T>(), K.d_ph, cpg, b, ld, x0, ld, w.r[l], L.N(),
+                                                                      w.b[l + 1], C.N(), rows);
+  else
+    k_node_down_strips<T, false><<<grid, 32 * kNodeStripWarps, 0, s>>>(L.lvl<T>(), K.d_ph, cpg, b, ld, x0, ld, w.r[l], L.N(),
+                                                                       w.b[l + 1], C.N(), rows);
+  PBS_LAUNCHED();
+}
+
+template <class T>
+void launch_node_up_strips(const Level& L, const Level& C, const KData& K, MgWork<T>& w, int l, const cx<T>* b, cx<T>* x, long ld,
+                           int ncols, int cpg, int rows, cudaStream_t s) {
+  k_node_up_strips<T><<<dim3(node_strip_blocks<kUpLanes>(L.n, L.m, rows), ncols), 32 * kNodeStripWarps, 0, s>>>(
+      L.lvl<T>(), K.d_ph, cpg, b, ld, w.r[l], L.N(), w.x[l + 1], C.N(), x, ld, rows);
+  PBS_LAUNCHED();
 }
 
 // The coarse levels from l down in one launch.
@@ -1111,12 +1087,12 @@ void node_cycle(const Hierarchy& H, const KData& K, MgWork<T>& w, int l, const c
   if (fine_tiled(L, nu_pre, nu_post)) {
     const Level& C = H.lev[l + 1];
     const auto down = [&](const FineShape& f) {
-      if (f.rb) launch_rb<T>(true, f, L, C, K, w, l, b, x0, nullptr, ld, ncols, cpg, s);
+      if (f.nt == 0) launch_node_down_strips<T>(L, C, K, w, l, b, x0, ld, ncols, cpg, f.ft, s);
       else if (f.ft == 64) launch_node_down<T, 64>(L, C, K, w, l, b, x0, ld, ncols, cpg, nu_pre, f.nt, s);
       else launch_node_down<T, 32>(L, C, K, w, l, b, x0, ld, ncols, cpg, nu_pre, f.nt, s);
     };
     const auto up = [&](const FineShape& f) {
-      if (f.rb) launch_rb<T>(false, f, L, C, K, w, l, b, nullptr, x, ld, ncols, cpg, s);
+      if (f.nt == 0) launch_node_up_strips<T>(L, C, K, w, l, b, x, ld, ncols, cpg, f.ft, s);
       else if (f.ft == 64) launch_node_up<T, 64>(L, C, K, w, l, b, x, ld, ncols, cpg, nu_post, f.nt, s);
       else launch_node_up<T, 32>(L, C, K, w, l, b, x, ld, ncols, cpg, nu_post, f.nt, s);
     };

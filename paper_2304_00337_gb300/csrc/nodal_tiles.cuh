@@ -10,7 +10,8 @@ namespace pbs {
 // ---- tiled fine-level nodal steps ------------------------------------------------
 // On levels too large for the fused tail, the pre-smoothing, residual and
 // restriction of the nodal cycle run as one kernel ("down") and the prolongation
-// and post-smoothing as another ("up").  A CTA owns an FT x FT tile of fine nodes of
+// and post-smoothing as another ("up"): here for two and three sweeps per side (one
+// sweep runs as row strips, node_strips.cuh).  A CTA owns an FT x FT tile of fine nodes of
 // one column and keeps a halo in shared memory wide enough that every colour step
 // can be carried out there: colour step s of S = 4 nu needs the previous state one
 // node further out, so the region shrinks by one ring per step.  Nodes outside the
@@ -174,6 +175,8 @@ __global__ void __launch_bounds__(kFineMaxThreads) k_node_up(Lvl<T> L, int nc, i
 
 
 // ---- register-blocked variants (FP32, one sweep per side) ---------------------
+// Not launched by the library any more (node_strips.cuh is faster on every level); the host
+// emulation checks them against the kernels above.
 // The same two steps with the work split by 2 x 2 node blocks.  Region node (a, b)
 // lives in shared memory in colour plane (a & 1) + 2 (b & 1), at position
 // (b >> 1) H + (a >> 1) of that plane (H = W / 2; the region origins are even, so a
