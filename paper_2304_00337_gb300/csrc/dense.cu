@@ -1803,7 +1803,7 @@ void block_update(Roles X, int q, const double2* C, int ldc, long cgs, double2* 
   const std::string key = std::string(dfa ? "update_df" : "update") + "|" + std::to_string(rows) + "|q" +
                           std::to_string(q) + "|p" + std::to_string(p) + "|g" + std::to_string(group_bucket(ngroups)) + "|" +
                           device_tag();
-  if (d_exps && update_tc_takes(q, p)) {
+  if (d_exps) {
     // one GB300, E and P of four groups, block 10, per iteration: 1024 x 1024 9.6 -> 3.2 ms, 256 x 256
     // 0.70 -> 0.22 ms; 208 x 144, block 14: 0.41 -> 0.10 ms.  Persistent CTAs, one per SM: about one, two or
     // four waves of them over the groups

@@ -316,7 +316,6 @@ void block_update(Roles X, int q, const double2* C, int ldc, long cgs, double2* 
                   cudaStream_t s);
 // The same on the tensor cores (update_tc.cu): d_exps from gram_groups, the exponent of trial column i of
 // group g at d_exps[g egs + 2 i]; `slices` CTAs per group (the result does not depend on it).
-bool update_tc_takes(int q, int p);
 void update_tc(Roles X, int q, const double2* C, int ldc, long cgs, const int* d_exps, int egs, double2* Y, long ldy, int p,
                const double2* Z, long ldz, long rows, int ngroups, int slices, cudaStream_t s);
 void random_block(double2* X, long ld, long rows, int ncols, uint64_t seed, cudaStream_t s);

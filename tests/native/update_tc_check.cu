@@ -88,20 +88,22 @@ static bool run(int pr, int q, int p, long rows, int G, bool with_z, int slices,
           ok = ok && y.x == 1e300 && y.y == 1e300;
           continue;
         }
-        long double sx = 0, sy = 0;
+        long double sx = 0, sy = 0, mag = 0;
         double fx = 0, fy = 0;
         for (int i = 0; i < q; ++i) {
           const C2 x = X[i / pr][((long)g * pr + i % pr) * ld + r], c = C[((long)g * p + j) * q + i];
           sx += (long double)x.x * c.x - (long double)x.y * c.y;
           sy += (long double)x.x * c.y + (long double)x.y * c.x;
+          mag += (std::fabs((long double)x.x) + std::fabs((long double)x.y)) * (std::fabs((long double)c.x) + std::fabs((long double)c.y));
           fx = std::fma(x.x, c.x, std::fma(-x.y, c.y, fx));
           fy = std::fma(x.x, c.y, std::fma(x.y, c.x, fy));
         }
         const C2 z = with_z ? Z[((long)g * p + j) * ld + r] : C2{0.0, 0.0};
         const long double tol = F * (2 * q * per + 0x1p-57L);
         const long double dx = std::fabs(y.x - (sx + z.x)), dy = std::fabs(y.y - (sy + z.y));
-        const long double bx = tol + 0x1p-53L * (std::fabs(sx) + std::fabs(sx + z.x)) * 1.01L,
-                          by = tol + 0x1p-53L * (std::fabs(sy) + std::fabs(sy + z.y)) * 1.01L;
+        const int parts = (q + 31) / 32;  // of the trial columns: each is rounded, and added in FP64
+        const long double bx = parts * tol + 0x1p-53L * (std::fabs(sx) + std::fabs(sx + z.x) + (parts > 1 ? 3 * mag : 0)) * 1.01L,
+                          by = parts * tol + 0x1p-53L * (std::fabs(sy) + std::fabs(sy + z.y) + (parts > 1 ? 3 * mag : 0)) * 1.01L;
         ok = ok && dx <= bx && dy <= by;
         worst = std::max({worst, (double)(dx / (bx + 1e-300L)), (double)(dy / (by + 1e-300L))});
         big = std::max({big, (double)std::fabs(sx), (double)std::fabs(sy)});
@@ -134,6 +136,10 @@ int main() {
     ok = run(8, 16, 8, rows, 1, true, 100, 0.0) && ok;
     ok = run(10, 10, 10, rows, 3, false, 2, 0.0) && ok;
   }
+  ok = run(24, 48, 24, 700, 2, true, 2, 0.0) && ok;           // two parts of each
+  ok = run(32, 64, 32, 300, 1, false, 2, 0.0) && ok;
+  ok = run(17, 17, 17, 300, 2, true, 2, 0.0) && ok;           // uneven parts
+  ok = run(11, 33, 31, 300, 1, false, 2, 0.0) && ok;
   ok = run(10, 20, 10, 3000, 1, false, 1, 3.0) && ok;   // column sizes over 60 decades
   ok = run(16, 16, 16, 3000, 1, false, 1, 4.0) && ok;
   ok = run(4, 12, 7, 500, 2, false, 2, 0.5) && ok;      // three roles, fewer outputs than columns
