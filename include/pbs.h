@@ -73,16 +73,18 @@ extern "C" {
 #define PBS_FP64 0  /* every kernel in FP64 ("plain"), the small Rayleigh-Ritz
                        eigensolve included; no double-float kernel runs
                        (pbs_launch_count_df does not move)                    */
-#define PBS_MIXED 1 /* FP32 multigrid V-cycles and nodal cycles; the Gram
-                       matrices, the Rayleigh quotients of the iteration, the
-                       projection right-hand side L^* M x, the search direction
-                       P and the small Rayleigh-Ritz eigensolve in double-float
-                       arithmetic on the FP32 pipe (FP64 storage, about 2^-47
-                       relative rounding); FP64 for everything that writes the
-                       iterate or differences it through the curl-curl stencil
-                       (residual A E - M E Lambda, E update, x - L phi) and for
-                       the reported eigenvalues (FP64 Rayleigh quotients of the
-                       converged block)                                       */
+#define PBS_MIXED 1 /* FP32 multigrid V-cycles and nodal cycles; the Rayleigh
+                       quotients of the iteration, the projection right-hand
+                       side L^* M x and the small Rayleigh-Ritz eigensolve in
+                       double-float arithmetic on the FP32 pipe (FP64 storage,
+                       about 2^-47 relative rounding); the Gram matrices and the
+                       updates of E and P on the tensor cores with fixed-point
+                       digits (2^-47 and 2^-62 of a column's largest value) or,
+                       where those do not apply, in double-float and FP64; FP64
+                       or exact integers for what writes the iterate or
+                       differences it through the curl-curl stencil (residual
+                       A E - M E Lambda, x - L phi) and FP64 for the reported
+                       eigenvalues (Rayleigh quotients of the converged block) */
 
 /* ---- operators for pbs_apply ----------------------------------------- */
 #define PBS_OP_A 0             /* edge -> edge: y = A x  (Section 3)            */

@@ -274,7 +274,7 @@ void deflate_constants(const Level& L, double2* X, long ld, int ncols, const int
 // per column: out[2c] = e^* M e, out[2c+1] = (C e)^* W (C e)
 void rayleigh_parts(const Level& L, const double* d_ph, int cpg, const double2* X, long ld, int ncols,
                     double* d_partials, double* d_out, bool dfa, cudaStream_t s);
-// R = A E - lam M E in the mixed policy: FP64 curls, double-float rest, R stored in
+// R = A E - lam M E in the mixed policy: exact integer curls, double-float rest, R stored in
 // FP32 (the preconditioner's input); the same norms (level 0 only)
 void residual_mixed(const Level& L, const double* d_ph, int cpg, const double2* E, float2* R, long ld, int ncols,
                     const double* d_lam, double* d_partials, double* d_out, cudaStream_t s);
