@@ -10,8 +10,9 @@ band 1 next to Gamma).  ``--workload c2`` is the 256 x 256 path of 31 Bloch vect
 (four chains with Rayleigh-quotient extrapolation), ``c4`` the 4096 x 4096 field of
 16 seeded disks (12 bands, block 16, 16 Bloch vectors).
 
-``value``: mixed precision (FP32 multigrid and nodal projection; double-float Gram,
-Rayleigh quotients and small Rayleigh-Ritz; FP64 residual, update and reported
+``value``: mixed precision (FP32 multigrid and nodal projection; Gram and block update
+on the tensor cores in fixed-point digits with exact sums; double-float Rayleigh
+quotients, residual (exact integer curls) and small Rayleigh-Ritz; FP64 reported
 eigenvalues), inputs and outputs resident on the device (``pbs_solve_path_device``);
 ``plain_fp64`` is the same workload with every kernel in FP64, and the per-band
 difference of the two policies' eigenvalues is reported.  ``e2e``: the host-buffer
@@ -58,7 +59,6 @@ WORKLOADS = {
 GOLDEN_C2 = os.path.join(ROOT, "tests", "golden", "rod256_path31.txt")
 PEAKS_PATH = os.path.join(ROOT, "MEASURED_PEAKS.json")
 SAMPLE_EVERY = 16  # the dominant kernel is timed on every 16th launch inside the timed region
-GRAM_DRAM_BYTES = 256.6e6  # measured per batched k_gram_df launch at 256x256 (4 groups of 30 columns)
 FP64_PEAK_TFLOPS = 1.2  # 152 SMs x 4 FP64 flop/clk x ~1.98 GHz; measured 1.20 TFLOP/s with an FMA-chain probe
 # Double-float kernels (mixed policy) run on the FP32 pipe: 152 SMs x 128 lanes x 1.98 GHz
 # instructions/s, and a compensated complex multiply-add (8 algorithmic flops) takes 48 of them.
@@ -401,19 +401,20 @@ def run_ours(args):
     if rank != 0:
         return
     peaks, peak_kind = _peaks()
-    df_classes = {"gram", "small_rr"}  # double-float arithmetic under the mixed policy
-    fp64_classes = {"block_update"}
-    if dominant in df_classes:
+    df_classes = {"small_rr"}  # double-float arithmetic under the mixed policy
+    digit_products = {"gram": 24, "block_update": 36}  # tensor-core products per product of the block
+    if dominant in digit_products:
+        achieved = dom_work / (dom_ms / 1e3) / 1e12
+        peak = peaks["bf16_tflops"] / digit_products[dominant]
+        roof = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TFLOP/s", "frac": achieved / peak,
+                "traffic": None, "kernel": dominant,
+                "peak_kind": f"{peak_kind} bf16_tflops over the {digit_products[dominant]} digit products of each product"}
+    elif dominant in df_classes:
         achieved = dom_work / (dom_ms / 1e3) / 1e12
         roof = {"bound": "alu", "achieved": achieved, "peak": DF_PEAK_TFLOPS, "unit": "TFLOP/s",
                 "frac": achieved / DF_PEAK_TFLOPS, "traffic": None, "kernel": dominant,
                 "peak_kind": "derived double-float rate on the FP32 pipe (152 SMs x 128 lanes x 1.98 GHz, "
                              "48 FP32 instructions per 8-flop compensated complex multiply-add)"}
-    elif dominant in fp64_classes:
-        achieved = dom_work / (dom_ms / 1e3) / 1e12
-        roof = {"bound": "alu", "achieved": achieved, "peak": FP64_PEAK_TFLOPS, "unit": "TFLOP/s",
-                "frac": achieved / FP64_PEAK_TFLOPS, "traffic": None, "kernel": dominant,
-                "peak_kind": "derived FP64 rate (152 SMs x 4 flop/clk x 1.98 GHz, matches a measured FMA probe)"}
     else:
         achieved = dom_work / (dom_ms / 1e3) / 1e9
         roof = {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
@@ -428,8 +429,9 @@ def run_ours(args):
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": ws, "steps": args.steps, "warmup": args.warmup,
         "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak", "vs_baseline": None,
-        "dtype": "c128 storage; FP64 residual and update; double-float (FP32 pipe) Gram, Rayleigh quotients "
-                 "and small Rayleigh-Ritz; c64 FP32 multigrid", "data": "synthetic",
+        "dtype": "c128 storage; Gram and update in 48- and 62-bit fixed-point digits with exact sums (tensor cores); "
+                 "double-float (FP32 pipe) Rayleigh quotients, residual (exact integer curls) and small "
+                 "Rayleigh-Ritz; c64 FP32 multigrid", "data": "synthetic",
         "config": {"workload": w["text"], "grid": f"{n}x{n}", "k_points": nk, "bands": nev, "block": w["block"],
                    "tol": TOL, "k_points_in_flight": w["kbatch"], "precision": "mixed",
                    "l2": "flushed (512 MiB write) before every timed step", "replicas": ws},
