@@ -6,15 +6,19 @@
 //   GM: v = z_x and z_y, z_x = sqrt(mx)(alpha x(i,j) + beta x(i,j+1)), z_y likewise along i;
 //   GA: v = sqrt(w) curl.
 // Each operand value is brought to a fixed-point integer of 48 bits, relative to a power of two
-// that bounds its trial column (k_gram_exponents), and cut into six signed 8-bit digits, held as
-// binary16 integers.  A digit product is exact in the tensor core's FP32 sums: P = sum over digit
+// that bounds its trial column's operands (k_gram_exponents: sqrt(mx) |x| and sqrt(my) |y| for GM,
+// sqrt(w) |curl| for GA), and cut into six signed 8-bit digits, held as binary16 integers.  A digit product is exact in the tensor core's FP32 sums: P = sum over digit
 // pairs i + j <= 5, and those with i odd and i + j = 6, of P_ij 2^{-8(i+j)} (the error-free
 // splitting of Ozaki, Ogita, Oishi and Rump, 2012; the squares of digit 3 do not average out on
 // the diagonal, so they are kept).  256 nodes add at most 2 x 512 x 2^14 = 2^24 to a sum of equal i + j <= 3, so FP32 sums
 // of 256 nodes are exact; they are then taken out of TMEM and added up as 64-bit integers.  The
-// only rounding is that of the 48-bit operands (2^-47 of the column's largest value; the
+// only rounding is that of the 48-bit operands (2^-47 of the column's largest operand; the
 // double-float kernel rounds each value to 2^-47 of itself, and its curls to 2^-47 of the edge
-// values they are differences of) and of the dropped pairs, whose signs are random.
+// values they are differences of) and of the dropped pairs, whose signs are random.  Both fields'
+// operands have to reach full scale for that: edge values are line integrals, |y| / |x| of a smooth
+// field is about h2/h1, and relative to a bound of the unweighted values the dropped pairs would
+// weigh (h2/h1)^2 times as much (GM of smooth fields on 32 x 48, of sqrt(G_aa G_bb): 2.4e-13 at
+// h2/h1 = 16, 3.8e-12 at 64; now 1e-15 to 4e-15 from 1/64 to 64).
 //
 // Digits come from integers, not from double-float: FP64 input is shifted into 64-bit fixed point
 // (the curl's differences are then exact), multiplied by 63-bit constants, and a byte permutation
@@ -65,10 +69,10 @@ inline Fix make_fix(double f) {
   r.lo = (int)((s - (double)r.hi) * 2147483648.0);
   return r;
 }
-// v 2^{52 - E}, |v| < 2^E, E > kMinExp, truncated to an integer.  (Zero and subnormals, exponent
+// v 2^{52 - E}, |v| < 2^{E+1}, E > kMinExp, truncated to an integer.  (Zero and subnormals, exponent
 // field 0, are shifted out whole.)
 __device__ __forceinline__ long long to_fixed(double v, int E) {
-  const int hi = __double2hiint(v), sh = min(E + 1023 - ((hi >> 20) & 0x7FF), 63);  // at least 1
+  const int hi = __double2hiint(v), sh = min(E + 1023 - ((hi >> 20) & 0x7FF), 63);  // at least 0
   const unsigned long long m =
       (((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(v)) >> sh;
   const long long s = (long long)(hi >> 31);
@@ -156,18 +160,18 @@ __device__ __forceinline__ PairY load_y(const double2* __restrict__ Y, int i, in
   return p;
 }
 
-// Exponents of the operands of every trial column: E[2 c] with |x|, |y| < 2^E, E[2 c + 1] with
-// sqrt(w) |curl| < 0.99 2^E (c = g q + column; kExpInf where a value is not finite; very negative
-// for a column of zeros).  A bound needs few bits: the curl is formed in binary32 from the leading
+// Exponents of every trial column c = g q + column: E[2 c] with |x|, |y| < 2^E, E[2 c + 1] with
+// sqrt(w) |curl| < 0.99 2^E, Em[2 c] with sx |x|, sy |y| < 2^E (sx, sy: sqrt(mx), sqrt(my) over 0.99;
+// kExpInf where a value is not finite; very negative for a column of zeros).  A bound needs few bits: the curl is formed in binary32 from the leading
 // 21 bits of its edge values, 2^-18 of which is added to it (the digits then still reach 2^-60 of
 // the edge values, below their FP64 rounding).  One pass over the block, bound by memory: 8 rows per
 // thread, two nodes wide, the upper row's x-edges carried to the next; a block whose largest value is
 // outside the middle of the binary32 range walks its tile again relative to that value.
 constexpr int kExpThreads = 256, kExpTile = 64;  // a block's tile: 64 nodes x 64 mesh rows
 __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, const double* __restrict__ ph, Roles roles, int q,
-                                                                const uint2* __restrict__ sw, int sw_exp,
-                                                                int* __restrict__ E) {
-  __shared__ int red[2][kExpThreads / 32];
+                                                                const uint2* __restrict__ sw, int sw_exp, double sx, double sy,
+                                                                int* __restrict__ E, int* __restrict__ Em) {
+  __shared__ int red[3][kExpThreads / 32];
   const int col = blockIdx.y, g = blockIdx.z, tid = threadIdx.x, lane = tid & 31;
   const int tx = (n + kExpTile - 1) / kExpTile, by = blockIdx.x / tx, bx = blockIdx.x - by * tx;
   const double2* X = trial_col(roles, g, col);
@@ -175,11 +179,11 @@ __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, co
   const Ph<double> p = load_ph<double>(ph, g);
   const int i = bx * kExpTile + 2 * lane, j0 = by * kExpTile + 8 * (tid >> 5);
   const bool in = i < n;
-  int base = 896, hi = 0, cb = 0;  // binary64 exponent field that becomes binary32's 0
+  int base = 896, hx = 0, hy = 0, cb = 0;  // base: binary64 exponent field that becomes binary32's 0
   for (int pass = 0; pass < 2; ++pass) {
-    int top = 0;        // largest high word (sign off): the exponent of the largest value
+    int topx = 0, topy = 0;  // largest high words (sign off): the exponents of the fields' largest values
     float cmax = 0.0f;  // largest 2^-sw_exp sqrt(w) (|c| + 2^-18 of the values), relative to 2^(base - 896)
-    auto lead = [&](double d) {
+    auto lead = [&](double d, int& top) {
       const int h = __double2hiint(d), a = h & 0x7FFFFFFF;
       top = max(top, a);
       const int f = a < ((base + 4) << 20) ? 0 : (a - (base << 20)) << 3;
@@ -190,8 +194,8 @@ __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, co
       const PairX v = load_x(X, i, j0, n, m, p.be, in && j0 < m);
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        x0[k][0] = lead(v.v[k].x);
-        x0[k][1] = lead(v.v[k].y);
+        x0[k][0] = lead(v.v[k].x, topx);
+        x0[k][1] = lead(v.v[k].y, topx);
       }
     }
     for (int j = j0; j < min(j0 + 8, m); ++j) {
@@ -200,15 +204,15 @@ __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, co
       float y[3][2];
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        y[k][0] = lead(u.v[k].x);
-        y[k][1] = lead(u.v[k].y);
+        y[k][0] = lead(u.v[k].x, topy);
+        y[k][1] = lead(u.v[k].y, topy);
       }
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
         const float s = in ? (float)sw[(long)j * n + i + k].x : 0.0f;
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-          const float x1 = lead(c ? v.v[k].y : v.v[k].x);
+          const float x1 = lead(c ? v.v[k].y : v.v[k].x, topx);
           const float d = fabsf((x1 - x0[k][c]) - (y[k + 1][c] - y[k][c]));
           const float e = fmaxf(fmaxf(fabsf(x1), fabsf(x0[k][c])), fmaxf(fabsf(y[k + 1][c]), fabsf(y[k][c])));
           cmax = fmaxf(cmax, s * fmaf(e, 0x1p-18f, d));
@@ -217,30 +221,39 @@ __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, co
       }
     }
     // high words order like the values, bits of non-negative floats too
-    const int t = __reduce_max_sync(0xffffffffu, top);
+    const int t = __reduce_max_sync(0xffffffffu, topx);
+    const int u = __reduce_max_sync(0xffffffffu, topy);
     const int c = __reduce_max_sync(0xffffffffu, __float_as_int(cmax));
     if (lane == 0) {
       red[0][tid >> 5] = t;
-      red[1][tid >> 5] = c;
+      red[1][tid >> 5] = u;
+      red[2][tid >> 5] = c;
     }
     __syncthreads();
-    hi = cb = 0;
+    hx = hy = cb = 0;
     for (int w = 0; w < kExpThreads / 32; ++w) {
-      hi = max(hi, red[0][w]);
-      cb = max(cb, red[1][w]);
+      hx = max(hx, red[0][w]);
+      hy = max(hy, red[1][w]);
+      cb = max(cb, red[2][w]);
     }
-    const int e = hi >> 20;
+    const int e = max(hx, hy) >> 20;
     if (e == 0 || e == 0x7FF || (e >= 960 && e <= 1080)) break;
     base = e - 127;
     __syncthreads();
   }
   if (tid != 0) return;
-  const int e = hi >> 20;
+  const int e = max(hx, hy) >> 20;
   if (e == 0) return;
-  int ex = e - 1022, ez;
+  int ex = e - 1022, ez, em;
   if (e == 0x7FF) {
-    ex = ez = kExpInf;
+    ex = ez = em = kExpInf;
   } else {
+    // s v < 2^(result) for the largest v with high word h
+    auto weighted = [](int h, double s) {
+      if ((h >> 20) == 0) return -kExpInf;
+      return (h >> 20) - 1023 + ilogb(s * __hiloint2double((h & 0xFFFFF) | 0x3FF00000, -1)) + 1;
+    };
+    em = max(weighted(hx, sx), weighted(hy, sy));
     // sw holds 31 bits; 2 % for the roundings and the margin; a block without curl counts as tiny
     const float v = __int_as_float(cb) * (1.02f * 0x1p-31f);
     ez = v > 0.0f ? ilogbf(v) + 1 + sw_exp + base - 896 : ex + sw_exp - 18;
@@ -248,19 +261,20 @@ __global__ void __launch_bounds__(kExpThreads) k_gram_exponents(int n, int m, co
   int* Ec = E + 2 * ((long)g * q + col);
   atomicMax(Ec, ex);
   atomicMax(Ec + 1, ez);
+  atomicMax(Em + 2 * ((long)g * q + col), em);
 }
 
 struct GramArgs {
   int n, m;
   long N;
-  Fix ax, bx, ay, by;  // mass factor over kappa
-  double kappa2;
+  Fix ax, bx, ay, by;  // mass factor times 2^ox (x-edges) and 2^oy (y-edges)
+  int ox, oy;          // x 2^{52 - Em - ox} < 2^53 likewise
   const uint2* sw;
   int sw_exp;
   const double* ph;
   Roles roles;
   int q;
-  const int* E;
+  const int *E, *Em;  // exponents, entry 2 (g q + column)
   double2* part;
   int npart;
 };
@@ -274,6 +288,7 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
                                               const int (&Ez)[2], const bool (&on)[2], const Ph<double>& p, int i, int j0,
                                               unsigned place, Wait&& wait, Ready&& ready) {
   const bool col_in = i < A.n;
+  const int dy = MASS ? A.oy - A.ox : 0;  // the fields' own fixed point
   long long xf[BLOCKS][2][2];  // x-edges of the current row: block, node, component
   PairX nx;                    // loads of the next step (a single block's; two blocks load as they go)
   PairY ny;
@@ -314,8 +329,8 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
       }
 #pragma unroll
       for (int k = 0; k < 3; ++k) {
-        y[k][0] = to_fixed(ny.v[k].x, Ex[b]);
-        y[k][1] = to_fixed(ny.v[k].y, Ex[b]);
+        y[k][0] = to_fixed(ny.v[k].x, Ex[b] + dy);
+        y[k][1] = to_fixed(ny.v[k].y, Ex[b] + dy);
       }
       if (BLOCKS == 1) {
         const bool in = on[0] && col_in && j + 1 < A.m && s + 1 < kChunk / kStage;
@@ -455,10 +470,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
       Xc[b] = trial_col(A.roles, g, on[b] ? col : 0);
       Ex[b] = Ez[b] = 0;
       if (on[b]) {
-        const int e0 = A.E[2 * ((long)g * A.q + col)], e1 = A.E[2 * ((long)g * A.q + col) + 1];
+        const int e0 = (mass ? A.Em : A.E)[2 * ((long)g * A.q + col)], e1 = A.E[2 * ((long)g * A.q + col) + 1];
         on[b] = e0 > kMinExp && e0 < kExpInf;  // zero columns stay zero, non-finite ones are marked at the end
-        Ex[b] = e0;
-        Ez[b] = e1;
+        Ex[b] = on[b] ? e0 + (mass ? A.ox : 0) : 0;
+        Ez[b] = on[b] ? e1 : 0;
       }
     }
     const bool any = __any_sync(0xffffffffu, on[0] || on[1]);
@@ -534,7 +549,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
   for (int t = tid; t < kCols * kCols; t += kThreads) {
     const int a = t % kCols, b = t / kCols, ca = I * kCols + a, cb = J * kCols + b;
     if (ca > cb || cb >= A.q) continue;
-    const int ea = A.E[2 * ((long)g * A.q + ca) + (mass ? 0 : 1)], eb = A.E[2 * ((long)g * A.q + cb) + (mass ? 0 : 1)];
+    const int* exps = mass ? A.Em : A.E + 1;
+    const int ea = exps[2 * ((long)g * A.q + ca)], eb = exps[2 * ((long)g * A.q + cb)];
     auto sum = [&](int r, int c) {
       const double even = S[r * 65 + c], odd = S[(64 + r) * 65 + c];
       return even + 0x1p-8 * (diag ? odd + S[(64 + c) * 65 + r] : odd);
@@ -543,8 +559,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
     if (ea <= kMinExp || eb <= kMinExp) {
       v = make_double2(0.0, 0.0);
     } else {
-      const double s = mass ? A.kappa2 : 1.0;
-      v = make_double2(s * scalbn(v.x, ea + eb - 46), s * scalbn(v.y, ea + eb - 46));
+      v = make_double2(scalbn(v.x, ea + eb - 46), scalbn(v.y, ea + eb - 46));
     }
     if (bad || ea == kExpInf || eb == kExpInf) v = make_double2(nan(""), nan(""));
     out[cb * (cb + 1) / 2 + ca] = v;
@@ -563,7 +578,8 @@ int gram_tc_partials(int n, int m, int q, int ngroups) {
   return (int)std::max<long>(1, std::min(np, chunks));
 }
 
-size_t gram_tc_scratch(int q, int ngroups) { return 2 * sizeof(int) * (size_t)q * ngroups; }
+// E and Em
+size_t gram_tc_scratch(int q, int ngroups) { return 4 * sizeof(int) * (size_t)q * ngroups; }
 
 void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
              int* d_exps, cudaStream_t s) {
@@ -571,27 +587,37 @@ void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups
   once([] { PBS_CUDA(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)); });
   // every byte 0x80: below -kExpInf
   PBS_CUDA(cudaMemsetAsync(d_exps, 0x80, gram_tc_scratch(q, ngroups), s));
+  int* d_em = d_exps + 2 * (long)q * ngroups;
+  // sqrt(mx) over 0.99, so that |z| < 0.99 times the bound 2^Em, and the power of two that brings
+  // sqrt(mx) to 0.495 .. 0.99: |x| < 2^(Em + ox + 1) then
+  const double sx = std::sqrt(L.h2 / L.h1), sy = std::sqrt(L.h1 / L.h2);
+  int ox = 0, oy = 0;
+  std::frexp(0.99 / sx, &ox);
+  std::frexp(0.99 / sy, &oy);
+  --ox, --oy;
   const unsigned tiles = ((L.n + kExpTile - 1) / kExpTile) * ((L.m + kExpTile - 1) / kExpTile);
-  k_gram_exponents<<<dim3(tiles, q, ngroups), kExpThreads, 0, s>>>(L.n, L.m, d_ph, roles, q, L.sw, L.sw_exp, d_exps);
+  k_gram_exponents<<<dim3(tiles, q, ngroups), kExpThreads, 0, s>>>(L.n, L.m, d_ph, roles, q, L.sw, L.sw_exp, sx / 0.99, sy / 0.99,
+                                                                   d_exps, d_em);
   PBS_LAUNCHED();
-  // the mass factor relative to kappa, so that |z| < 0.99 times the bound of the edge values
   const double r3 = 1.0 / std::sqrt(3.0), al = 0.5 * (1.0 + r3), be = 0.5 * (1.0 - r3);
-  const double sx = std::sqrt(L.h2 / L.h1), sy = std::sqrt(L.h1 / L.h2), kappa = std::max(sx, sy) / 0.99;
+  const double fx = std::ldexp(sx, ox), fy = std::ldexp(sy, oy);
   GramArgs a{};
   a.n = L.n;
   a.m = L.m;
   a.N = L.N();
-  a.ax = make_fix(sx * al / kappa);
-  a.bx = make_fix(sx * be / kappa);
-  a.ay = make_fix(sy * al / kappa);
-  a.by = make_fix(sy * be / kappa);
-  a.kappa2 = kappa * kappa;
+  a.ax = make_fix(fx * al);
+  a.bx = make_fix(fx * be);
+  a.ay = make_fix(fy * al);
+  a.by = make_fix(fy * be);
+  a.ox = ox;
+  a.oy = oy;
   a.sw = L.sw;
   a.sw_exp = L.sw_exp;
   a.ph = d_ph;
   a.roles = roles;
   a.q = q;
   a.E = d_exps;
+  a.Em = d_em;
   a.part = d_partials;
   a.npart = npart;
   const int nb = (q + kCols - 1) / kCols;
