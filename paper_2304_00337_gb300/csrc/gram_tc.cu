@@ -7,18 +7,21 @@
 //   GA: v = sqrt(w) curl.
 // Each operand value is brought to a fixed-point integer of 48 bits, relative to a power of two
 // that bounds its trial column's operands (k_gram_exponents: sqrt(mx) |x| and sqrt(my) |y| for GM,
-// sqrt(w) |curl| for GA), and cut into six signed 8-bit digits, held as binary16 integers.  A digit product is exact in the tensor core's FP32 sums: P = sum over digit
-// pairs i + j <= 5, and those with i odd and i + j = 6, of P_ij 2^{-8(i+j)} (the error-free
-// splitting of Ozaki, Ogita, Oishi and Rump, 2012; the squares of digit 3 do not average out on
-// the diagonal, so they are kept).  256 nodes add at most 2 x 512 x 2^14 = 2^24 to a sum of equal i + j <= 3, so FP32 sums
-// of 256 nodes are exact; they are then taken out of TMEM and added up as 64-bit integers.  The
-// only rounding is that of the 48-bit operands (2^-47 of the column's largest operand; the
-// double-float kernel rounds each value to 2^-47 of itself, and its curls to 2^-47 of the edge
-// values they are differences of) and of the dropped pairs, whose signs are random.  Both fields'
-// operands have to reach full scale for that: edge values are line integrals, |y| / |x| of a smooth
-// field is about h2/h1, and relative to a bound of the unweighted values the dropped pairs would
-// weigh (h2/h1)^2 times as much (GM of smooth fields on 32 x 48, of sqrt(G_aa G_bb): 2.4e-13 at
-// h2/h1 = 16, 3.8e-12 at 64; now 1e-15 to 4e-15 from 1/64 to 64).
+// sqrt(w) |curl| for GA), and cut into six signed 8-bit digits, held as binary16 integers.  A digit
+// product is exact in the tensor core's FP32 sums: P = sum over digit pairs i + j <= 6, and those
+// with i odd and i + j = 7, of P_ij 2^{-8(i+j)} (the error-free splitting of Ozaki, Ogita, Oishi and
+// Rump, 2012).  256 nodes add at most 2 x 512 x 2^14 = 2^24 to a sum of equal i + j <= 3, so FP32
+// sums of 256 nodes are exact; they are then taken out of TMEM and added up as 64-bit integers, in
+// units that leave the CTA's chunks their room (2^-46 to 2^-53 of the scales).  What is left is the
+// rounding of the 48-bit operands, 2^-47 of the column's largest operand; the double-float kernel
+// rounds each value to 2^-47 of itself, and its curls to 2^-47 of the edge values they are
+// differences of.  Errors on 32 x 48, of sqrt(G_aa G_bb): 1e-15 to 3e-15 for noise, up to 6e-15 for
+// smooth fields, double-float 0.5e-15 to 1e-15 and up to 5e-15.  Two choices matter for that:
+//  * the pairs (2, 4) and (4, 2), 2^-48 of the scales each (without them 6e-15 to 1e-14 for noise and
+//    6e-14 for smooth curls; with them 1.27 ms at 1024 x 1024, q = 30, as before);
+//  * both fields' operands at full scale: edge values are line integrals, |y| / |x| of a smooth field
+//    is about h2/h1, and relative to a bound of the unweighted values the dropped pairs weigh
+//    (h2/h1)^2 times as much (2.4e-13 for smooth fields at h2/h1 = 16, 3.8e-12 at 64).
 //
 // Digits come from integers, not from double-float: FP64 input is shifted into 64-bit fixed point
 // (the curl's differences are then exact), multiplied by 63-bit constants, and a byte permutation
@@ -30,7 +33,7 @@
 // and every npart-th chunk of 32 nodes x 8 mesh rows.  16 producer warps fill a ring of 32-node stages; one
 // thread of a 17th warp issues the MMAs (A = two digits of block I, 128 rows; B = up to four
 // digits of block J, 64 rows each; K-major, no swizzle); after each chunk the producers read
-// TMEM.  Accumulator D_t (t = 0 .. 5, 128 rows x 64 columns) holds the pairs i + j = t of even i in
+// TMEM.  Accumulator D_t (t = 0 .. 6, 128 rows x 64 columns) holds the pairs i + j = t of even i in
 // rows 0-63 and i + j = t + 1 of odd i in rows 64-127: A = digits (2 u, 2 u + 1), B = digit t - 2 u.
 // For I = J the product is symmetric, even-odd pairs are the transposes of odd-even ones, and the
 // rows 0-63 of odd t are not used.
@@ -418,6 +421,9 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
   long long acc[16];  // this thread's sums: row lane + 32 (warp & 3) of the pair, 16 columns from 16 (warp >> 2)
 #pragma unroll
   for (int k = 0; k < 16; ++k) acc[k] = 0;
+  // a chunk adds less than 2^55 at weight 2^32: 2^up times that for up to 2^(7 - up) chunks
+  int up = 7;
+  for (int c = (nchunk + A.npart - 1) / A.npart; c > 1 && up > 0; c = (c + 1) / 2) --up;
 
   if (warp == kProducers / 32) {
     if (lane == 0) {
@@ -441,7 +447,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
               tc_mma(tmem, tc_desc(a, kOctet), tc_desc(b, kOctet), tc_idesc(256), acm);
               tc_mma(tmem + 256, tc_desc(a, kOctet), tc_desc(b + 4 * 1024, kOctet), tc_idesc(128), acm);
               tc_mma(tmem + 128, tc_desc(a + 2048, kOctet), tc_desc(b, kOctet), tc_idesc(256), 1);
-              tc_mma(tmem + 256, tc_desc(a + 4096, kOctet), tc_desc(b, kOctet), tc_idesc(128), 1);
+              tc_mma(tmem + 384, tc_desc(a + 2048, kOctet), tc_desc(b + 4 * 1024, kOctet), tc_idesc(64), acm);
+              tc_mma(tmem + 256, tc_desc(a + 4096, kOctet), tc_desc(b, kOctet), tc_idesc(192), 1);
             }
           }
           tc_commit(empty + 8 * st);
@@ -513,13 +520,14 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
       tc_fence_after();
       const unsigned ta = tmem + ((unsigned)(warp & 3) << 21) + 16 * (warp >> 2);
       const bool odd = (warp & 2) != 0;
-      // weights of D_t in the 64-bit sum: 2^(32 - 8 t); on the diagonal odd t count on odd rows
+      // weights of D_t in the 64-bit sum: 2^(32 + up - 8 t); on the diagonal odd t count on odd rows
       // only, halved (their product is symmetric there)
-      for (int t = 0; t < 6; ++t) {
+#pragma unroll
+      for (int t = 0; t < 7; ++t) {
         float d[16];
         tc_ld16(ta + 64 * t, d);
         if (diag && (t & 1) && !odd) continue;
-        const int sh = 32 - 8 * t - (diag && (t & 1) ? 1 : 0);  // t = 5: -8 or -9
+        const int sh = 32 + up - 8 * t - (diag && (t & 1) ? 1 : 0);  // t = 6: -16 to -9
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
           const long long v = (long long)__float2int_rn(d[k]);
@@ -559,7 +567,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
     if (ea <= kMinExp || eb <= kMinExp) {
       v = make_double2(0.0, 0.0);
     } else {
-      v = make_double2(scalbn(v.x, ea + eb - 46), scalbn(v.y, ea + eb - 46));
+      v = make_double2(scalbn(v.x, ea + eb - 46 - up), scalbn(v.y, ea + eb - 46 - up));
     }
     if (bad || ea == kExpInf || eb == kExpInf) v = make_double2(nan(""), nan(""));
     out[cb * (cb + 1) / 2 + ca] = v;

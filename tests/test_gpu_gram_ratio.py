@@ -94,3 +94,37 @@ def test_gram_does_not_depend_on_the_cell_shape(ctx, r, kind):
         assert np.all(err <= tol), (r, kind, float(np.max(err / np.maximum(tol, 1e-300))),
                                     float(np.max(err / np.maximum(np.outer(d, d), 1e-300))))
         assert np.array_equal(got, got.conj().T)
+
+
+@pytest.mark.parametrize("q", [12, 40])
+def test_products_of_exact_operands(ctx, q):
+    # Integers below 2^44 as edge values, w = 16 and no phases: the operands sqrt(w) curl are integers
+    # that 48 bits hold exactly, so all that is lost are the digit pairs left out and the last places.
+    # On 4 x 4 nodes those pairs would show if two more of them were (2^-48 of the scales each).
+    n, k = 4, (0.0, 0.0)
+    rng = np.random.default_rng(q)
+    e = [[int(v) for v in rng.integers(-2 ** 44 + 1, 2 ** 44, 4 * n * n)] for _ in range(q)]
+    S = np.array([np.array(c[:2 * n * n], float) + 1j * np.array(c[2 * n * n:], float) for c in e])
+    Sd = torch.from_numpy(S).cuda()
+    G = torch.zeros((2, q, q), dtype=torch.complex128, device="cuda")
+    ctx.gram(pbs.Geometry(np.ones((n, n))), k, q, Sd.data_ptr(), G[0].data_ptr(), G[1].data_ptr(),
+             torch.cuda.current_stream(), precision=pbs.PBS_MIXED)
+    torch.cuda.synchronize()
+    got = G[1].cpu().numpy().T
+
+    def curls(c):  # x(i, j + 1) - x(i, j) - y(i + 1, j) + y(i, j)
+        x, y = c[:n * n], c[n * n:]
+        return [4 * (x[(j + 1) % n * n + i] - x[j * n + i] - y[j * n + (i + 1) % n] + y[j * n + i])
+                for j in range(n) for i in range(n)]
+
+    re, im = [curls(c[:2 * n * n]) for c in e], [curls(c[2 * n * n:]) for c in e]
+    # the exponents bound |z| by a power of two below 2.1 times the largest
+    scale = [2.1 * max(map(abs, re[c] + im[c])) for c in range(q)]
+    for a in range(q):
+        for b in range(a, q):
+            want_re = sum(u * v for u, v in zip(re[a], re[b])) + sum(u * v for u, v in zip(im[a], im[b]))
+            want_im = sum(u * v for u, v in zip(re[a], im[b])) - sum(u * v for u, v in zip(im[a], re[b]))
+            size = sum((abs(u) + abs(s)) * (abs(v) + abs(t)) for u, s, v, t in zip(re[a], im[a], re[b], im[b]))
+            # 2 n^2 real products; pairs (2, 5), (4, 3) at 2^-56 and what follows; eight roundings to FP64
+            tol = scale[a] * scale[b] * (2 * n * n * 2.01 * 2.0 ** -56 + 4 * 2.0 ** -53) + 8 * 2.0 ** -53 * size
+            assert abs(int(got[a, b].real) - want_re) <= tol and abs(int(got[a, b].imag) - want_im) <= tol, (a, b)
