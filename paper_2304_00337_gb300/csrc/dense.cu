@@ -1650,9 +1650,9 @@ bool gram_tc_rule(const Level& L, int q) {
   return q >= 9 || gram_on_tensor_cores();
 }
 
-const int* gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
+ColumnExps gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
                        double2* d_partials, long partial_capacity, bool dfa, cudaStream_t s) {
-  if (q <= 0 || ngroups <= 0) return nullptr;
+  if (q <= 0 || ngroups <= 0) return {};
   if (q > kMaxTrial) fail(PBS_EINVAL, "trial block too wide");
   const int ne = q * (q + 1) / 2;
   const int np0 = gram_partials(L.N(), ngroups);
@@ -1683,9 +1683,9 @@ const int* gram_groups(const Level& L, const double* d_ph, Roles roles, int q, i
     const int np = (int)std::min<long>(gram_tc_partials(L.n, L.m, q, ngroups), room);
     if (np < 1) fail(PBS_EINVAL, "gram partials buffer too small");
     const long used = (long)ngroups * np * 2 * ne;
-    int* exps = reinterpret_cast<int*>(d_partials + used);
+    int* d_exps = reinterpret_cast<int*>(d_partials + used);
     timer_begin(KC_GRAM, s, work);
-    gram_tc(L, d_ph, roles, q, ngroups, np, d_partials, exps, s);
+    const ColumnExps exps = gram_tc(L, d_ph, roles, q, ngroups, np, d_partials, d_exps, s);
     k_gram_finalize<<<dim3((2 * ne + kFinEntries - 1) / kFinEntries, ngroups), 8 * kFinEntries, 0, s>>>(d_partials, np, q, GM, GA);
     timer_end(KC_GRAM, s);
     PBS_LAUNCHED();
@@ -1720,7 +1720,7 @@ const int* gram_groups(const Level& L, const double* d_ph, Roles roles, int q, i
   timer_begin(KC_GRAM, s, work);
   launch(var[pick]);
   timer_end(KC_GRAM, s);
-  return nullptr;
+  return {};
 }
 
 long gram_partials_size(long rows, int q, int ngroups) {
@@ -1796,21 +1796,20 @@ template <int PB> void launch_update(Roles X, int q, const double2* C, int ldc, 
 }
 
 void block_update(Roles X, int q, const double2* C, int ldc, long cgs, double2* Y, long ldy, int p,
-                  const double2* Z, long ldz, long rows, int ngroups, bool dfa, const int* d_exps, int egs,
-                  cudaStream_t s) {
+                  const double2* Z, long ldz, long rows, int ngroups, bool dfa, const ColumnExps& exps, cudaStream_t s) {
   if (p <= 0 || rows <= 0 || ngroups <= 0) return;
   if (p > kMaxBlock) fail(PBS_EINVAL, "block_update: p too large");
   const std::string key = std::string(dfa ? "update_df" : "update") + "|" + std::to_string(rows) + "|q" +
                           std::to_string(q) + "|p" + std::to_string(p) + "|g" + std::to_string(group_bucket(ngroups)) + "|" +
                           device_tag();
-  if (d_exps) {
+  if (exps.e) {
     // one GB300, E and P of four groups, block 10, per iteration: 1024 x 1024 9.6 -> 3.2 ms, 256 x 256
     // 0.70 -> 0.22 ms; 208 x 144, block 14: 0.41 -> 0.10 ms.  Persistent CTAs, one per SM: about one, two or
     // four waves of them over the groups
     const int one = std::max(1, 152 / ngroups);
     const int slices[3] = {one, 2 * one, 4 * one};
     auto run = [&](int c) {
-      update_tc(X, q, C, ldc, cgs, d_exps, egs, Y, ldy, p, Z, ldz, rows, ngroups, slices[c], s);
+      update_tc(X, q, C, ldc, cgs, exps.e, exps.stride, Y, ldy, p, Z, ldz, rows, ngroups, slices[c], s, exps.ox, exps.oy);
     };
     const int pick = tune_pick(key + "|tc", 3, run, s);
     timer_begin(KC_BLOCK_UPDATE, s, 8.0 * q * p * rows * ngroups);  // flops

@@ -589,8 +589,8 @@ int gram_tc_partials(int n, int m, int q, int ngroups) {
 // E and Em
 size_t gram_tc_scratch(int q, int ngroups) { return 4 * sizeof(int) * (size_t)q * ngroups; }
 
-void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
-             int* d_exps, cudaStream_t s) {
+ColumnExps gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
+                   int* d_exps, cudaStream_t s) {
   static PerDeviceOnce once;
   once([] { PBS_CUDA(cudaFuncSetAttribute(k_gram_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem)); });
   // every byte 0x80: below -kExpInf
@@ -631,6 +631,7 @@ void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups
   const int nb = (q + kCols - 1) / kCols;
   k_gram_tc<<<dim3(npart, ngroups, nb * (nb + 1)), kThreads, kSmem, s>>>(a);
   PBS_LAUNCHED();
+  return ColumnExps{d_em, 2 * q, ox + 1, oy + 1};
 }
 
 }  // namespace pbs

@@ -290,9 +290,15 @@ struct Roles {
 };
 // Per group g (phases from entry g of d_ph): GM_g = S^* M S, GA_g = (C S)^* W (C S), q x q
 // column-major at GM + g q^2, GA + g q^2.
-// Returns the exponents of the trial columns (entry 2 (g q + a): |x| < 2^e over column a of group g) if
-// the tensor-core kernel ran, else null; they lie in d_partials, valid until that is written again.
-const int* gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
+// Returns the exponents of the trial columns if the tensor-core kernel ran, else none; they lie in
+// d_partials, valid until that is written again.
+struct ColumnExps {
+  const int* e = nullptr;  // column a of group g: e[g stride + 2 a]
+  int stride = 0;
+  int ox = 0, oy = 0;  // its x-edges are below 2^(e + ox), its y-edges below 2^(e + oy)
+  ColumnExps from(int a) const { return ColumnExps{e ? e + 2 * a : nullptr, stride, ox, oy}; }
+};
+ColumnExps gram_groups(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, double2* GM, double2* GA,
                        double2* d_partials, long partial_capacity, bool dfa, cudaStream_t s);
 long gram_partials_size(long rows, int q, int ngroups);  // double2 elements
 // The mixed policy's Gram on the tensor cores (gram_tc.cu): partial sums in the layout of
@@ -300,8 +306,8 @@ long gram_partials_size(long rows, int q, int ngroups);  // double2 elements
 bool gram_on_tensor_cores();  // the environment sets PBS_GRAM=tc: every width runs there
 int gram_tc_partials(int n, int m, int q, int ngroups);
 size_t gram_tc_scratch(int q, int ngroups);
-void gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
-             int* d_exps, cudaStream_t s);
+ColumnExps gram_tc(const Level& L, const double* d_ph, Roles roles, int q, int ngroups, int npart, double2* d_partials,
+                   int* d_exps, cudaStream_t s);
 // Rayleigh-Ritz in coefficient space for ngroups groups: C (q x p per group), theta (p per
 // group), status in d_info[8 g], scratch small_rr_scratch(q) bytes per group; dfa selects
 // double-float (mixed policy) instead of FP64 arithmetic
@@ -309,15 +315,15 @@ void small_rr(const double2* GM, const double2* GA, int q, int p, double2* C, do
               int* d_info, int ngroups, bool dfa, cudaStream_t s);
 size_t small_rr_scratch(int q);
 // Y_g[:, j] = sum_i X_g[:, i] C_g[i, j] (+ Z_g[:, j]) for each group
-// (dfa: double-float, for the search direction only; the iterate's update is FP64); d_exps, where
+// (dfa: double-float, for the search direction only; the iterate's update is FP64); exps, where
 // given: the columns' exponents, for the tensor cores
 void block_update(Roles X, int q, const double2* C, int ldc, long cgs, double2* Y, long ldy, int p,
-                  const double2* Z, long ldz, long rows, int ngroups, bool dfa, const int* d_exps, int egs,
-                  cudaStream_t s);
-// The same on the tensor cores (update_tc.cu): d_exps from gram_groups, the exponent of trial column i of
-// group g at d_exps[g egs + 2 i]; `slices` CTAs per group (the result does not depend on it).
+                  const double2* Z, long ldz, long rows, int ngroups, bool dfa, const ColumnExps& exps, cudaStream_t s);
+// The same on the tensor cores (update_tc.cu): the exponent of trial column i of group g at
+// d_exps[g egs + 2 i], plus ox for the first half of the rows and oy for the second (ColumnExps);
+// `slices` CTAs per group (the result does not depend on it).
 void update_tc(Roles X, int q, const double2* C, int ldc, long cgs, const int* d_exps, int egs, double2* Y, long ldy, int p,
-               const double2* Z, long ldz, long rows, int ngroups, int slices, cudaStream_t s);
+               const double2* Z, long ldz, long rows, int ngroups, int slices, cudaStream_t s, int ox = 0, int oy = 0);
 void random_block(double2* X, long ld, long rows, int ncols, uint64_t seed, cudaStream_t s);
 
 // ---- generalised Householder orthonormalisation (householder.cu) ----------

@@ -716,7 +716,7 @@ double rr_single(pbs_ctx* ctx, const KData& Kv, const double2* S, int q, int p, 
   if (info[0] != 0)
     fail(PBS_ENUMERIC, info[0] == -2 ? "non-finite Gram matrix"
                                      : info[0] == -3 ? "Rayleigh-Ritz breakdown" : "trial space lost rank");
-  block_update(R, q, W.C, q, (long)q * p, dst, W.D, p, nullptr, 0, W.D, 1, false, nullptr, 0, s);
+  block_update(R, q, W.C, q, (long)q * p, dst, W.D, p, nullptr, 0, W.D, 1, false, {}, s);
   double tm = 0.0;
   for (double t : th) tm = std::max(tm, std::fabs(t));
   return tm;
@@ -822,7 +822,7 @@ void rr_groups(pbs_ctx* ctx, const double2* S, int p, double2* dst, bool dfa, st
     for (int j = 0; j < p; ++j) tm = std::max(tm, std::fabs(th[(size_t)g * p + j]));
     theta_max[g] = tm;
   }
-  block_update(R, p, W.C, p, (long)p * p, dst, W.D, p, nullptr, 0, W.D, G, false, nullptr, 0, s);
+  block_update(R, p, W.C, p, (long)p * p, dst, W.D, p, nullptr, 0, W.D, G, false, {}, s);
 }
 
 void init_random_all(pbs_ctx* ctx, const pbs_opts& o, std::vector<Group>& gr, cudaStream_t s) {
@@ -1145,7 +1145,7 @@ PathResult solve_chain_list(pbs_ctx* ctx, const pbs_opts& o, int nk, const doubl
       // exists, and always for span 2, so its columns are dropped) or [E_hat] (span 1)
       const Roles trial = o.span == 1 ? Roles{{Wd, Wd, Wd}, p, D} : Roles{{W.E(), W.P(), W.W()}, p, D};
       const int qt = o.span == 1 ? p : q;
-      const int* exps = gram_groups(L0, ctx->K.d_ph, trial, qt, Ga, W.GM, W.GA, W.gpart, W.gpart_cap, dfa, s);
+      ColumnExps exps = gram_groups(L0, ctx->K.d_ph, trial, qt, Ga, W.GM, W.GA, W.gpart, W.gpart_cap, dfa, s);
       small_rr(W.GM, W.GA, qt, p, W.C, W.theta, W.rr_scr, W.info, Ga, dfa, s);
       PBS_CUDA(cudaMemcpyAsync(h_info.data(), W.info, sizeof(int) * 8 * Ga, cudaMemcpyDeviceToHost, s));
       PBS_CUDA(cudaStreamSynchronize(s));
@@ -1160,7 +1160,7 @@ PathResult solve_chain_list(pbs_ctx* ctx, const pbs_opts& o, int nk, const doubl
         const Roles tg{{W.E() + (long)g * p * D, W.P() + (long)g * p * D, W.W() + (long)g * p * D}, p, D};
         double2* GMg = W.GM + (long)g * q * q;
         double2* GAg = W.GA + (long)g * q * q;
-        exps = nullptr;  // the buffer they lie in is written again
+        exps = {};  // the buffer they lie in is written again
         gram_groups(L0, Kv.d_ph, tg, q, 1, GMg, GAg, W.gpart, W.gpart_cap, dfa, s);
         small_rr(GMg, GAg, q, p, W.C + (long)g * q * p, W.theta + (long)g * q, W.rr_scr, W.info + 8 * g, 1, dfa, s);
         int inf2[2];
@@ -1170,7 +1170,7 @@ PathResult solve_chain_list(pbs_ctx* ctx, const pbs_opts& o, int nk, const doubl
       }
       if (o.span == 1) {
         // E_new = E_hat C over the old E (E_hat lives in W); P stays zero
-        block_update(trial, p, W.C, p, (long)p * p, W.E(), D, p, nullptr, 0, D, Ga, false, exps, 2 * p, s);
+        block_update(trial, p, W.C, p, (long)p * p, W.E(), D, p, nullptr, 0, D, Ga, false, exps, s);
         PBS_CUDA(cudaMemsetAsync(W.P(), 0, sizeof(double2) * D * Gpa, s));
       } else {
         // P_new = [P, W] C[p:q] over R, E_new = E C[0:p] + P_new over W, then the
@@ -1178,10 +1178,9 @@ PathResult solve_chain_list(pbs_ctx* ctx, const pbs_opts& o, int nk, const doubl
         double2* P2 = W.R();
         double2* E2 = W.W();
         const Roles pw{{W.P(), W.W(), W.W()}, p, D};
-        block_update(pw, 2 * p, W.C + p, q, (long)q * p, P2, D, p, nullptr, 0, D, Ga, dfa,
-                     exps ? exps + 2 * p : nullptr, 2 * q, s);
+        block_update(pw, 2 * p, W.C + p, q, (long)q * p, P2, D, p, nullptr, 0, D, Ga, dfa, exps.from(p), s);
         const Roles ee{{W.E(), W.E(), W.E()}, p, D};
-        block_update(ee, p, W.C, q, (long)q * p, E2, D, p, P2, D, D, Ga, false, exps, 2 * q, s);
+        block_update(ee, p, W.C, q, (long)q * p, E2, D, p, P2, D, D, Ga, false, exps, s);
         W.half = 1 - W.half;
         if (o.span == 2) PBS_CUDA(cudaMemsetAsync(W.P(), 0, sizeof(double2) * D * Gpa, s));  // gradient method: no P
       }

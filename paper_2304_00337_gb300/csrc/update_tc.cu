@@ -4,11 +4,13 @@
 // component), Y is a real product of height `rows`.  k_block_update (dense.cu) did it on the FP64
 // pipe, which takes 64 cycles per warp instruction, k_block_update_df with 20 FP32 operations per
 // product.  Here each value of X is brought to a 62-bit fixed-point integer relative to a power of
-// two that bounds its trial column (the exponents of gram_tc.cu), each coefficient likewise relative
-// to the largest of its output column, and both are cut into eight signed 8-bit digits held as
-// binary16 integers (the error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012).  The FP32 sums
-// of digit products are exact (at most 64 x 7 x 2^14 < 2^23), digit pairs of equal i + j <= 7 share
-// an accumulator, and the eight sums are put together in 64-bit integers.  Operands keep 2^-62 of
+// two that bounds its trial column's x- or y-edges (the exponents of gram_tc.cu, for the weighted
+// edge values: with h2/h1 = r the fields differ by about r, and relative to one bound for both the
+// smaller would lose log2 r of its bits), each coefficient likewise relative to the largest of its
+// output column, and both are cut into eight signed 8-bit digits held as binary16 integers (the
+// error-free splitting of Ozaki, Ogita, Oishi and Rump, 2012).  The FP32 sums of digit products are
+// exact (at most 64 x 7 x 2^14 < 2^23), digit pairs of equal i + j <= 7 share an accumulator, and the
+// eight sums are put together in 64-bit integers.  Operands keep 2^-62 of
 // their bound and the dropped pairs are below 7.1 2^-62 of the largest product, so what is left is the
 // one rounding of the result to FP64 (by integers), and the addition of Z.  Largest error relative to
 // the largest value, random columns: 1.0e-16, sums of FP64 products 3e-16 to 5e-16.
@@ -55,6 +57,7 @@ struct UpdateArgs {
   long ldz;
   long rows;
   int nbuf;
+  int off;  // added to the exponents of X: values of column i are below 2^(E + off)
 };
 
 // v 2^{62 - E} truncated to an integer, for |v| < 2^E, E > kMinExp (zero and subnormals are shifted out)
@@ -169,6 +172,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_tc(UpdateArgs A) {
   }
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   __syncthreads();
+  // the exponents of the values from here on
+  if (tid < 32) Ex[tid] = max(Ex[tid], kMinExp) + A.off;
+  if (tid < 16) F[tid] += A.off;
+  __syncthreads();
   const unsigned tmem = *tmem_slot;
   const long tiles = (A.rows + kTile - 1) / kTile;
   const int first = blockIdx.x, step = gridDim.x;
@@ -215,7 +222,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_update_tc(UpdateArgs A) {
           unsigned bytes[4][4];  // per column: digits (0, 1), (2, 3), (4, 5), (6, 7) of both components
 #pragma unroll
           for (int k = 0; k < 4; ++k) {
-            const int e = max(Ex[4 * (wg + 4 * u) + k], kMinExp);
+            const int e = Ex[4 * (wg + 4 * u) + k];
             const unsigned long long x = fixed62(v[u][k].x, e) + kBias, y = fixed62(v[u][k].y, e) + kBias;
             const unsigned xh = (unsigned)(x >> 32), xl = (unsigned)x, yh = (unsigned)(y >> 32), yl = (unsigned)y;
             bytes[k][0] = __byte_perm(xh, yh, 0x6273);  // x digit 0, y digit 0, x digit 1, y digit 1 from the low byte up
@@ -329,7 +336,18 @@ template <int QU, int JW> void launch(UpdateArgs a, int slices, int ngroups, cud
 }  // namespace
 
 void update_tc(Roles X, int q, const double2* C, int ldc, long cgs, const int* d_exps, int egs, double2* Y, long ldy, int p,
-               const double2* Z, long ldz, long rows, int ngroups, int slices, cudaStream_t s) {
+               const double2* Z, long ldz, long rows, int ngroups, int slices, cudaStream_t s, int ox, int oy) {
+  if (ox != oy) {
+    // the two fields of unequal exponents one after the other (an offset per row instead, for every
+    // mesh, made the launch of square cells 11 % longer)
+    const long half = rows / 2;
+    for (int f = 0; f < 2; ++f) {
+      const Roles Xf{{X.b[0] + f * half, X.b[1] + f * half, X.b[2] + f * half}, X.pr, X.ld};
+      update_tc(Xf, q, C, ldc, cgs, d_exps, egs, Y + f * half, ldy, p, Z ? Z + f * half : nullptr, ldz, half, ngroups, slices, s,
+                f ? oy : ox, f ? oy : ox);
+    }
+    return;
+  }
   slices = (int)std::max<long>(1, std::min<long>(slices, (rows + kTile - 1) / kTile));
   // wide blocks (24 outputs of 72 trial columns, three groups at 128 x 128: 0.53 -> 0.17 ms per iteration)
   // in even parts: outputs of 16 at most (the accumulators of two tiles), trial columns of
@@ -340,7 +358,7 @@ void update_tc(Roles X, int q, const double2* C, int ldc, long cgs, const int* d
     for (int iq = 0; iq < nq; ++iq) {
       const int i0 = q * iq / nq, qi = q * (iq + 1) / nq - i0;
       UpdateArgs a{X, qi, C + (long)j0 * ldc + i0, ldc, cgs, d_exps + 2 * i0, egs, Y + j0 * ldy, ldy, iq > 0, pj, p, i0,
-                   Z && iq == nq - 1 ? Z + j0 * ldz : nullptr, ldz, rows, 1};
+                   Z && iq == nq - 1 ? Z + j0 * ldz : nullptr, ldz, rows, 1, ox};
       if (qi <= 16) {
         if (pj <= 8) launch<1, 2>(a, slices, ngroups, s);
         else if (pj <= 12) launch<1, 3>(a, slices, ngroups, s);
