@@ -1100,13 +1100,18 @@ void node_cycle(const Hierarchy& H, const KData& K, MgWork<T>& w, int l, const c
     const int nd = fine_shapes<T>(L, nu_pre, true, fd), nup = fine_shapes<T>(L, nu_post, false, fu);
     // both steps are idempotent (the down step reads b, the up step b, its saved
     // pre-smoothed x and the coarse correction, and neither writes what it reads)
-    const std::string key = fine_key<T>(L, ncols, cpg);
-    const int pd = tune_pick("node_down|" + key + "|nu" + std::to_string(nu_pre), nd, [&](int c) { down(fd[c]); }, s);
+    // (strips have their number of candidates in the key: plain keys with one sweep per side hold an
+    // earlier build's choices among tiles, other shapes under the same index)
+    const auto key = [&](const char* step, int nu, int count) {
+      return std::string(step) + (nu == 1 ? "strips" + std::to_string(count) + "|" : "") + fine_key<T>(L, ncols, cpg) + "|nu" +
+             std::to_string(nu);
+    };
+    const int pd = tune_pick(key("node_down|", nu_pre, nd), nd, [&](int c) { down(fd[c]); }, s);
     timer_begin(KC_NODE_SMOOTH, s, fine_bytes<T>(L, ncols, nu_pre, true));
     down(fd[pd]);
     timer_end(KC_NODE_SMOOTH, s);
     node_cycle<T>(H, K, w, l + 1, w.b[l + 1], w.x[l + 1], C.N(), ncols, cpg, nu_pre, nu_post, s);
-    const int pu = tune_pick("node_up|" + key + "|nu" + std::to_string(nu_post), nup, [&](int c) { up(fu[c]); }, s);
+    const int pu = tune_pick(key("node_up|", nu_post, nup), nup, [&](int c) { up(fu[c]); }, s);
     timer_begin(KC_NODE_SMOOTH, s, fine_bytes<T>(L, ncols, nu_post, false));
     up(fu[pu]);
     timer_end(KC_NODE_SMOOTH, s);
