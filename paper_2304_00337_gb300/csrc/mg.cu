@@ -910,14 +910,17 @@ template <class T, int FT> void set_fine_smem() {
 // row strips (ft rows, nt = 0), the others as tiles (side ft, nt threads).  One GB300, down + up step
 // in us, strips of 16 / 32 / 64 rows against the best tile: FP32, 40 columns: 1024 x 1024 449 / 438 /
 // 437, 846; 512 x 512 139 / 146 / 174, 234; 256 x 256 42 / 40 / 57, 65; 128 x 128 24 / 31 / 51, 29;
-// FP64, 20 columns: 512 x 512 1107 / 1160 / 1147, 1549; 128 x 128 121 / 219 / 413, 189.  The first
-// shape fits every level this path takes.
+// FP64, 20 columns: 512 x 512 1107 / 1160 / 1147, 1549; 128 x 128 121 / 219 / 413, 189.  With few
+// columns a strip is a chain of rows and little else, and short strips pay for their five halo rows:
+// 4 / 8 / 16 rows against the best tile, 10 columns, FP32: 72 x 72 13 / 16 / 21, 22; 128 x 128 13 / 16 /
+// 21, 22; 208 x 144 13 / 17 / 21, 25; 256 x 256 21 / 17 / 22; FP64: 72 x 72 43 / 70 / 119, 111; 128 x 128
+// 76 / 68 / 119, 197; 256 x 256 201 / 176 / 210.  The first shape fits every level this path takes.
 struct FineShape {
   int ft, nt;
 };
-constexpr FineShape kStripShapes[] = {{16, 0}, {32, 0}, {64, 0}};
+constexpr FineShape kStripShapes[] = {{16, 0}, {32, 0}, {64, 0}, {8, 0}, {4, 0}};
 constexpr FineShape kTileShapes[] = {{32, 256}, {64, 512}, {64, 256}};
-constexpr int kNumFineShapes = 3;
+constexpr int kNumFineShapes = 5;
 template <class T>
 int fine_shapes(const Level& L, int nu, bool down, FineShape* out) {
   int n = 0;
