@@ -1524,7 +1524,7 @@ void lift_adj_mass(const Level& L, const double* d_ph, int cpg, const double2* X
   if (ncols <= 0) return;
   timer_begin(KC_LIFT_ADJ_MASK, s, (16.0 * L.D() + 2.0 * sizeof(T) * L.N()) * ncols);
   if (dfa) {
-    const int rows = strip_rows(L.n, L.m);
+    const int rows = strip_rows(L.n, L.m, ncols);
     k_lift_adj_mass_strips<T><<<dim3(strip_blocks<30>(L.n, L.m, rows), ncols), 32 * kStripWarps, 0, s>>>(
         L.lvl<df>(), d_ph, cpg, X, ldx, Rhs, ldr, rows);
     count_df_launch();
@@ -1549,7 +1549,7 @@ void rayleigh_parts(const Level& L, const double* d_ph, int cpg, const double2* 
                     double* d_partials, double* d_out, bool dfa, cudaStream_t s) {
   if (ncols <= 0) return;
   const dim3 g = grid2(L.n, L.m, ncols);
-  const int rows = strip_rows(L.n, L.m), nblk = dfa ? (int)strip_blocks<31>(L.n, L.m, rows) : (int)(g.x * g.y);
+  const int rows = strip_rows(L.n, L.m, ncols), nblk = dfa ? (int)strip_blocks<31>(L.n, L.m, rows) : (int)(g.x * g.y);
   if (dfa) {
     k_rayleigh_strips<<<dim3(nblk, ncols), 32 * kStripWarps, 0, s>>>(L.lvl<df>(), L.wts_df(), d_ph, cpg, X, ld, rows,
                                                                       d_partials);
@@ -1565,7 +1565,7 @@ void rayleigh_parts(const Level& L, const double* d_ph, int cpg, const double2* 
 void residual_mixed(const Level& L, const double* d_ph, int cpg, const double2* E, float2* R, long ld, int ncols,
                     const double* d_lam, double* d_partials, double* d_out, cudaStream_t s) {
   if (ncols <= 0) return;
-  const int rows = strip_rows(L.n, L.m), nblk = (int)strip_blocks<30>(L.n, L.m, rows);
+  const int rows = strip_rows(L.n, L.m, ncols), nblk = (int)strip_blocks<30>(L.n, L.m, rows);
   timer_begin(KC_RESIDUAL, s, 24.0 * L.D() * ncols);  // read E (16 B), write R (8 B) per edge DOF
   k_residual_strips<<<dim3(nblk, ncols), 32 * kStripWarps, 0, s>>>(L.lvl<df>(), L.wts_df(), d_ph, cpg, E, R, ld, d_lam, rows,
                                                                     d_partials);

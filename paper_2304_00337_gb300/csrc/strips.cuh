@@ -295,16 +295,23 @@ __global__ void __launch_bounds__(32 * kStripWarps)
   }
 }
 
-// Rows of a strip: more of them share the halo row, fewer are more strips in flight.  Rayleigh quotient,
-// residual and right-hand side of 40 columns in us, for 4 / 8 / 16 / 32 rows:
-//   64 x 64 (32 columns)  10, 15, 10 / 12, 17, 13 / 21, 25, 19 / 35, 41, 33
-//   128 x 128             21, 35, 23 / 21, 33, 21 / 27, 39, 27 / 37, 45, 35
-//   256 x 256             54, 107, 56 / 52, 92, 51 / 51, 89, 52 / 62, 106, 62
-//   512 x 512             187, 382, 198 / 162, 319, 173 / 153, 293, 164 / 154, 289, 170
-//   1024 x 1024           721, 1423, 732 / 613, 1174, 631 / 565, 1048, 585 / 547, 998, 568
-inline int strip_rows(int n, int m) {
-  const long N = (long)n * m;
-  return N >= 1024L * 1024 ? 32 : (N >= 512L * 512 ? 16 : (N >= 96L * 96 ? 8 : 4));
+// Rows of a strip: more of them share the halo rows, fewer are more strips in flight and, where the
+// chip is not full, a shorter chain of rows.  Doubled from two while the launch has more warps than a
+// limit per choice.  Rayleigh quotient, residual and right-hand side in us for 2 / 4 / 8 / 16 / 32 rows:
+//   16 x 16, 10 columns     8, 8, 6 / 8, 10, 8 / 12, 13, 10
+//   96 x 96, 4 columns      8, 8, 6 / 8, 10, 8 / 12, 16, 12
+//   128 x 128, 10 columns   10, 16, 10 / 10, 15, 10 / 12, 17, 12 / 21, 25, 19
+//   128 x 128, 40 columns   23, 40, 23 / 21, 34, 21 / 21, 32, 21 / 25, 37, 25 / 35, 43, 33
+//   256 x 256, 40 columns   66, 136, 66 / 51, 103, 53 / 49, 89, 49 / 49, 86, 50 / 60, 102, 60
+//   512 x 512, 10 columns   63, 131, 66 / 49, 99, 52 / 45, 86, 48 / 47, 88, 54 / 58, 95, 60
+//   512 x 512, 40 columns   240, 501, 242 / 180, 368, 190 / 155, 309, 166 / 146, 282, 156 / 147, 279, 163
+//   1024 x 1024, 40 columns 928, 1888, 901 / 692, 1373, 703 / 588, 1133, 606 / 541, 1010, 561 / 523, 962, 544
+// (a rule on the mesh alone, eight rows from 96 x 96 on, took 15 us for the right-hand side of two
+// columns there, the 32 x 8 tiles before it 10).  From two rows on no launch has more blocks than the
+// mesh has 32 x 8 tiles, for which the partial sums have room.
+inline int strip_rows(int n, int m, int ncols) {
+  const auto warps = [&](int rows) { return (long)((n + 29) / 30) * ((m + rows - 1) / rows) * ncols; };
+  return warps(2) <= 3000 ? 2 : warps(4) <= 3700 ? 4 : warps(8) <= 12000 ? 8 : warps(16) <= 24000 ? 16 : 32;
 }
 template <int WIDTH> inline unsigned strip_blocks(int n, int m, int rows) {
   const long warps = (long)((n + WIDTH - 1) / WIDTH) * ((m + rows - 1) / rows);
