@@ -1677,11 +1677,10 @@ ColumnExps gram_groups(const Level& L, const double* d_ph, Roles roles, int q, i
                           std::to_string(group_bucket(ngroups)) + "|" + device_tag();
   // flops: three complex MACs per entry and node
   const double work = 8.0 * ne * 3.0 * L.N() * ngroups;
-  if (dfa && gram_tc_rule(L, q) && !tune_forced(key)) {
-    // (the scratch for the exponents is part of every partials buffer)
-    const long room = (partial_capacity - (long)(gram_tc_scratch(q, ngroups) / sizeof(double2)) - 1) / (2L * ngroups * ne);
-    const int np = (int)std::min<long>(gram_tc_partials(L.n, L.m, q, ngroups), room);
-    if (np < 1) fail(PBS_EINVAL, "gram partials buffer too small");
+  // (the scratch for the exponents is part of every partials buffer)
+  const long room = (partial_capacity - (long)(gram_tc_scratch(q, ngroups) / sizeof(double2)) - 1) / (2L * ngroups * ne);
+  const int np = gram_tc_npart(L.n, L.m, gram_tc_partials(L.n, L.m, q, ngroups), room);
+  if (dfa && gram_tc_rule(L, q) && np > 0 && !tune_forced(key)) {
     const long used = (long)ngroups * np * 2 * ne;
     int* d_exps = reinterpret_cast<int*>(d_partials + used);
     timer_begin(KC_GRAM, s, work);
@@ -1724,8 +1723,9 @@ ColumnExps gram_groups(const Level& L, const double* d_ph, Roles roles, int q, i
 }
 
 long gram_partials_size(long rows, int q, int ngroups) {
-  // partial sums for up to twice the default split (a tuning candidate); the tensor-core kernel has
-  // no more (gram_groups falls back where it had), and its exponents follow them
+  // partial sums for up to twice the default split (a tuning candidate); the tensor-core kernel takes
+  // as many of its own as fit (gram_groups runs the double-float kernel where those are too few), and
+  // its exponents follow them
   return 2L * ngroups * gram_partials(rows, ngroups) * q * (q + 1) + (long)(gram_tc_scratch(q, ngroups) / sizeof(double2)) + 1;
 }
 

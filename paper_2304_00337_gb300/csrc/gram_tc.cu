@@ -54,7 +54,8 @@ constexpr int kThreads = kProducers + 32;  // and the warp whose first lane issu
 constexpr int kCols = 32;                  // trial columns per block: 64 operand rows
 constexpr int kSlices = 6;
 constexpr int kRows = 64 * kSlices;        // operand rows of a block in shared memory, digit-major
-constexpr int kChunk = 256, kStage = 32;   // nodes per TMEM sum, per ring stage
+constexpr int kChunk = 256, kStage = 32;   // nodes per TMEM sum (gram_tc_chunks), per ring stage
+static_assert(kStage == 32 && kChunk == 8 * kStage, "gram_tc_chunks counts tiles of 32 x 8 nodes");
 constexpr int kOctet = kRows * 16;         // bytes of 8 nodes of a block's rows
 constexpr int kArray = kStage / 8 * kOctet;
 constexpr int kSmem = 196608 + 1024;       // ring and barriers
@@ -576,13 +577,12 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
 
 }  // namespace
 
-// Partial sums per group: enough CTAs for a few waves of one per SM, at most 128 chunks each (the
-// 64-bit sums then cannot overflow).
+// Partial sums per group: enough CTAs for a few waves of one per SM, at most kGramTcRoom chunks each.
 int gram_tc_partials(int n, int m, int q, int ngroups) {
   const int nb = (q + kCols - 1) / kCols, per = nb * (nb + 1);  // CTAs per group and partial block
-  const long chunks = (long)((n + kStage - 1) / kStage) * ((m + 7) / 8);
+  const long chunks = gram_tc_chunks(n, m);
   long np = (4L * 152 + (long)per * ngroups - 1) / ((long)per * ngroups);
-  np = std::max(np, (chunks + 127) / 128);
+  np = std::max(np, (chunks + kGramTcRoom - 1) / kGramTcRoom);
   return (int)std::max<long>(1, std::min(np, chunks));
 }
 

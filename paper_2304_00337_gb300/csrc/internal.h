@@ -303,6 +303,15 @@ ColumnExps gram_groups(const Level& L, const double* d_ph, Roles roles, int q, i
 long gram_partials_size(long rows, int q, int ngroups);  // double2 elements
 // The mixed policy's Gram on the tensor cores (gram_tc.cu): partial sums in the layout of
 // gram_groups, npart per group; d_exps: gram_tc_scratch bytes.
+// Its CTAs take whole chunks of 32 nodes x 8 mesh rows and keep their sums in 64-bit integers, which
+// have room for 128 chunks.
+constexpr int kGramTcRoom = 128;
+inline long gram_tc_chunks(int n, int m) { return (long)((n + 31) / 32) * ((m + 7) / 8); }
+// partial sums per group where `want` are wanted and `fit` fit the buffer; 0: too few for the integer sums
+inline int gram_tc_npart(int n, int m, int want, long fit) {
+  const long np = fit < want ? fit : want;
+  return np >= 1 && np * kGramTcRoom >= gram_tc_chunks(n, m) ? (int)np : 0;
+}
 bool gram_on_tensor_cores();  // the environment sets PBS_GRAM=tc: every width runs there
 int gram_tc_partials(int n, int m, int q, int ngroups);
 size_t gram_tc_scratch(int q, int ngroups);
