@@ -702,8 +702,11 @@ template <class R> struct Ar;
 template <> struct Ar<df> {
   using C = cdf;
   using lead_t = float;  // leading part: comparisons, magnitudes and pivot limits
-  struct Acc {           // running sum of products
-    acc2 a;
+  // Running sum of products, renormalised at every term: a lane adds up to 24 of them (q = 96), and
+  // compensated binary32 sums without a fold made the Ritz values' error grow with q (7e-15 of the norm
+  // at q = 96, now 4.5e-15 from q = 42 on; 3 % of the solve).
+  struct Acc {
+    df a;
   };
   static __device__ __forceinline__ df mk(float v) { return df_make(v, 0.0f); }
   static __device__ __forceinline__ df zero() { return df_zero(); }
@@ -742,9 +745,9 @@ template <> struct Ar<df> {
   static constexpr int kRescaleExp = 48;         // ... and the exponent shift they apply
   static __device__ __forceinline__ int expo(df a) { return (int)((__float_as_uint(a.hi) >> 23) & 0xFFu) - 127; }
   static __device__ __forceinline__ bool neg(df a) { return (__float_as_uint(a.hi) >> 31) != 0; }
-  static __device__ __forceinline__ void acc_zero(Acc& a) { a.a = acc2_zero(); }
-  static __device__ __forceinline__ void acc_mul(Acc& a, df x, df y) { dot2(a.a, x, y); }
-  static __device__ __forceinline__ df acc_get(const Acc& a) { return acc2_df(a.a); }
+  static __device__ __forceinline__ void acc_zero(Acc& a) { a.a = df_zero(); }
+  static __device__ __forceinline__ void acc_mul(Acc& a, df x, df y) { a.a = a.a + x * y; }
+  static __device__ __forceinline__ df acc_get(const Acc& a) { return a.a; }
 };
 template <> struct Ar<double> {
   using C = cd;
@@ -1195,7 +1198,9 @@ __global__ void __launch_bounds__(kRRThreads) k_small_rr(const double2* __restri
       R a0 = lo - A::mk(1e-6f * tnorm), b0 = hi + A::mk(1e-6f * tnorm);
       for (int it = 0; it < 30; ++it) {
         const R w = b0 - a0;
-        const bool done = A::to(w) <= 4e-15 * (double)tnorm;
+        // (ten steps of 33 or thirteen of 17; at 4e-15 the twelfth of 17 was the last one, 3.4e-15 wide, and
+        // Ritz values of more than 16 lost a factor of 2.5: 9e-16 of the norm instead of 4e-16 in FP64)
+        const bool done = A::to(w) <= 1.4e-15 * (double)tnorm;
         if (__all_sync(0xffffffffu, done)) break;
         const R x = a0 + A::mulf(w, float(sl + 1) / float(wd + 1));
         const int cnt = sturm_count_r<R>(ta, te2, r, x);
