@@ -211,11 +211,6 @@ __device__ __forceinline__ cdf cdf_conj(cdf a) { return cdf_make(a.re, -a.im); }
 __device__ __forceinline__ cdf operator*(cdf a, cdf b) {
   return cdf_make(a.re * b.re - a.im * b.im, a.re * b.im + a.im * b.re);
 }
-// conj(a) * b
-__device__ __forceinline__ cdf cdf_mulc(cdf a, cdf b) {
-  return cdf_make(a.re * b.re + a.im * b.im, a.re * b.im - a.im * b.re);
-}
 __device__ __forceinline__ cdf cdf_scale(cdf a, df s) { return cdf_make(a.re * s, a.im * s); }
-__device__ __forceinline__ df cdf_norm2(cdf a) { return a.re * a.re + a.im * a.im; }
 
 }  // namespace pbs

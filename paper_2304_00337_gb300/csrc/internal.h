@@ -254,16 +254,17 @@ void nodal_vcycle_from(const Hierarchy& H, const KData& K, MgWork<T>& w, int l0,
 // Every kernel below reads and writes FP64 blocks.  Where a `dfa` flag is given it
 // selects the arithmetic: false = FP64, true = double-float on the FP32 pipe
 // (about 2^-47 relative; the mixed-precision policy).  What writes the iterate or
-// differences it through the curl-curl stencil (residual, E C, x - L phi) stays in
-// FP64: a relative perturbation eta of the iterate moves the relative residual by
-// about eta lambda_max / lambda.
+// differences it through the curl-curl stencil keeps FP64's accuracy: x - L phi is FP64,
+// the mixed residual's curls are exact integers, E C is 62-bit fixed point on the tensor
+// cores or FP64 (a relative perturbation eta of the iterate moves the relative residual by
+// about eta lambda_max / lambda).
 void convert_d2f(const double2* X, float2* Y, long n, cudaStream_t s);
 void convert_f2d(const float2* X, double2* Y, long n, cudaStream_t s);
 // x <- x - L phi (FP64 x, phi in T), level 0
 template <class T>
 void sub_lift(const Level& L, const double* d_ph, int cpg, const cx<T>* Phi, long ldp, double2* X, long ldx, int ncols,
               cudaStream_t s);
-// rhs = L^* M x  (FP64), stored in T
+// rhs = L^* M x (FP64, or double-float where dfa), stored in T
 template <class T>
 void lift_adj_mass(const Level& L, const double* d_ph, int cpg, const double2* X, long ldx, cx<T>* Rhs, long ldr,
                    int ncols, bool dfa, cudaStream_t s);

@@ -13,9 +13,11 @@
 // eight sums are put together in 64-bit integers.  Operands keep 2^-62 of
 // their bound and the dropped pairs are below 7.1 2^-62 of the largest product, so what is left is the
 // one rounding of the result to FP64 (by integers), and the addition of Z.  Largest error relative to
-// the largest value, random columns: 1.0e-16, sums of FP64 products 3e-16 to 5e-16.
+// the largest value of an output column's field, for columns of similar size: 1.0e-16, sums of FP64
+// products 3e-16 to 5e-16; in general up to (2 q 16 2^-62 + 2^-57) of the bound, the largest |C_ij| 2^E_i.
 //
-// One persistent CTA per SM: 16 warps convert tiles of 128 rows into shared memory (a thread has one
+// One persistent CTA per SM (each allocates the whole TMEM, and 544 threads of more than 60 registers leave
+// no room for a second one, however little shared memory a narrow launch takes): 16 warps convert tiles of 128 rows into shared memory (a thread has one
 // row and quadruples of trial columns: loads of 32 neighbouring rows, 16-byte stores in the MMA's
 // K-major layout), one thread of a 17th warp issues the MMAs (A = one digit of X, M = 128; B = the
 // first digits of C side by side, so that pair (i, j) lands in accumulator i + j), and the 16 warps
