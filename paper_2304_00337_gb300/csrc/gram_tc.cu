@@ -73,29 +73,30 @@ inline Fix make_fix(double f) {
   r.lo = (int)((s - (double)r.hi) * 2147483648.0);
   return r;
 }
-// v 2^{52 - E}, |v| < 2^{E+1}, E > kMinExp, truncated to an integer.  (Zero and subnormals, exponent
-// field 0, are shifted out whole.)
+// v 2^{60 - E}, |v| < 2^{E+1}, E > kMinExp, truncated to an integer.  (Zero and subnormals, exponent
+// field 0, are shifted out whole.  Truncation pulls every value towards zero, which adds up on the
+// diagonal of a Gram: at 2^{52 - E} it was the largest error there, 1e-15 to 3e-15 for noise.)
 __device__ __forceinline__ long long to_fixed(double v, int E) {
   const int hi = __double2hiint(v), sh = min(E + 1023 - ((hi >> 20) & 0x7FF), 63);  // at least 0
   const unsigned long long m =
-      (((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(v)) >> sh;
+      (((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(v)) << 8 >> sh;
   const long long s = (long long)(hi >> 31);
   return ((long long)m ^ s) - s;
 }
-// Operand digits of 16 z + bias with z = X f / 32 (+ Y g / 32), |z| < 0.99 2^47, rounded to the nearest
-// integer: six bytes that carry 0x80 too much each.  h f.hi and the two high products are exact to
-// a few units of 2^-4.
-constexpr long long kDigitBias = 0x808080808080ll * 16 + 8;
+// Operand digits of z, |z| < 0.99 2^47, rounded to the nearest integer: six bytes that carry 0x80 too
+// much each.  digits1: z = X f / 32 (X a curl in units of 2^{Ez - 52}), the products exact to a few
+// units of 2^-4; digits2: z = (X f + Y g) / 2^13, to a few units of 2^-12.
+constexpr long long kDigitBias = 0x808080808080ll;
 __device__ __forceinline__ unsigned long long digits1(long long X, Fix f) {
   const int h = (int)(X >> 32);
-  const long long t = (long long)h * f.hi + kDigitBias + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
+  const long long t = (long long)h * f.hi + (kDigitBias * 16 + 8) + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
   return (unsigned long long)(t + 2 * (long long)__mulhi(h, f.lo)) >> 4;
 }
 __device__ __forceinline__ unsigned long long digits2(long long X, Fix f, long long Y, Fix g) {
   const int h = (int)(X >> 32), k = (int)(Y >> 32);
-  const long long t = (long long)h * f.hi + ((long long)k * g.hi + kDigitBias);
+  const long long t = (long long)h * f.hi + ((long long)k * g.hi + (kDigitBias * 4096 + 2048));
   const unsigned l = __umulhi((unsigned)X, (unsigned)f.hi) + __umulhi((unsigned)Y, (unsigned)g.hi);  // below 2^32
-  return (unsigned long long)(t + (long long)l + 2 * (long long)(__mulhi(h, f.lo) + __mulhi(k, g.lo))) >> 4;
+  return (unsigned long long)(t + (long long)l + 2 * (long long)(__mulhi(h, f.lo) + __mulhi(k, g.lo))) >> 12;
 }
 
 // Operand values of two neighbouring nodes and one component (biased digits b0, b1): stores digit s
@@ -272,7 +273,7 @@ struct GramArgs {
   int n, m;
   long N;
   Fix ax, bx, ay, by;  // mass factor times 2^ox (x-edges) and 2^oy (y-edges)
-  int ox, oy;          // x 2^{52 - Em - ox} < 2^53 likewise
+  int ox, oy;          // x 2^{60 - Em - ox} < 2^61 likewise
   const uint2* sw;
   int sw_exp;
   const double* ph;
@@ -342,7 +343,8 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
         ny = load_y(Xc[0] + A.N, i, j + 1, A.n, p.al, in);
       }
       const unsigned at = dst + b * kArray;
-      const int sh = Ex[b] + A.sw_exp - Ez[b];
+      const int sh = Ex[b] + A.sw_exp - Ez[b] - 8;
+      const long long half = sh >= 0 ? 0 : 1ll << (min(-sh, 62) - 1);
 #pragma unroll
       for (int im = 0; im < 2; ++im) {
         // (a row or column outside the level leaves zeros: its loads were zero, and the last row's
@@ -357,7 +359,7 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
             const long long d = (x1[k][im] - xf[b][k][im]) - (y[k + 1][im] - y[k][im]);
-            const long long e = sh >= 0 ? (long long)((unsigned long long)d << min(sh, 62)) : d >> min(-sh, 62);
+            const long long e = sh >= 0 ? (long long)((unsigned long long)d << min(sh, 62)) : (d + half) >> min(-sh, 62);
             z[k] = digits1(e, Fix{(int)w[k].x, (int)w[k].y});
           }
           store_digits(at + im * 512, z[0], z[1]);
