@@ -5,23 +5,30 @@
 // component), columns mesh nodes:
 //   GM: v = z_x and z_y, z_x = sqrt(mx)(alpha x(i,j) + beta x(i,j+1)), z_y likewise along i;
 //   GA: v = sqrt(w) curl.
-// Each operand value is brought to a fixed-point integer of 48 bits, relative to a power of two
-// that bounds its trial column's operands (k_gram_exponents: sqrt(mx) |x| and sqrt(my) |y| for GM,
-// sqrt(w) |curl| for GA), and cut into six signed 8-bit digits, held as binary16 integers.  A digit
-// product is exact in the tensor core's FP32 sums: P = sum over digit pairs i + j <= 6, and those
-// with i odd and i + j = 7, of P_ij 2^{-8(i+j)} (the error-free splitting of Ozaki, Ogita, Oishi and
-// Rump, 2012).  256 nodes add at most 2 x 512 x 2^14 = 2^24 to a sum of equal i + j <= 3, so FP32
+// Each operand value is brought to a fixed-point integer relative to a power of two that bounds its
+// trial column's operands (k_gram_exponents: sqrt(mx) |x| and sqrt(my) |y| for GM, sqrt(w) |curl| for
+// GA), of 48 bits (GM) or 49 (GA), and cut into six signed digits of 8 bits (GA's first: nine), held as
+// binary16 integers.  A digit product is exact in the tensor core's FP32 sums: P = sum over digit pairs
+// i + j <= 6, and those with i odd and i + j = 7, of P_ij 2^{-8(i+j)} (the error-free splitting of
+// Ozaki, Ogita, Oishi and Rump, 2012).  256 nodes add at most 2 x 512 x 2^14 = 2^24 to a sum of equal
+// i + j <= 3 (GA, one product per node: 256 x 2^16 for two ninth bits, and 2 x 256 x 2^15), so FP32
 // sums of 256 nodes are exact; they are then taken out of TMEM and added up as 64-bit integers, in
 // units that leave the CTA's chunks their room (2^-46 to 2^-53 of the scales).  What is left is the
-// rounding of the 48-bit operands, 2^-47 of the column's largest operand; the double-float kernel
-// rounds each value to 2^-47 of itself, and its curls to 2^-47 of the edge values they are
-// differences of.  Errors on 32 x 48, of sqrt(G_aa G_bb): 1e-15 to 3e-15 for noise, up to 6e-15 for
-// smooth fields, double-float 0.5e-15 to 1e-15 and up to 5e-15.  Two choices matter for that:
+// rounding of the operands, 2^-48 (GM) and 2^-49 (GA) of a power of two up to four times the column's
+// largest operand; the double-float kernel rounds each value to 2^-47 of itself, and its curls to 2^-47
+// of the edge values they are differences of, always towards zero.  Largest errors relative to
+// sqrt(G_aa G_bb), 32 x 48 / 128 x 96, 12 columns, h2/h1 from 1/64 to 64: noise 1.2e-15 / 4e-16, smooth
+// fields 5e-16 / 4e-16 in GM and 2e-15 / 1.5e-15 (curls of 1/20 of their edges' size) in GA;
+// double-float 1.9e-15 / 3.4e-15, 2.6e-15 / 4.6e-15 and 2.9e-15 / 3.5e-15.  What matters for that:
 //  * the pairs (2, 4) and (4, 2), 2^-48 of the scales each (without them 6e-15 to 1e-14 for noise and
-//    6e-14 for smooth curls; with them 1.27 ms at 1024 x 1024, q = 30, as before);
+//    6e-14 for smooth curls);
 //  * both fields' operands at full scale: edge values are line integrals, |y| / |x| of a smooth field
 //    is about h2/h1, and relative to a bound of the unweighted values the dropped pairs weigh
-//    (h2/h1)^2 times as much (2.4e-13 for smooth fields at h2/h1 = 16, 3.8e-12 at 64).
+//    (h2/h1)^2 times as much (2.4e-13 for smooth fields at h2/h1 = 16, 3.8e-12 at 64);
+//  * inputs in 61 bits (in 53, cut off towards zero, a bias of 1e-15 to 2e-15 on the diagonal);
+//  * GA's ninth bit: its operands are rounded, not its values, and the weights spread them (without it
+//    1.3e-15 to 2e-15 for noise on 32 x 48, now 6e-16 to 7e-16).
+// 1024 x 1024, q = 30: 1.27 ms without the last three, 1.30 ms with them.
 //
 // Digits come from integers, not from double-float: FP64 input is shifted into 64-bit fixed point
 // (the curl's differences are then exact), multiplied by 63-bit constants, and a byte permutation
@@ -83,14 +90,15 @@ __device__ __forceinline__ long long to_fixed(double v, int E) {
   const long long s = (long long)(hi >> 31);
   return ((long long)m ^ s) - s;
 }
-// Operand digits of z, |z| < 0.99 2^47, rounded to the nearest integer: six bytes that carry 0x80 too
-// much each.  digits1: z = X f / 32 (X a curl in units of 2^{Ez - 52}), the products exact to a few
-// units of 2^-4; digits2: z = (X f + Y g) / 2^13, to a few units of 2^-12.
-constexpr long long kDigitBias = 0x808080808080ll;
+// Operand digits of z rounded to the nearest integer: six bytes that carry 0x80 too much each, and in
+// digits1 a ninth bit of the first digit, which carries 0x100 too much.  digits1: z = X f / 16 (X a curl
+// in units of 2^{Ez - 52}), |z| < 0.99 2^48, the products exact to a few units of 2^-3; digits2:
+// z = (X f + Y g) / 2^13, |z| < 0.99 2^47, to a few units of 2^-12.
+constexpr long long kDigitBias = 0x808080808080ll, kDigitBias9 = 0x1008080808080ll;
 __device__ __forceinline__ unsigned long long digits1(long long X, Fix f) {
   const int h = (int)(X >> 32);
-  const long long t = (long long)h * f.hi + (kDigitBias * 16 + 8) + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
-  return (unsigned long long)(t + 2 * (long long)__mulhi(h, f.lo)) >> 4;
+  const long long t = (long long)h * f.hi + (kDigitBias9 * 8 + 4) + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
+  return (unsigned long long)(t + 2 * (long long)__mulhi(h, f.lo)) >> 3;
 }
 __device__ __forceinline__ unsigned long long digits2(long long X, Fix f, long long Y, Fix g) {
   const int h = (int)(X >> 32), k = (int)(Y >> 32);
@@ -100,9 +108,9 @@ __device__ __forceinline__ unsigned long long digits2(long long X, Fix f, long l
 }
 
 // Operand values of two neighbouring nodes and one component (biased digits b0, b1): stores digit s
-// of both at base + 1024 s (64 rows of 16 bytes) as two binary16 integers -128 .. 127.  A byte next to
-// the byte 0x64 is the binary16 number 1024 + byte.
-__device__ __forceinline__ void store_digits(unsigned base, unsigned long long b0, unsigned long long b1) {
+// of both at base + 1024 s (64 rows of 16 bytes) as two binary16 integers -128 .. 127 (the first digit
+// of nine bits: -256 .. 255).  A byte next to the byte 0x64 is the binary16 number 1024 + byte.
+template <bool NINE> __device__ __forceinline__ void store_digits(unsigned base, unsigned long long b0, unsigned long long b1) {
   const unsigned l0 = (unsigned)b0, h0 = (unsigned)(b0 >> 32), l1 = (unsigned)b1, h1 = (unsigned)(b1 >> 32);
   const __half2 bias = __halves2half2(__ushort_as_half(0x6480), __ushort_as_half(0x6480));  // 1024 + 128
   auto put = [&](int s, unsigned two) {
@@ -111,7 +119,14 @@ __device__ __forceinline__ void store_digits(unsigned base, unsigned long long b
   };
   // (byte i, byte i + 1 of both words), then each pair with the exponent byte
   const unsigned t45 = __byte_perm(h0, h1, 0x5140), t23 = __byte_perm(l0, l1, 0x7362), t01 = __byte_perm(l0, l1, 0x5140);
-  put(0, __byte_perm(t45, 0x64646464u, 0x4342));
+  if (NINE) {
+    const unsigned two = __byte_perm(h0, h1, 0x6521) | 0x64006400u;
+    const __half2 bias9 = __halves2half2(__ushort_as_half(0x6500), __ushort_as_half(0x6500));  // 1024 + 256
+    const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&two), bias9);
+    asm volatile("st.shared.b32 [%0], %1;" ::"r"(base), "r"(*reinterpret_cast<const unsigned*>(&d)) : "memory");
+  } else {
+    put(0, __byte_perm(t45, 0x64646464u, 0x4342));
+  }
   put(1, __byte_perm(t45, 0x64646464u, 0x4140));
   put(2, __byte_perm(t23, 0x64646464u, 0x4342));
   put(3, __byte_perm(t23, 0x64646464u, 0x4140));
@@ -351,8 +366,8 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
         // carried x-edges are not used)
         if (MASS) {
           const long long u0 = row_in ? xf[b][0][im] : 0, u1 = row_in ? xf[b][1][im] : 0;
-          store_digits(at + im * 512, digits2(u0, A.ax, x1[0][im], A.bx), digits2(u1, A.ax, x1[1][im], A.bx));
-          store_digits(at + BLOCKS * kArray + im * 512, digits2(y[0][im], A.ay, y[1][im], A.by),
+          store_digits<false>(at + im * 512, digits2(u0, A.ax, x1[0][im], A.bx), digits2(u1, A.ax, x1[1][im], A.bx));
+          store_digits<false>(at + BLOCKS * kArray + im * 512, digits2(y[0][im], A.ay, y[1][im], A.by),
                        digits2(y[1][im], A.ay, y[2][im], A.by));
         } else {
           unsigned long long z[2];
@@ -362,7 +377,7 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
             const long long e = sh >= 0 ? (long long)((unsigned long long)d << min(sh, 62)) : (d + half) >> min(-sh, 62);
             z[k] = digits1(e, Fix{(int)w[k].x, (int)w[k].y});
           }
-          store_digits(at + im * 512, z[0], z[1]);
+          store_digits<true>(at + im * 512, z[0], z[1]);
         }
       }
 #pragma unroll
@@ -424,9 +439,10 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
   long long acc[16];  // this thread's sums: row lane + 32 (warp & 3) of the pair, 16 columns from 16 (warp >> 2)
 #pragma unroll
   for (int k = 0; k < 16; ++k) acc[k] = 0;
-  // a chunk adds less than 2^55 at weight 2^32: 2^up times that for up to 2^(7 - up) chunks
-  int up = 7;
-  for (int c = (nchunk + A.npart - 1) / A.npart; c > 1 && up > 0; c = (c + 1) / 2) --up;
+  // a chunk adds less than 2^55 (GA: 2^56) at weight 2^32: 2^up times that for up to 2^(7 - up) chunks
+  // (2^(6 - up))
+  int up = mass ? 7 : 6;
+  for (int c = (nchunk + A.npart - 1) / A.npart; c > 1; c = (c + 1) / 2) --up;
 
   if (warp == kProducers / 32) {
     if (lane == 0) {
@@ -530,7 +546,7 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
         float d[16];
         tc_ld16(ta + 64 * t, d);
         if (diag && (t & 1) && !odd) continue;
-        const int sh = 32 + up - 8 * t - (diag && (t & 1) ? 1 : 0);  // t = 6: -16 to -9
+        const int sh = 32 + up - 8 * t - (diag && (t & 1) ? 1 : 0);  // t = 6: -17 to -9
 #pragma unroll
         for (int k = 0; k < 16; ++k) {
           const long long v = (long long)__float2int_rn(d[k]);
@@ -570,7 +586,8 @@ __global__ void __launch_bounds__(kThreads, 1) k_gram_tc(GramArgs A) {
     if (ea <= kMinExp || eb <= kMinExp) {
       v = make_double2(0.0, 0.0);
     } else {
-      v = make_double2(scalbn(v.x, ea + eb - 46 - up), scalbn(v.y, ea + eb - 46 - up));
+      const int ex = ea + eb - (mass ? 46 : 48) - up;
+      v = make_double2(scalbn(v.x, ex), scalbn(v.y, ex));
     }
     if (bad || ea == kExpInf || eb == kExpInf) v = make_double2(nan(""), nan(""));
     out[cb * (cb + 1) / 2 + ca] = v;

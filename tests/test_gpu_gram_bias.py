@@ -57,3 +57,25 @@ def test_diagonal(ctx, n, m, q, r):
         big = np.maximum(np.abs(v.real), np.abs(v.imag)).reshape(q, -1).max(axis=1)
         sd = float(np.max(2.0 * 2.0 ** -48 * 4.0 * big / np.sqrt(12.0) / np.sqrt(want)))
         assert abs(np.mean(err)) <= 6.0 * sd / np.sqrt(q) + 2 * 2.0 ** -53, (np.mean(err), sd)
+
+
+@pytest.mark.parametrize("n,m,q", [(64, 64, 12), (256, 192, 40), (2048, 1024, 72)])
+def test_operands_at_the_end_of_their_range(ctx, n, m, q):
+    # every curl of a column has the same size, just below its bound: the first digits stand at the ends
+    # of their nine bits at every node and the integer sums are as large as they get (2048 x 1024, 72
+    # columns: 128 chunks each).  Values of 20 bits and w = 4^k: nothing is rounded but the FP64 sums.
+    x = torch.zeros((q, 2, m, n), dtype=torch.complex128, device="cuda")
+    row = (1.0 - 2.0 * (torch.arange(m, device="cuda") % 2))[:, None]
+    rng = np.random.default_rng(q)
+    s = np.array([complex(*rng.choice([-1.0, 1.0], 2)) * 2.0 ** int(rng.integers(-9, 10)) for _ in range(q)])
+    v = round(0.97 * 2 ** 20) / 2 ** 20
+    for c in range(q):
+        x[c, 0] = (0.5 * v * complex(s[c])) * row  # curls -+ v s
+    w = 4.0 ** int(np.ceil(np.log(n * m) / np.log(4)))
+    G = torch.zeros((2, q, q), dtype=torch.complex128, device="cuda")
+    ctx.gram(pbs.Geometry(np.full((m, n), n * m / w)), (0.0, 0.0), q, x.data_ptr(), G[0].data_ptr(), G[1].data_ptr(),
+             torch.cuda.current_stream(), precision=pbs.PBS_MIXED)
+    torch.cuda.synchronize()
+    got, want = G[1].cpu().numpy().T, n * m * w * v * v * np.outer(s.conj(), s)
+    # up to 1000 partial sums of one size, added in eight lanes
+    assert np.max(np.abs(got - want) / np.abs(np.outer(s, s))) <= n * m * w * 2.0 * 130 * 2.0 ** -53
