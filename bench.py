@@ -402,7 +402,7 @@ def run_ours(args):
         return
     peaks, peak_kind = _peaks()
     df_classes = {"small_rr"}  # double-float arithmetic under the mixed policy
-    digit_products = {"gram": 24, "block_update": 36}  # tensor-core products per product of the block
+    digit_products = {"gram": 28, "block_update": 36}  # tensor-core products per product of the block
     if dominant in digit_products:
         achieved = dom_work / (dom_ms / 1e3) / 1e12
         peak = peaks["bf16_tflops"] / digit_products[dominant]

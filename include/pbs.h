@@ -79,7 +79,8 @@ extern "C" {
                        double-float arithmetic on the FP32 pipe (FP64 storage,
                        about 2^-47 relative rounding); the Gram matrices and the
                        updates of E and P on the tensor cores with fixed-point
-                       digits (2^-47 and 2^-62 of a column's largest value) or,
+                       digits (operands rounded to 2^-47 and 2^-62 of the
+                       largest one of their column, its weights included) or,
                        where those do not apply, in double-float and FP64; FP64
                        or exact integers for what writes the iterate or
                        differences it through the curl-curl stencil (residual
@@ -259,9 +260,11 @@ PBS_API int pbs_apply(pbs_ctx *ctx, const pbs_geom *geom, const pbs_opts *opts, 
  * Block Gram matrices of the pencil at k (Section 4, used by Rayleigh-Ritz):
  * GM = S^* M S and GA = (C S)^* W (C S) = S^* A S, W = diag(1/(eps_c h1 h2)).
  * S: device D x q; GM, GA: device q x q column-major.  `precision` selects the
- * arithmetic: PBS_FP64, or PBS_MIXED = double-float on the FP32 pipe (about
- * 2^-47 relative rounding, compensated sums), the arithmetic the mixed policy
- * uses inside the solver.  Inputs and outputs are FP64 either way.
+ * arithmetic: PBS_FP64, or PBS_MIXED = the arithmetic the mixed policy uses
+ * inside the solver: fixed-point operands on the tensor cores with exact sums
+ * (from nine columns on, permittivities within a factor of 2^16; operands
+ * rounded to 2^-47 of their column's largest one) or double-float on the FP32
+ * pipe (about 2^-47 relative rounding, compensated sums).  Inputs and outputs are FP64 either way.
  */
 PBS_API int pbs_gram(pbs_ctx *ctx, const pbs_geom *geom, const double k[2], int q, const pbs_c64 *S, pbs_c64 *GM,
              pbs_c64 *GA, int precision, void *cuda_stream);
