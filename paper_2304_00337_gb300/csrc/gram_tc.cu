@@ -17,18 +17,19 @@
 // rounding of the operands, 2^-48 (GM) and 2^-49 (GA) of a power of two up to four times the column's
 // largest operand; the double-float kernel rounds each value to 2^-47 of itself, and its curls to 2^-47
 // of the edge values they are differences of, always towards zero.  Largest errors relative to
-// sqrt(G_aa G_bb), 32 x 48 / 128 x 96, 12 columns, h2/h1 from 1/64 to 64: noise 1.2e-15 / 4e-16, smooth
-// fields 5e-16 / 4e-16 in GM and 2e-15 / 1.5e-15 (curls of 1/20 of their edges' size) in GA;
+// sqrt(G_aa G_bb), 32 x 48 / 128 x 96, 12 columns, h2/h1 from 1/64 to 64: noise 1.2e-15 / 5e-16, smooth
+// fields 8e-16 / 4e-16 in GM and 1.6e-15 / 1.9e-15 (curls of 1/20 of their edges' size) in GA;
 // double-float 1.9e-15 / 3.4e-15, 2.6e-15 / 4.6e-15 and 2.9e-15 / 3.5e-15.  What matters for that:
 //  * the pairs (2, 4) and (4, 2), 2^-48 of the scales each (without them 6e-15 to 1e-14 for noise and
 //    6e-14 for smooth curls);
 //  * both fields' operands at full scale: edge values are line integrals, |y| / |x| of a smooth field
 //    is about h2/h1, and relative to a bound of the unweighted values the dropped pairs weigh
 //    (h2/h1)^2 times as much (2.4e-13 for smooth fields at h2/h1 = 16, 3.8e-12 at 64);
-//  * inputs in 61 bits (in 53, cut off towards zero, a bias of 1e-15 to 2e-15 on the diagonal);
+//  * inputs rounded down, what that takes given back by a constant (cut off towards zero they left a
+//    bias of 1e-15 to 2e-15 on the diagonal; eight bits more for them cost 2 % of the kernel);
 //  * GA's ninth bit: its operands are rounded, not its values, and the weights spread them (without it
 //    1.3e-15 to 2e-15 for noise on 32 x 48, now 6e-16 to 7e-16).
-// 1024 x 1024, q = 30: 1.27 ms without the last three, 1.30 ms with them.
+// None of the four shows in the time: 1024 x 1024, q = 30: 1.26 ms, q = 42: 4.1.
 //
 // Digits come from integers, not from double-float: FP64 input is shifted into 64-bit fixed point
 // (the curl's differences are then exact), multiplied by 63-bit constants, and a byte permutation
@@ -80,31 +81,32 @@ inline Fix make_fix(double f) {
   r.lo = (int)((s - (double)r.hi) * 2147483648.0);
   return r;
 }
-// v 2^{60 - E}, |v| < 2^{E+1}, E > kMinExp, truncated to an integer.  (Zero and subnormals, exponent
-// field 0, are shifted out whole.  Truncation pulls every value towards zero, which adds up on the
-// diagonal of a Gram: at 2^{52 - E} it was the largest error there, 1e-15 to 3e-15 for noise.)
+// v 2^{52 - E}, |v| < 2^{E+1}, E > kMinExp, rounded down to an integer (one unit off where v is zero or
+// subnormal, exponent field 0, and its sign is set).  Down, not towards zero: that pulls in every value,
+// which adds up on the diagonal of a Gram (1e-15 to 2e-15 for noise), where half a unit of all alike is
+// taken back by the constants of digits1 and digits2.
 __device__ __forceinline__ long long to_fixed(double v, int E) {
   const int hi = __double2hiint(v), sh = min(E + 1023 - ((hi >> 20) & 0x7FF), 63);  // at least 0
-  const unsigned long long m =
-      (((unsigned long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(v)) << 8 >> sh;
+  const long long m = ((long long)((hi & 0xFFFFF) | 0x100000) << 32) | (unsigned)__double2loint(v);
   const long long s = (long long)(hi >> 31);
-  return ((long long)m ^ s) - s;
+  return ((m ^ s) - s) >> sh;
 }
 // Operand digits of z rounded to the nearest integer: six bytes that carry 0x80 too much each, and in
-// digits1 a ninth bit of the first digit, which carries 0x100 too much.  digits1: z = X f / 16 (X a curl
-// in units of 2^{Ez - 52}), |z| < 0.99 2^48, the products exact to a few units of 2^-3; digits2:
-// z = (X f + Y g) / 2^13, |z| < 0.99 2^47, to a few units of 2^-12.
-constexpr long long kDigitBias = 0x808080808080ll, kDigitBias9 = 0x1008080808080ll;
+// digits1 a ninth bit of the first digit, which carries 0x100 too much.  digits1: z = X f / 16,
+// |z| < 0.99 2^48; digits2: z = (X f + Y g) / 32, |z| < 0.99 2^47.  h f.hi is exact; the high products
+// (and X, Y) are rounded down, by 1.7 units of 2^-3 on average in digits1 and 3.2 of 2^-4 in digits2, which
+// comes on top of the half that rounds to nearest (4 + 2, 8 + 3).
+constexpr long long kDigitBias = 0x808080808080ll * 16 + 8 + 3, kDigitBias9 = 0x1008080808080ll * 8 + 4 + 2;
 __device__ __forceinline__ unsigned long long digits1(long long X, Fix f) {
   const int h = (int)(X >> 32);
-  const long long t = (long long)h * f.hi + (kDigitBias9 * 8 + 4) + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
+  const long long t = (long long)h * f.hi + kDigitBias9 + (long long)__umulhi((unsigned)X, (unsigned)f.hi);
   return (unsigned long long)(t + 2 * (long long)__mulhi(h, f.lo)) >> 3;
 }
 __device__ __forceinline__ unsigned long long digits2(long long X, Fix f, long long Y, Fix g) {
   const int h = (int)(X >> 32), k = (int)(Y >> 32);
-  const long long t = (long long)h * f.hi + ((long long)k * g.hi + (kDigitBias * 4096 + 2048));
+  const long long t = (long long)h * f.hi + ((long long)k * g.hi + kDigitBias);
   const unsigned l = __umulhi((unsigned)X, (unsigned)f.hi) + __umulhi((unsigned)Y, (unsigned)g.hi);  // below 2^32
-  return (unsigned long long)(t + (long long)l + 2 * (long long)(__mulhi(h, f.lo) + __mulhi(k, g.lo))) >> 12;
+  return (unsigned long long)(t + (long long)l + 2 * (long long)(__mulhi(h, f.lo) + __mulhi(k, g.lo))) >> 4;
 }
 
 // Operand values of two neighbouring nodes and one component (biased digits b0, b1): stores digit s
@@ -288,7 +290,7 @@ struct GramArgs {
   int n, m;
   long N;
   Fix ax, bx, ay, by;  // mass factor times 2^ox (x-edges) and 2^oy (y-edges)
-  int ox, oy;          // x 2^{60 - Em - ox} < 2^61 likewise
+  int ox, oy;          // x 2^{52 - Em - ox} < 2^53 likewise
   const uint2* sw;
   int sw_exp;
   const double* ph;
@@ -358,8 +360,7 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
         ny = load_y(Xc[0] + A.N, i, j + 1, A.n, p.al, in);
       }
       const unsigned at = dst + b * kArray;
-      const int sh = Ex[b] + A.sw_exp - Ez[b] - 8;
-      const long long half = sh >= 0 ? 0 : 1ll << (min(-sh, 62) - 1);
+      const int sh = Ex[b] + A.sw_exp - Ez[b];
 #pragma unroll
       for (int im = 0; im < 2; ++im) {
         // (a row or column outside the level leaves zeros: its loads were zero, and the last row's
@@ -374,7 +375,7 @@ __device__ __forceinline__ void produce_chunk(const GramArgs& A, const double2* 
 #pragma unroll
           for (int k = 0; k < 2; ++k) {
             const long long d = (x1[k][im] - xf[b][k][im]) - (y[k + 1][im] - y[k][im]);
-            const long long e = sh >= 0 ? (long long)((unsigned long long)d << min(sh, 62)) : (d + half) >> min(-sh, 62);
+            const long long e = sh >= 0 ? (long long)((unsigned long long)d << min(sh, 62)) : d >> min(-sh, 62);
             z[k] = digits1(e, Fix{(int)w[k].x, (int)w[k].y});
           }
           store_digits<true>(at + im * 512, z[0], z[1]);

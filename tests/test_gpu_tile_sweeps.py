@@ -6,62 +6,77 @@ index that is no candidate would be tuned instead and leave a key in the cache.
 """
 import json
 
+import numpy as np
 import pytest
 
+from oracle import fem, multigrid as mg
 from test_gpu_tuner import _child
 
 pytestmark = pytest.mark.gpu
 
 CHILD = r"""
-import json
+import json, sys
 import numpy as np, torch
 import __graft_entry__ as ge
 ge.build()
 import paper_2304_00337_gb300 as pbs
-from oracle import fem, multigrid as mg
+import test_gpu_tile_sweeps as t
+ref = np.load(%r)
 out = []
-rng = np.random.default_rng(11)
-def block(n):
-    return rng.standard_normal((2, n)) + 1j * rng.standard_normal((2, n))
-def rel(y, want):
-    return float(np.max(np.linalg.norm(y - want, axis=1) / np.linalg.norm(want, axis=1)))
 with pbs.Context(0) as ctx:
-    for a, b, n, m, k in ((1.0, 0.5, 192, 96, (0.4, -1.3)), (1.0, 1.0, 128, 128, (0.0, 0.0))):
-        eps = rng.uniform(1.0, 9.0, (m, n))
-        geom, mesh = pbs.Geometry(eps, a, b), fem.Mesh(a, b, n, m)
-        nlev, ops = mg.nodal_hierarchy(mesh, eps, k, 4), fem.assemble(mesh, eps, k)
-        gamma = fem.is_gamma(*fem.bloch_phases(k, a, b))
-        # at Gamma the nodal operator annihilates the constants: compared modulo them
-        mod = (lambda y: y - y.mean(axis=1, keepdims=True)) if gamma else (lambda y: y)
-        xn, xe = mod(block(mesh.N)), block(mesh.D)
+    for c, (a, b, n, m, k) in enumerate(t.MESHES):
         for nu in (2, 3):
-            wn = mod(np.stack([mg.nodal_vcycle(nlev, c, nu, nu) for c in xn]))
-            we = mg.project_approx(ops, nlev, xe.T, 2, nu, nu).T
             for prec in (pbs.PBS_FP64, pbs.PBS_MIXED):
-                for op, x, want in (("VCYCLE_NODAL", xn, wn), ("PROJECT", xe, we)):
-                    xd = torch.from_numpy(np.ascontiguousarray(x)).cuda()
+                for op in ("VCYCLE_NODAL", "PROJECT"):
+                    x, want = ref[f"{c} {op} x"], ref[f"{c} {op} {nu}"]
+                    xd = torch.from_numpy(x).cuda()
                     y = torch.zeros_like(xd)
                     o = pbs.default_opts(precision=prec, nu_pre=nu, nu_post=nu, nodal_cycles=2)
-                    ctx.apply(geom, op, xd.data_ptr(), y.data_ptr(), 2, k=k, opts=o, stream=torch.cuda.current_stream())
+                    ctx.apply(pbs.Geometry(ref[f"{c} eps"], a, b), op, xd.data_ptr(), y.data_ptr(), 2, k=k, opts=o,
+                              stream=torch.cuda.current_stream())
                     torch.cuda.synchronize()
-                    got = y.cpu().numpy()
-                    out.append([n, nu, prec, op, rel(mod(got) if op != "PROJECT" else got, want)])
+                    d = t.modulo(y.cpu().numpy(), k, op) - want
+                    out.append([n, nu, prec, op, float(np.max(np.linalg.norm(d, axis=1) / np.linalg.norm(want, axis=1)))])
 print(json.dumps(out))
 """
 
+MESHES = [(1.0, 0.5, 192, 96, (0.4, -1.3)), (1.0, 1.0, 128, 128, (0.0, 0.0))]
 
-@pytest.mark.parametrize("shape", [0, 1, 2])
-def test_two_and_three_sweeps(tmp_path, shape):
+
+def modulo(y, k, op):
+    """At Gamma the nodal operator annihilates the constants: cycles are compared modulo them."""
+    return y - y.mean(axis=1, keepdims=True) if k == (0.0, 0.0) and op == "VCYCLE_NODAL" else y
+
+
+@pytest.fixture(scope="module")
+def reference(tmp_path_factory):
     torch = pytest.importorskip("torch")
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
+    rng = np.random.default_rng(11)
+    out = {}
+    for c, (a, b, n, m, k) in enumerate(MESHES):
+        eps, mesh = rng.uniform(1.0, 9.0, (m, n)), fem.Mesh(a, b, n, m)
+        nlev, ops = mg.nodal_hierarchy(mesh, eps, k, 4), fem.assemble(mesh, eps, k)
+        xn, xe = (rng.standard_normal((2, d)) + 1j * rng.standard_normal((2, d)) for d in (mesh.N, mesh.D))
+        xn = modulo(xn, k, "VCYCLE_NODAL")
+        out.update({f"{c} eps": eps, f"{c} VCYCLE_NODAL x": xn, f"{c} PROJECT x": xe})
+        for nu in (2, 3):
+            out[f"{c} VCYCLE_NODAL {nu}"] = modulo(np.stack([mg.nodal_vcycle(nlev, v, nu, nu) for v in xn]), k, "VCYCLE_NODAL")
+            out[f"{c} PROJECT {nu}"] = np.ascontiguousarray(mg.project_approx(ops, nlev, xe.T, 2, nu, nu).T)
+    path = tmp_path_factory.mktemp("sweeps") / "reference.npz"
+    np.savez(path, **out)
+    return str(path)
+
+
+@pytest.mark.parametrize("shape", [0, 1, 2])
+def test_two_and_three_sweeps(tmp_path, reference, shape):
     cache = tmp_path / "tune.json"
     got = _child({"PBS_TUNE_CACHE": str(cache), "PBS_TUNE": "1", "PBS_TUNE_FORCE": f"node_down={shape},node_up={shape}"},
-                 CHILD)
+                 CHILD % reference)
     # the bars of the same cycles with one sweep per side: 1e-11 and 1e-12 in FP64, 1e-5 in FP32
     for n, nu, prec, op, err in got:
         assert err <= (1e-5 if prec else 1e-12 if op == "PROJECT" else 1e-11), (n, nu, prec, op, err)
     keys = [k for k in json.loads(cache.read_text()) if k.startswith("node_")] if cache.exists() else []
-    # FP64 with three sweeps has one shape on these levels and tunes nothing; smaller levels have one too.  (The 64 x
-    # 64 level below 128 x 128 is not tiled.)
+    # (where only one shape fits, FP64 with three sweeps and small levels, nothing is tuned)
     assert not keys, keys
