@@ -914,11 +914,14 @@ template <class T, int FT> void set_fine_smem() {
 // columns a strip is a chain of rows and little else, and short strips pay for their five halo rows:
 // 4 / 8 / 16 rows against the best tile, 10 columns, FP32: 72 x 72 13 / 16 / 21, 22; 128 x 128 13 / 16 /
 // 21, 22; 208 x 144 13 / 17 / 21, 25; 256 x 256 21 / 17 / 22; FP64: 72 x 72 43 / 70 / 119, 111; 128 x 128
-// 76 / 68 / 119, 197; 256 x 256 201 / 176 / 210.  The first shape fits every level this path takes.
+// 76 / 68 / 119, 197; 256 x 256 201 / 176 / 210.  The first shape fits every level this path takes and is
+// what runs without tuning: strips of 8 rows are faster than the tiles on every level and number of
+// columns (one column, FP64, a cycle's fine steps: 72 x 72 76 against 110, 208 x 144 152 against 218,
+// with 16 rows 125 and 251; 40 columns, FP32, 1024 x 1024 787 against 1875, with 16 rows 737).
 struct FineShape {
   int ft, nt;
 };
-constexpr FineShape kStripShapes[] = {{16, 0}, {32, 0}, {64, 0}, {8, 0}, {4, 0}};
+constexpr FineShape kStripShapes[] = {{8, 0}, {16, 0}, {32, 0}, {64, 0}, {4, 0}};
 constexpr FineShape kTileShapes[] = {{32, 256}, {64, 512}, {64, 256}};
 constexpr int kNumFineShapes = 5;
 template <class T>
@@ -1103,18 +1106,23 @@ void node_cycle(const Hierarchy& H, const KData& K, MgWork<T>& w, int l, const c
     const int nd = fine_shapes<T>(L, nu_pre, true, fd), nup = fine_shapes<T>(L, nu_post, false, fu);
     // both steps are idempotent (the down step reads b, the up step b, its saved
     // pre-smoothed x and the coarse correction, and neither writes what it reads)
-    // (strips have their number of candidates in the key: plain keys with one sweep per side hold an
-    // earlier build's choices among tiles, other shapes under the same index)
-    const auto key = [&](const char* step, int nu, int count) {
-      return std::string(step) + (nu == 1 ? "strips" + std::to_string(count) + "|" : "") + fine_key<T>(L, ncols, cpg) + "|nu" +
-             std::to_string(nu);
+    // (strips name their candidates in the key: plain keys with one sweep per side hold an earlier
+    // build's choices among tiles, other shapes under the same index)
+    const auto key = [&](const char* step, int nu, const FineShape* f, int count) {
+      std::string k = step;
+      if (nu == 1) {
+        k += "strips";
+        for (int c = 0; c < count; ++c) k += (c ? "." : "") + std::to_string(f[c].ft);
+        k += "|";
+      }
+      return k + fine_key<T>(L, ncols, cpg) + "|nu" + std::to_string(nu);
     };
-    const int pd = tune_pick(key("node_down|", nu_pre, nd), nd, [&](int c) { down(fd[c]); }, s);
+    const int pd = tune_pick(key("node_down|", nu_pre, fd, nd), nd, [&](int c) { down(fd[c]); }, s);
     timer_begin(KC_NODE_SMOOTH, s, fine_bytes<T>(L, ncols, nu_pre, true));
     down(fd[pd]);
     timer_end(KC_NODE_SMOOTH, s);
     node_cycle<T>(H, K, w, l + 1, w.b[l + 1], w.x[l + 1], C.N(), ncols, cpg, nu_pre, nu_post, s);
-    const int pu = tune_pick(key("node_up|", nu_post, nup), nup, [&](int c) { up(fu[c]); }, s);
+    const int pu = tune_pick(key("node_up|", nu_post, fu, nup), nup, [&](int c) { up(fu[c]); }, s);
     timer_begin(KC_NODE_SMOOTH, s, fine_bytes<T>(L, ncols, nu_post, false));
     up(fu[pu]);
     timer_end(KC_NODE_SMOOTH, s);
